@@ -11,11 +11,20 @@
 // parameters, counter (j, i / 4, 1, 0) the four normals of samples 4(i/4) .. 4(i/4)+3
 // (Box-Muller on uniforms u = (x >> 8) 2^-24).
 //
-// Fold: one block per light curve. Each warp owns a private copy of the bins in shared
-// memory. Lanes take four consecutive samples each; samples that land in the same bin in
-// one step are merged with __match_any_sync and their sum is added, in lane order, by the
-// group's lowest lane, so no two threads update a bin at once. The per-warp bins are added
-// in warp order at the end (deterministic). Phases are the 64-bit fixed point of the fold.
+// Fold: one block per light curve, lanes taking four consecutive samples each (the four
+// normals of one Philox call). What bounds it is instruction issue: the device's FP64 rate is
+// one warp instruction per 64 cycles and scheduler, so a sample does no FP64 at all.
+//  * tau_i = rint(fl(i cadence) 2^24) comes from a 64-bit fixed-point product i * cadence
+//    2^(24+40), and the box membership from the fixed-point phase of the light curve's own
+//    period; both know how far they can be off, and a sample that close to a rounding or box
+//    edge (one in some 10^5) is decided by the FP64 formula itself, so every bin, count and
+//    membership is that of the formula.
+//  * flux: x is summed as integers, rint(x 2^e) with |x| 2^e <= 2^22 (an FP32 add with a large
+//    constant rounds it), by shared-memory reductions: the low 11 bits, the rest and the count
+//    each have a word per bin. Integer sums are exact and independent of their order; sum and
+//    sum of squares (a 64-bit integer per lane) also give the flux standard deviation.
+// 4,096 curves of 65,536 samples: 12.5 ms with FP64 phases, fmod, moments and a 32-shuffle
+// merge of equal bins per sample; see kSynthThreads for the time now.
 #include <cmath>
 #include <cstdint>
 
@@ -52,37 +61,88 @@ __host__ __device__ __forceinline__ Philox4 philox4x32_10(uint32_t c0, uint32_t 
 __device__ __forceinline__ double unif64(uint32_t x) { return (double)(x >> 8) * (1.0 / 16777216.0); }
 __device__ __forceinline__ float unif32(uint32_t x) { return (float)(x >> 8) * (1.0f / 16777216.0f); }
 
-// parameters of light curve j
+// Parameters of a light curve, derived by one warp and shared by its block.
 struct LcParams {
     int kind;        // 0 transit, 1 noise, 2 sinusoid, 3 eclipsing binary
-    double sigma, period, epoch, duration, depth, depth2, amp, fold_period;
+    int fixed;       // the fixed-point phases below hold for every sample
+    double period, epoch, duration, fold_period;
+    float sigma, depth, depth2, amp;
+    uint32_t Fl, Fh;  // fold frequency, rint(2^40 / fold_period)
+    uint32_t Gl, Gh;  // light curve's own frequency, rint(2^40 / period)
+    uint32_t off;     // epoch / period in 2^-32 cycles
+    uint32_t half;    // half the duration in 2^-32 cycles
+    uint32_t guard;   // bound of the phase's error in 2^-32 cycles
+    float cyc;        // 2^-24 / period: cycles per unit of tau
+    float scale;      // 2^e
+    int e;
+    // the cadence in units of tau: integer part, fraction in 2^-64; and in 2^-20 (64-bit)
+    uint32_t step_i;
+    uint64_t step_f, step20;
+    uint32_t tguard;  // bound of the fixed-point time's error in 2^-20 units of tau
 };
 
-__device__ LcParams lc_params(uint64_t seed, int64_t j, const gpfc_synth_params &sp)
+// Called by one whole warp; lane 0's values are the light curve's.
+__device__ LcParams lc_params(uint64_t seed, int64_t j, const gpfc_synth_params &sp, int lane)
 {
     const uint32_t k0 = (uint32_t)seed, k1 = (uint32_t)(seed >> 32);
     const Philox4 a = philox4x32_10((uint32_t)j, 0u, 0u, 0xFFFFFFFFu, k0, k1);
     const Philox4 b = philox4x32_10((uint32_t)j, 1u, 0u, 0xFFFFFFFFu, k0, k1);
     LcParams p{};
     p.kind = (j & 1) ? 1 + (int)((j >> 1) % 3) : 0;
-    p.sigma = exp(log(sp.sigma_min) + unif64(a.v[0]) * log(sp.sigma_max / sp.sigma_min));
+    // the three log-uniform draws (sigma, depth, amplitude) on three lanes at once
+    const double lo = lane == 0 ? sp.sigma_min : sp.depth_min, hi = lane == 0 ? sp.sigma_max : sp.depth_max;
+    const double lu = exp(log(lo) + unif64(lane == 0 ? a.v[0] : (lane == 1 ? b.v[0] : b.v[2])) * log(hi / lo));
+    const double sigma = __shfl_sync(0xffffffffu, lu, 0), depth = __shfl_sync(0xffffffffu, lu, 1);
+    const double amp = __shfl_sync(0xffffffffu, lu, 2);
     // explicit round-to-nearest operations (no fused multiply-add), so that these values
     // are bit-identical to any IEEE-754 evaluation of the same formulas
     p.period = __dadd_rn(sp.p_min, __dmul_rn(unif64(a.v[1]), __dsub_rn(sp.p_max, sp.p_min)));
     p.epoch = __dmul_rn(unif64(a.v[2]), p.period);
     p.duration = __ddiv_rn(__dadd_rn(sp.dur_min_h, __dmul_rn(unif64(a.v[3]), __dsub_rn(sp.dur_max_h, sp.dur_min_h))),
                            24.0);
-    p.depth = exp(log(sp.depth_min) + unif64(b.v[0]) * log(sp.depth_max / sp.depth_min));
-    p.depth2 = __dmul_rn(p.depth, __dadd_rn(0.2, __dmul_rn(0.8, unif64(b.v[1]))));
-    p.amp = exp(log(sp.depth_min) + unif64(b.v[2]) * log(sp.depth_max / sp.depth_min));
+    const double depth2 = __dmul_rn(depth, __dadd_rn(0.2, __dmul_rn(0.8, unif64(b.v[1]))));
     const double T = __dmul_rn((double)sp.n_cadences, sp.cadence);
     const double df = __ddiv_rn(__dmul_rn(__dsub_rn(__dmul_rn(2.0, unif64(b.v[3])), 1.0), sp.drift_bins),
                                 __dmul_rn(256.0, T));
     p.fold_period = __ddiv_rn(1.0, __dadd_rn(__ddiv_rn(1.0, p.period), df));
+    p.sigma = (float)sigma;
+    p.depth = (float)depth;
+    p.depth2 = (float)depth2;
+    p.amp = (float)amp;
+    const unsigned long long F = (unsigned long long)__double2ll_rn(__ddiv_rn(1099511627776.0, p.fold_period));
+    p.Fl = (uint32_t)F;
+    p.Fh = (uint32_t)(F >> 32);
+    // |x| < 5.78 sigma (the largest Box-Muller radius for u >= 2^-24) plus the signal
+    const double xmax = 5.78 * sigma + (p.kind == 2 ? amp : (p.kind == 0 ? depth : (p.kind == 3 ? depth + depth2 : 0.0)));
+    p.e = max(-100, min(100, 21 - ilogb(xmax)));
+    p.scale = (float)ldexp(1.0, p.e);
+    // fixed-point phase of the light curve's own period: off by at most 2^-25 d of tau, half a
+    // unit of 2^-40 c/d over T, and a few units of 2^-32 cycles
+    const double freq = 1.0 / p.period;
+    const unsigned long long G = (unsigned long long)__double2ll_rn(1099511627776.0 * freq);
+    p.Gl = (uint32_t)G;
+    p.Gh = (uint32_t)(G >> 32);
+    p.off = (uint32_t)__double2ll_rn(p.epoch * freq * 4294967296.0);
+    const double half = 0.5 * p.duration * freq;
+    p.half = (uint32_t)__double2ll_rn(fmin(half, 0.5) * 4294967296.0);
+    const double guard = 4294967296.0 * (freq * 5.9604644775390625e-08 + T * 9.094947017729282e-13) + 16.0;
+    p.guard = (uint32_t)fmin(guard, 1e9);
+    p.cyc = (float)(freq * 5.9604644775390625e-08);
+    // fixed-point time of four consecutive samples: the first exact to 2^-32 and cut to 2^-20
+    // units of tau, three additions of a step cut to 2^-20; and the rounding of i * cadence in FP64
+    const double c24 = sp.cadence * 16777216.0;
+    const double tguard = 6.0 + 1048576.0 * (T * 16777216.0) * 2.220446049250313e-16;
+    p.fixed = c24 < 8388608.0 && T * 16777216.0 < 4398046511104.0 && tguard < 65536.0 && freq < 1e6 && freq > 1e-6 &&
+              guard < 1e6 && half < 0.49;
+    p.tguard = p.fixed ? (uint32_t)tguard : 0u;
+    p.step_i = p.fixed ? (uint32_t)c24 : 0u;
+    p.step_f = p.fixed ? (uint64_t)((c24 - floor(c24)) * 18446744073709551616.0) : 0ull;
+    p.step20 = p.fixed ? (uint64_t)(c24 * 1048576.0) : 0ull;
     return p;
 }
 
-__device__ __forceinline__ bool in_box(double t, double period, double centre, double dur)
+// The box membership in FP64: |t - nearest mid-transit| < dur / 2.
+__device__ __noinline__ bool in_box(double t, double period, double centre, double dur)
 {
     const double half = __dmul_rn(0.5, period);
     const double d = fmod(__dadd_rn(__dsub_rn(t, centre), half), period);
@@ -90,110 +150,154 @@ __device__ __forceinline__ bool in_box(double t, double period, double centre, d
     return fabs(dd) < __dmul_rn(0.5, dur);
 }
 
-constexpr int kSynthWarps = 8;
-
-__global__ void __launch_bounds__(kSynthWarps * 32) synth_fold_kernel(SynthParams P)
+// The membership from the signed fixed-point phase about the mid-transit; 0 or 1, or 2 within
+// the guard of an edge.
+__device__ __forceinline__ int in_box_fixed(int32_t su, uint32_t half, uint32_t guard)
 {
-    __shared__ float s_sum[kSynthWarps][256];
-    __shared__ uint32_t s_cnt[kSynthWarps][256];
-    __shared__ double s_mom[kSynthWarps][2];
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int nb = P.nbins;
+    const uint32_t a = su < 0 ? 0u - (uint32_t)su : (uint32_t)su;
+    return a - half + guard <= 2u * guard ? 2 : (a < half ? 1 : 0);
+}
+
+__device__ __noinline__ long long tau_fp64(int i, double cadence)
+{
+    return __double2ll_rn(__dmul_rn(__dmul_rn((double)i, cadence), 16777216.0));
+}
+
+// Threads per light curve: 256, so that several blocks share an SM and one's set-up overlaps
+// the others' samples; 1,024 where there are too few light curves to fill the SMs that way.
+constexpr int kSynthThreads = 256, kSynthWide = 1024;
+
+constexpr int kSynthSpan = 1 << 19;  // samples between emptyings of the 32-bit bin words
+
+template <bool POW2, int THREADS>
+__global__ void __launch_bounds__(THREADS) synth_fold_kernel(SynthParams P, int shift)
+{
+    __shared__ uint32_t s_lo[256], s_hi[256], s_cnt[256];  // sum = hi 2^11 + lo, hi signed
+    __shared__ LcParams s_lp;
+    __shared__ long long s_m1[8];
+    __shared__ double s_m2[32];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int nb = P.nbins, n = P.sp.n_cadences, tid = threadIdx.x;
     const uint32_t k0 = (uint32_t)P.seed, k1 = (uint32_t)(P.seed >> 32);
     for (int64_t q = blockIdx.x; q < P.n; q += gridDim.x) {
         const int64_t j = P.first + q;
-        const LcParams lp = lc_params(P.seed, j, P.sp);
-        const double Fd = __ddiv_rn(1099511627776.0, lp.fold_period);
-        const unsigned long long F = (unsigned long long)__double2ll_rn(Fd);
-        for (int b = lane; b < nb; b += 32) {
-            s_sum[warp][b] = 0.f;
-            s_cnt[warp][b] = 0u;
+        if (warp == 0) {
+            const LcParams l = lc_params(P.seed, j, P.sp, lane);
+            if (lane == 0) s_lp = l;
         }
-        __syncwarp();
-        // a multiple of 128 samples per warp keeps every lane's first sample at i % 4 == 0
-        const int per_warp = ((P.sp.n_cadences + kSynthWarps - 1) / kSynthWarps + 127) & ~127;
-        const int i_begin = warp * per_warp;
-        const int i_end = min(P.sp.n_cadences, i_begin + per_warp);
-        double m1 = 0.0, m2 = 0.0;  // sum of x and x^2 over this lane's samples
-        for (int base = i_begin; base < i_end; base += 128) {
-            const int i0 = base + 4 * lane;  // this lane's 4 samples (i0 % 4 == 0 when base is)
-            const Philox4 r = philox4x32_10((uint32_t)j, (uint32_t)(i0 >> 2), 1u, 0u, k0, k1);
-            float z[4];
-#pragma unroll
-            for (int h = 0; h < 2; ++h) {
-                const float u1 = 1.0f - unif32(r.v[2 * h]);  // (0, 1]
-                const float u2 = unif32(r.v[2 * h + 1]);
-                const float rad = sqrtf(-2.0f * logf(u1));
-                float s, c;
-                sincospif(2.0f * u2, &s, &c);
-                z[2 * h] = rad * c;
-                z[2 * h + 1] = rad * s;
-            }
-#pragma unroll
-            for (int qq = 0; qq < 4; ++qq) {
-                const int i = i0 + qq;
-                const bool valid = i < i_end;
-                const double t = __dmul_rn((double)i, P.sp.cadence);
-                float x = (float)lp.sigma * z[qq];
-                if (lp.kind == 0) {
-                    if (in_box(t, lp.period, lp.epoch, lp.duration)) x -= (float)lp.depth;
-                } else if (lp.kind == 2) {
-                    x += (float)(lp.amp * sinpi(2.0 * (t - lp.epoch) / lp.period));
-                } else if (lp.kind == 3) {
-                    if (in_box(t, lp.period, lp.epoch, lp.duration)) x -= (float)lp.depth;
-                    if (in_box(t, lp.period, __dadd_rn(lp.epoch, __dmul_rn(0.5, lp.period)), lp.duration))
-                        x -= (float)lp.depth2;
-                }
-                if (valid) {
-                    m1 += (double)x;
-                    m2 += (double)x * (double)x;
-                }
-                const long long tau = __double2ll_rn(__dmul_rn(t, 16777216.0));
-                const unsigned long long phi = (unsigned long long)tau * F;
-                const int bin = valid ? (int)__umul64hi(phi, (unsigned long long)nb) : -1;
-                const unsigned m = __match_any_sync(0xffffffffu, bin);
-                float gs = 0.f;
-                for (int src = 0; src < 32; ++src) {
-                    const float xs = __shfl_sync(0xffffffffu, x, src);
-                    if ((m >> src) & 1u) gs += xs;
-                }
-                if (valid && (__ffs(m) - 1) == lane) {
-                    s_sum[warp][bin] += gs;
-                    s_cnt[warp][bin] += (uint32_t)__popc(m);
-                }
-                __syncwarp();
-            }
-        }
-        for (int o = 16; o > 0; o >>= 1) {
-            m1 += __shfl_xor_sync(0xffffffffu, m1, o);
-            m2 += __shfl_xor_sync(0xffffffffu, m2, o);
-        }
-        if (lane == 0) {
-            s_mom[warp][0] = m1;
-            s_mom[warp][1] = m2;
-        }
+        if (tid < 256) s_lo[tid] = s_hi[tid] = s_cnt[tid] = 0u;
         __syncthreads();
-        if (threadIdx.x == 0 && P.sigma_out) {
-            double a = 0.0, b2 = 0.0;
-            for (int w = 0; w < kSynthWarps; ++w) {
-                a += s_mom[w][0];
-                b2 += s_mom[w][1];
+        const LcParams &lp = s_lp;
+        const int kind = lp.kind;
+        const bool fixed = lp.fixed != 0, boxes = kind == 0 || kind == 3;
+        const uint32_t Fl = lp.Fl, Fh = lp.Fh, Gl = lp.Gl, Gh = lp.Gh, half = lp.half, guard = lp.guard;
+        const uint32_t step_i = lp.step_i, sfl = (uint32_t)lp.step_f, sfh = (uint32_t)(lp.step_f >> 32), tguard = lp.tguard;
+        const uint64_t step20 = lp.step20;
+        const float sigma = lp.sigma, scale = lp.scale;
+        unsigned long long m2 = 0ull;          // sum of squares of this lane's integers
+        long long tot = 0;                     // bin tid: sum and count
+        uint32_t cnt = 0u;
+        for (int64_t span = 0; span < n; span += kSynthSpan) {
+            const int i_end = (int)min((int64_t)n, span + kSynthSpan);
+            for (int64_t base = span + 128 * warp; base < i_end; base += 128 * nw) {
+                const int i0 = (int)base + 4 * lane;  // this lane's four samples
+                if (i0 >= i_end) break;               // (no warp-wide operation below)
+                const Philox4 r = philox4x32_10((uint32_t)j, (uint32_t)(i0 >> 2), 1u, 0u, k0, k1);
+                // time of sample i0 in 2^-20 units of tau
+                const uint64_t p0 = (uint64_t)(uint32_t)i0 * sfl, p1 = (uint64_t)(uint32_t)i0 * sfh + (p0 >> 32);
+                uint64_t tf = (((uint64_t)(uint32_t)i0 * step_i + (p1 >> 32)) << 20) | ((uint32_t)p1 >> 12);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const float u1 = 1.0f - unif32(r.v[2 * h]);  // (0, 1]
+                    const float u2 = unif32(r.v[2 * h + 1]);
+                    const float rad = sqrtf(-2.0f * logf(u1));
+                    float sn, cs;
+                    sincospif(2.0f * u2, &sn, &cs);
+#pragma unroll
+                    for (int m = 0; m < 2; ++m, tf += step20) {
+                        const int i = i0 + 2 * h + m;
+                        if (i >= i_end) break;
+                        // tau: the rounded fixed-point time, or FP64 near a half
+                        const uint64_t tr = tf + (1ull << 19);
+                        long long tau = (long long)(tr >> 20);
+                        const uint32_t fr = (uint32_t)tr & 0xFFFFFu;
+                        if (!fixed || fr - tguard > 0xFFFFFu - 2u * tguard) tau = tau_fp64(i, P.sp.cadence);
+                        const uint32_t tl = (uint32_t)(unsigned long long)tau, th = (uint32_t)((unsigned long long)tau >> 32);
+                        float x = sigma * (m ? rad * sn : rad * cs);
+                        if (kind != 1) {
+                            const uint32_t ph = (uint32_t)(((unsigned long long)tl * Gl +
+                                                            ((unsigned long long)(th * Gl + tl * Gh) << 32)) >> 32);
+                            const int32_t su = (int32_t)(ph - lp.off);
+                            if (boxes) {
+                                int in = fixed ? in_box_fixed(su, half, guard) : 2;
+                                if (in == 2)
+                                    in = in_box(__dmul_rn((double)i, P.sp.cadence), lp.period, lp.epoch, lp.duration);
+                                if (in) x -= lp.depth;
+                                if (kind == 3) {
+                                    in = fixed ? in_box_fixed((int32_t)((uint32_t)su ^ 0x80000000u), half, guard) : 2;
+                                    if (in == 2)
+                                        in = in_box(__dmul_rn((double)i, P.sp.cadence), lp.period,
+                                                    __dadd_rn(lp.epoch, __dmul_rn(0.5, lp.period)), lp.duration);
+                                    if (in) x -= lp.depth2;
+                                }
+                            } else if (fixed) {
+                                // phase in cycles, with the part of the time below the unit of tau
+                                const float dt = (float)((int32_t)fr - (1 << 19)) * 9.5367431640625e-07f;
+                                x += lp.amp * sinpif(2.0f * fmaf(dt, lp.cyc, (float)su * 2.3283064365386963e-10f));
+                            } else {
+                                const double t = __dmul_rn((double)i, P.sp.cadence);
+                                x += (float)((double)lp.amp * sinpi(2.0 * (t - lp.epoch) / lp.period));
+                            }
+                        }
+                        // rint(x 2^e): the sum with 3 2^22 has a unit in its last place of 1
+                        const int xq = __float_as_int(fmaf(x, scale, 12582912.0f)) - 0x4B400000;
+                        m2 += (unsigned long long)((long long)xq * (long long)xq);
+                        const unsigned long long phi = (unsigned long long)tl * Fl +
+                                                       ((unsigned long long)(th * Fl + tl * Fh) << 32);
+                        const uint32_t bin = POW2 ? (uint32_t)(phi >> 32) >> shift
+                                                  : (uint32_t)__umul64hi(phi, (unsigned long long)nb);
+                        atomicAdd(&s_lo[bin], (uint32_t)xq & 2047u);
+                        atomicAdd(&s_hi[bin], (uint32_t)(xq >> 11));
+                        atomicAdd(&s_cnt[bin], 1u);
+                    }
+                }
             }
-            const double nn = (double)P.sp.n_cadences, mu = a / nn;
-            P.sigma_out[q] = (float)sqrt(fmax(b2 / nn - mu * mu, 0.0));
-        }
-        for (int b = threadIdx.x; b < nb; b += blockDim.x) {
-            float s = 0.f;
-            uint32_t c = 0u;
-            for (int w = 0; w < kSynthWarps; ++w) {
-                s += s_sum[w][b];
-                c += s_cnt[w][b];
+            __syncthreads();
+            if (tid < nb) {
+                tot += ((long long)(int32_t)s_hi[tid] << 11) + (long long)s_lo[tid];
+                cnt += s_cnt[tid];
+                s_lo[tid] = s_hi[tid] = s_cnt[tid] = 0u;
             }
-            if (P.folded) P.folded[q * nb + b] = c ? 1.0f + s / (float)c : __int_as_float(0x7fc00000);
-            if (P.counts) P.counts[q * nb + b] = (int32_t)c;
+            __syncthreads();
         }
-        if (threadIdx.x == 0 && P.label) P.label[q] = lp.kind == 0 ? 1.f : 0.f;
-        if (threadIdx.x == 0 && P.period_out) P.period_out[q] = lp.fold_period;
+        const double unit = ldexp(1.0, -lp.e);
+        if (tid < nb) {
+            const size_t o = (size_t)q * nb + tid;
+            if (P.folded)
+                P.folded[o] = cnt ? (float)(1.0 + (double)tot * unit / (double)cnt) : __int_as_float(0x7fc00000);
+            if (P.counts) P.counts[o] = (int32_t)cnt;
+        }
+        if (P.sigma_out) {
+            for (int o = 16; o > 0; o >>= 1) {
+                tot += __shfl_xor_sync(0xffffffffu, tot, o);
+                m2 += __shfl_xor_sync(0xffffffffu, m2, o);
+            }
+            if (lane == 0) {
+                if (warp < 8) s_m1[warp] = tot;  // (256 bins: the first eight warps)
+                s_m2[warp] = (double)m2;
+            }
+            __syncthreads();
+            if (tid == 0) {
+                long long a = 0;
+                double b2 = 0.0;
+                for (int w = 0; w < min(nw, 8); ++w) a += s_m1[w];
+                for (int w = 0; w < nw; ++w) b2 += s_m2[w];
+                const double nn = (double)n, mu = (double)a / nn;
+                P.sigma_out[q] = (float)(sqrt(fmax(b2 / nn - mu * mu, 0.0)) * unit);
+            }
+        }
+        if (tid == 0 && P.label) P.label[q] = kind == 0 ? 1.f : 0.f;
+        if (tid == 0 && P.period_out) P.period_out[q] = lp.fold_period;
         __syncthreads();
     }
 }
@@ -267,9 +371,18 @@ cudaError_t launch_paper_vectors(const VectorParams &p, int num_sms, cudaStream_
 
 cudaError_t launch_synth(const SynthParams &p, int num_sms, cudaStream_t st)
 {
-    const int64_t want = p.n;
-    const int grid = (int)(want < (int64_t)num_sms * 8 ? want : (int64_t)num_sms * 8);
-    synth_fold_kernel<<<grid, kSynthWarps * 32, 0, st>>>(p);
+    const int threads = p.n < (int64_t)num_sms * 2 ? kSynthWide : kSynthThreads;
+    const int grid = (int)(p.n < (int64_t)num_sms * 8 ? p.n : (int64_t)num_sms * 8);
+    int shift = 32;
+    while (shift > 0 && (1 << (32 - shift)) < p.nbins) --shift;
+    const bool pow2 = (p.nbins & (p.nbins - 1)) == 0;
+    if (threads == kSynthThreads) {
+        if (pow2) synth_fold_kernel<true, kSynthThreads><<<grid, threads, 0, st>>>(p, shift);
+        else synth_fold_kernel<false, kSynthThreads><<<grid, threads, 0, st>>>(p, 0);
+    } else {
+        if (pow2) synth_fold_kernel<true, kSynthWide><<<grid, threads, 0, st>>>(p, shift);
+        else synth_fold_kernel<false, kSynthWide><<<grid, threads, 0, st>>>(p, 0);
+    }
     return cudaGetLastError();
 }
 
