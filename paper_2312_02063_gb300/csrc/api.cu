@@ -1956,14 +1956,20 @@ int gpfc_detrend(gpfc_ctx *ctx, const double *times, const float *flux, const ui
         p.seg_start = c.take<int64_t>(n + 1);
         p.seg_keep = c.take<int64_t>(n);
         p.seg_off = c.take<int64_t>(n);
-        p.G4 = c.take<double>(4 * n);
-        p.LB = c.take<double>(4 * n);
-        p.rhs = c.take<double>(n);
-        p.coef = c.take<double>(n);
-        p.trend = c.take<double>(n);
-        p.best = c.take<double>(n);
-        p.used = c.take<uint8_t>(n);
-        p.used2 = c.take<uint8_t>(n);
+        const size_t k = (size_t)p.n_sp * n;
+        p.basis = c.take<double4>(k);
+        p.interval = c.take<int32_t>(k);
+        p.first = c.take<int32_t>(k + p.n_sp + 1);
+        p.inv6 = c.take<double>(6 * k);
+        p.part14 = c.take<double>(14 * k);
+        p.G4 = c.take<double>(4 * k);
+        p.LB = c.take<double>(4 * k);
+        p.rhs = c.take<double>(k);
+        p.coef = c.take<double>(k);
+        p.trend = c.take<double>(k);
+        p.used = c.take<uint8_t>(k);
+        p.used2 = c.take<uint8_t>(k);
+        p.bic = c.take<double>(k);
         p.det = c.take<float>(n);
         return c.off + 256;
     };

@@ -26,9 +26,15 @@ struct DetrendParams {
     int64_t *seg_start;     // [n + 1]
     int64_t *seg_keep;      // [n]
     int64_t *seg_off;       // [n]
-    double *G4, *LB;        // [n][4] banded normal matrix rows and Cholesky factor
-    double *rhs, *coef, *trend, *best;  // [n]
-    uint8_t *used, *used2;  // [n]
+    // one copy per candidate spacing, [n_sp][n]: a point's four B-splines and its knot interval,
+    // the first point of each interval [n + 1], and per interval or coefficient (at its segment's
+    // points) the reciprocal knot differences [6], the 14 sums of the normal equations, the banded
+    // matrix [4], its factor [4], right side and solution
+    double4 *basis;
+    int32_t *interval, *first;
+    double *inv6, *part14, *G4, *LB, *rhs, *coef, *trend;
+    uint8_t *used, *used2;
+    double *bic;            // [n_sp][n]: by segment (infinite: the candidate was skipped)
     float *det;             // [n]
     // outputs (caller-owned, device)
     double *t_out;
