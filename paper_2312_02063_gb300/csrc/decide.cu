@@ -8,11 +8,16 @@
 // each flagged against the best peak's period for harmonics (Fig. 14 notes them): 1 for
 // the best, +m if P = m Pb, -m if P = Pb / m (m = 2..4), else 0.
 //
-// One block of kPkThreads threads per star. Statistics are FP64 block reductions. For the
-// runs, thread t owns the runs that start in its contiguous chunk of periods and follows
-// a run past the chunk's end until it closes; qualifying runs go to a shared candidate
-// list (the first kPkCap of them; the best peak and the count are exact in any case).
+// A star is taken by one block of kPkThreads threads, or by a cluster of them that split its
+// periods and meet through distributed shared memory. Statistics are FP64 sums in a fixed
+// order. For the runs, thread t owns the runs that start in its contiguous chunk of periods and
+// follows a run past the chunk's end until it closes; qualifying runs go to the candidate
+// list of the cluster's first block (the first kPkCap of them; the best peak and the count are
+// exact in any case). What bounds it: FP64 instructions (one per warp and scheduler every 64
+// cycles), five a period; one block takes 0.60 ms for 250,000 periods, see kPkCluster for a
+// cluster of sixteen.
 #include <cmath>
+#include <cooperative_groups.h>
 #include <cstdint>
 
 #include "gpfc_common.cuh"
@@ -23,32 +28,32 @@ namespace gpfc {
 constexpr int kPkThreads = 1024;
 constexpr int kPkCap = 2048;
 
+// Block reductions through one warp (every warp adding all partials would cost 32 FP64
+// instructions a warp); the value is returned to all threads.
+template <class T, class Op>
+__device__ __forceinline__ T pk_block_reduce(T v, T *red, T zero, Op op)
+{
+    for (int o = 16; o > 0; o >>= 1) v = op(v, __shfl_xor_sync(0xffffffffu, v, o));
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    __syncthreads();
+    if (lane == 0) red[warp] = v;
+    __syncthreads();
+    if (warp == 0) {
+        v = lane < kPkThreads / 32 ? red[lane] : zero;
+        for (int o = 16; o > 0; o >>= 1) v = op(v, __shfl_xor_sync(0xffffffffu, v, o));
+        if (lane == 0) red[0] = v;
+    }
+    __syncthreads();
+    return red[0];
+}
 template <class T>
 __device__ __forceinline__ T pk_block_sum(T v, T *red)
 {
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    __syncthreads();
-    if (lane == 0) red[warp] = v;
-    __syncthreads();
-    T t = 0;
-    for (int w = 0; w < kPkThreads / 32; ++w) t += red[w];
-    return t;
+    return pk_block_reduce(v, red, (T)0, [](T a, T b) { return a + b; });
 }
-
 __device__ __forceinline__ unsigned long long pk_block_max(unsigned long long v, unsigned long long *red)
 {
-    for (int o = 16; o > 0; o >>= 1) {
-        const unsigned long long u = __shfl_xor_sync(0xffffffffu, v, o);
-        v = u > v ? u : v;
-    }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    __syncthreads();
-    if (lane == 0) red[warp] = v;
-    __syncthreads();
-    unsigned long long t = 0ull;
-    for (int w = 0; w < kPkThreads / 32; ++w) t = red[w] > t ? red[w] : t;
-    return t;
+    return pk_block_reduce(v, red, 0ull, [](unsigned long long a, unsigned long long b) { return a > b ? a : b; });
 }
 
 __device__ __forceinline__ float key_value(unsigned long long key)
@@ -62,8 +67,11 @@ __device__ __forceinline__ int64_t key_index(unsigned long long key)
     return (int64_t)(0xFFFFFFFFu - (uint32_t)(key & 0xFFFFFFFFull));
 }
 
-__global__ void __launch_bounds__(kPkThreads) peaks_kernel(const PeakParams p)
+// C blocks (a cluster, or one block) per star at a time.
+template <int C>
+__global__ void __launch_bounds__(kPkThreads, 1) peaks_kernel(const PeakParams p)
 {
+    namespace cg = cooperative_groups;
     __shared__ double red_d[kPkThreads / 32];
     __shared__ float red_f[kPkThreads / 32];
     __shared__ int red_i[kPkThreads / 32];
@@ -71,45 +79,84 @@ __global__ void __launch_bounds__(kPkThreads) peaks_kernel(const PeakParams p)
     __shared__ float c_h[kPkCap];
     __shared__ int c_i[kPkCap];
     __shared__ int c_w[kPkCap];
-    __shared__ int c_n;
-    for (int s = blockIdx.x; s < p.nstars; s += gridDim.x) {
+    __shared__ int c_n, c_peaks[C];  // candidates; qualifying runs and best key of each block
+    __shared__ unsigned long long c_best[C];
+    __shared__ double part_sum, part_ss;  // this block's partial sums, read by the cluster
+    __shared__ int part_cnt;
+    __shared__ float part_mx;
+    const cg::cluster_group cluster = cg::this_cluster();
+    const int rank = C > 1 ? (int)cluster.block_rank() : 0;
+    auto meet = [&]() {
+        if (C > 1) cluster.sync();
+        else __syncthreads();
+    };
+    auto of = [&](auto *ptr, int r) { return C > 1 ? cluster.map_shared_rank(ptr, r) : ptr; };
+    for (int s = blockIdx.x / C; s < p.nstars; s += gridDim.x / C) {
         const int64_t gb = p.grid_off ? p.grid_off[s] : 0, ge = p.grid_off ? p.grid_off[s + 1] : p.np;
         const float *sc = p.score + gb;
         const int64_t len = ge - gb;
+        const int64_t lo = len * rank / C, hi = len * (rank + 1) / C;  // this block's periods
         if (threadIdx.x == 0) c_n = 0;
         // statistics of the finite scores
         double sum = 0.0;
         int cnt = 0;
-        for (int64_t k = threadIdx.x; k < len; k += kPkThreads)
-            if (isfinite(sc[k])) {
-                sum += (double)sc[k];
+        for (int64_t k = lo + threadIdx.x; k < hi; k += kPkThreads) {
+            const float v = sc[k];
+            if (isfinite(v)) {
+                sum += (double)v;
                 ++cnt;
             }
+        }
         sum = pk_block_sum(sum, red_d);
-        const int ntot = pk_block_sum(cnt, red_i);
-        const double mean = ntot > 0 ? sum / (double)ntot : NAN;
+        cnt = pk_block_sum(cnt, red_i);
+        if (threadIdx.x == 0) {
+            part_sum = sum;
+            part_cnt = cnt;
+        }
+        meet();
+        int ntot = 0;
+        double tot = 0.0;
+#pragma unroll 1
+        for (int r = 0; r < C; ++r) {
+            tot += *of(&part_sum, r);
+            ntot += *of(&part_cnt, r);
+        }
+        const double mean = ntot > 0 ? tot / (double)ntot : NAN;
         double ss = 0.0;
         float mx = -INFINITY;
-        for (int64_t k = threadIdx.x; k < len; k += kPkThreads)
-            if (isfinite(sc[k])) {
-                const double d = (double)sc[k] - mean;
+        for (int64_t k = lo + threadIdx.x; k < hi; k += kPkThreads) {
+            const float v = sc[k];
+            if (isfinite(v)) {
+                const double d = (double)v - mean;
                 ss += d * d;
-                mx = fmaxf(mx, sc[k]);
+                mx = fmaxf(mx, v);
             }
+        }
         ss = pk_block_sum(ss, red_d);
-        {
-            for (int o = 16; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
-            __syncthreads();
-            if ((threadIdx.x & 31) == 0) red_f[threadIdx.x >> 5] = mx;
-            __syncthreads();
-            for (int w = 0; w < kPkThreads / 32; ++w) mx = fmaxf(mx, red_f[w]);
+        mx = pk_block_reduce(mx, red_f, -INFINITY, [](float a, float b) { return fmaxf(a, b); });
+        if (threadIdx.x == 0) {
+            part_ss = ss;
+            part_mx = mx;
+        }
+        meet();
+        ss = 0.0;
+        mx = -INFINITY;
+#pragma unroll 1
+        for (int r = 0; r < C; ++r) {
+            ss += *of(&part_ss, r);
+            mx = fmaxf(mx, *of(&part_mx, r));
         }
         const double sd = ntot > 0 ? sqrt(ss / (double)ntot) : NAN;
         const double thr = mean + p.k_sigma * sd;
-        auto above = [&](int64_t k) { return isfinite(sc[k]) && (double)sc[k] > thr; };
+        // a float is above thr exactly if it is above the largest float not above thr
+        const float thr_f = __double2float_rd(thr);
+        auto above = [&](int64_t k) {
+            const float v = sc[k];
+            return isfinite(v) && v > thr_f;
+        };
         // runs starting in this thread's chunk
-        const int64_t chunk = (len + kPkThreads - 1) / kPkThreads;
-        const int64_t a = (int64_t)threadIdx.x * chunk, b = min(len, a + chunk);
+        const int64_t chunk = (hi - lo + kPkThreads - 1) / kPkThreads;
+        const int64_t a = lo + (int64_t)threadIdx.x * chunk, b = min(hi, a + chunk);
         int64_t i = a;
         if (i < b && i > 0 && above(i - 1))  // the run through a started in an earlier chunk
             while (i < len && above(i)) ++i;
@@ -129,17 +176,29 @@ __global__ void __launch_bounds__(kPkThreads) peaks_kernel(const PeakParams p)
                 ++nq;
                 const unsigned long long key = argmax_key(sc[arg], arg);
                 best = key > best ? key : best;
-                const int slot = atomicAdd(&c_n, 1);
+                const int slot = atomicAdd(of(&c_n, 0), 1);
                 if (slot < kPkCap) {
-                    c_h[slot] = sc[arg];
-                    c_i[slot] = (int)arg;
-                    c_w[slot] = (int)(e - i);
+                    of(c_h, 0)[slot] = sc[arg];
+                    of(c_i, 0)[slot] = (int)arg;
+                    of(c_w, 0)[slot] = (int)(e - i);
                 }
             }
             i = e;
         }
-        const int npk = pk_block_sum(nq, red_i);
+        nq = pk_block_sum(nq, red_i);
         best = pk_block_max(best, red_k);
+        if (threadIdx.x == 0) {
+            of(c_peaks, 0)[rank] = nq;
+            of(c_best, 0)[rank] = best;
+        }
+        meet();  // every block's candidates are in the first one's list
+        if (rank != 0) continue;  // (the next meeting is after the next star's first sums)
+        int npk = 0;
+        best = 0ull;
+        for (int r = 0; r < C; ++r) {
+            npk += c_peaks[r];
+            best = c_best[r] > best ? c_best[r] : best;
+        }
         const int ncand = min(c_n, kPkCap);
         // the highest max_peaks candidates, one block argmax each
         const int nlist = p.peaks ? min(p.max_peaks, ncand) : 0;
@@ -198,10 +257,34 @@ __global__ void __launch_bounds__(kPkThreads) peaks_kernel(const PeakParams p)
     }
 }
 
+// Blocks per star: sixteen where the stars are few and their grids long enough to give every
+// thread of a cluster something (a cluster's meetings cost a few microseconds), else one.
+constexpr int kPkCluster = 16;
+constexpr int64_t kPkLong = 16384;
+
 cudaError_t launch_peaks(const PeakParams &p, int num_sms, cudaStream_t st)
 {
+    if (p.nstars * (int64_t)kPkCluster <= 2 * (int64_t)num_sms && p.np / p.nstars >= kPkLong) {
+        static const cudaError_t attr = cudaFuncSetAttribute(peaks_kernel<kPkCluster>,
+                                                             cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3((unsigned)(p.nstars * kPkCluster));
+        cfg.blockDim = dim3(kPkThreads);
+        cfg.stream = st;
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = kPkCluster;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        int fits = 0;
+        if (attr == cudaSuccess && cudaOccupancyMaxActiveClusters(&fits, peaks_kernel<kPkCluster>, &cfg) == cudaSuccess &&
+            fits > 0)
+            return cudaLaunchKernelEx(&cfg, peaks_kernel<kPkCluster>, p);
+        cudaGetLastError();
+    }
     const int grid = p.nstars < num_sms * 2 ? p.nstars : num_sms * 2;
-    peaks_kernel<<<grid, kPkThreads, 0, st>>>(p);
+    peaks_kernel<1><<<grid, kPkThreads, 0, st>>>(p);
     return cudaGetLastError();
 }
 
