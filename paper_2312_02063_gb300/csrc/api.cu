@@ -35,6 +35,7 @@ struct gpfc_ctx {
         int nbins, mode, lg;
         gpfc_fold_config cfg;
         float ms;
+        bool packed;  // the one-word fold (fold_pack.cu) was the fastest
     };
     std::vector<Tuned> tuned;
     bool autotune = true;
@@ -150,8 +151,14 @@ int ensure_ws(gpfc_ctx *ctx, size_t bytes)
 
 struct FoldPlan {
     int warps, ppc, grid, G, layout, chunk, tile, bps, streams;
+    int packed;  // layout 3 with sum and count in one word (fold_pack.cu); kModeFold only
     int64_t ntasks;
 };
+
+cudaError_t launch_plan(const FoldPlan &pl, const FoldParams &p, int grid, cudaStream_t st)
+{
+    return pl.packed ? launch_fold_pack(p, grid, st) : launch_fold(p, kModeFold, grid, st);
+}
 
 // At 256 bins and more the reduction layout: its updates need no load, so three period
 // groups of 8-byte bins can be folded by twelve warps at once (1.3x the 64-bit
@@ -171,13 +178,61 @@ int floor_log2(int64_t n)
 }
 
 // The tuned config for (nbins, mode, n), if the autotuner has one.
-const gpfc_fold_config *find_tuned(const gpfc_ctx *ctx, int nbins, int mode, int64_t n)
+const gpfc_ctx::Tuned *find_tuned(const gpfc_ctx *ctx, int nbins, int mode, int64_t n)
 {
     if (!ctx->autotune) return nullptr;
     const int lg = floor_log2(n);
     for (const auto &t : ctx->tuned)
-        if (t.nbins == nbins && t.mode == mode && t.lg == lg) return &t.cfg;
+        if (t.nbins == nbins && t.mode == mode && t.lg == lg) return &t;
     return nullptr;
+}
+
+// Whether a fold that writes profiles may take the one-word form of layout 3: wherever that
+// layout is the default (or set), fits (else the FP32 layout runs) and nothing else about the
+// launch is set. Its results are the layout's own, and it was the faster one at every size
+// measured: 192 periods of 62,835 samples and 256 bins in 1.04 M cycles of a multiprocessor,
+// against 2 x 0.755 M (fold_pack.cu); searches by CNN, two words -> one: 250,000 periods
+// 9.6 -> 8.4 ms, 100,000 periods 4.1 -> 3.8 ms.
+bool pack_ok(const gpfc_ctx *ctx, int nbins)
+{
+    const gpfc_fold_config &c = ctx->fold_cfg;
+    return default_layout(nbins) == kLayoutRed32 && (c.layout == 0 || c.layout == kLayoutRed32) && c.warps == 0 &&
+           c.chunk == 0 && c.tile == 0 && c.blocks_per_sm == 0 && c.streams == 0 &&
+           fold_max_warps(nbins, kLayoutRed32, kTile) >= 1 && fold_pack_groups(nbins) >= 1;
+}
+
+// Its plan over np periods in nstars grids of about equal length. A block takes as many
+// period groups as fit (each sample is read once for all), fewer where the grid would leave
+// multiprocessors idle, or where a star's last block would be mostly empty: the cost of a
+// star's blocks is taken as their period groups plus one each for the reading.
+FoldPlan plan_packed(const gpfc_ctx *ctx, int64_t n, int64_t np, int nbins, int64_t nstars)
+{
+    FoldPlan pl{};
+    pl.packed = 1;
+    pl.layout = kLayoutRed32;
+    pl.chunk = kPackChunk;
+    pl.tile = kMaxTile;
+    pl.bps = 1;
+    const int64_t per_sm = (np + (int64_t)32 * ctx->num_sms - 1) / ((int64_t)32 * ctx->num_sms);
+    const int maxg = (int)std::max<int64_t>(1, std::min<int64_t>(fold_pack_groups(nbins), per_sm));
+    pl.warps = maxg;
+    if (nstars > 1) {
+        const int64_t avg = std::max<int64_t>(1, np / nstars);
+        int64_t best = INT64_MAX;
+        for (int g = maxg; g >= 1; --g) {
+            const int64_t cost = (avg + 32 * g - 1) / (32 * g) * (g + 1);
+            if (cost < best) {
+                best = cost;
+                pl.warps = g;
+            }
+        }
+    }
+    pl.ppc = 32 * pl.warps;
+    pl.streams = std::max(1, kMaxRedWarps / pl.warps);
+    pl.ntasks = (np + pl.ppc - 1) / pl.ppc;
+    pl.grid = (int)std::min<int64_t>(pl.ntasks, ctx->num_sms);
+    pl.G = (int)std::min<int64_t>(256, std::max<int64_t>(1, (n + 8191) / 8192));
+    return pl;
 }
 
 // Launch plan of a fold over np periods of stars of about n samples. Fields of the
@@ -225,16 +280,21 @@ FoldPlan plan_with(const gpfc_ctx *ctx, int64_t n, int64_t np, int nbins, const 
     return pl;
 }
 
-FoldPlan plan_fold(gpfc_ctx *ctx, int64_t n, int64_t np, int nbins, const gpfc_fold_config *tuned = nullptr)
+// With `profiles` (the fold writes profiles, for the caller or for a separate scorer) the plan
+// may be the one-word fold's.
+FoldPlan plan_fold(gpfc_ctx *ctx, int64_t n, int64_t np, int nbins, const gpfc_ctx::Tuned *tuned, bool profiles,
+                   int64_t nstars = 1)
 {
     gpfc_fold_config cfg = ctx->fold_cfg;
-    if (tuned) {
-        if (!cfg.warps) cfg.warps = tuned->warps;
-        if (!cfg.layout) cfg.layout = tuned->layout;
-        if (!cfg.tile) cfg.tile = tuned->tile;
-        if (!cfg.blocks_per_sm) cfg.blocks_per_sm = tuned->blocks_per_sm;
+    if (tuned && !tuned->packed) {
+        if (!cfg.warps) cfg.warps = tuned->cfg.warps;
+        if (!cfg.layout) cfg.layout = tuned->cfg.layout;
+        if (!cfg.tile) cfg.tile = tuned->cfg.tile;
+        if (!cfg.blocks_per_sm) cfg.blocks_per_sm = tuned->cfg.blocks_per_sm;
     }
-    const FoldPlan pl = plan_with(ctx, n, np, nbins, cfg);
+    const FoldPlan pl = profiles && pack_ok(ctx, nbins) && (!tuned || tuned->packed)
+                            ? plan_packed(ctx, n, np, nbins, nstars)
+                            : plan_with(ctx, n, np, nbins, cfg);
     ctx->last_plan = gpfc_fold_config{pl.warps, pl.layout, pl.chunk, pl.tile, pl.bps, pl.streams};
     return pl;
 }
@@ -261,8 +321,8 @@ size_t carve_fold(void *base, const FoldPlan &pl, int64_t n_total, int nstars, i
     fb.smp.xq = c.take<int32_t>(se);
     fb.smp.thg = c.take<int32_t>(se / 16 + 64);
     fb.smp.flags = c.take<uint8_t>(se / 16 + 64);
-    fb.ws_sc = c.take<float2>((size_t)pl.grid * nbins * pl.ppc);
-    fb.ws_cnt = c.take<uint32_t>((size_t)pl.grid * nbins * pl.ppc);
+    fb.ws_sc = c.take<float2>((size_t)pl.grid * nbins * pl.ppc * (pl.packed ? kPackPlanes / 2 : 1));
+    fb.ws_cnt = c.take<uint32_t>(pl.packed ? 0 : (size_t)pl.grid * nbins * pl.ppc);
     fb.key = c.take<unsigned long long>(nstars);
     return c.off + 256;
 }
@@ -449,14 +509,14 @@ int run_fold(gpfc_ctx *ctx, const double *times, const float *flux, int64_t n, c
              int64_t np, int32_t nbins, double t0, int mode, FoldParams p, bool want_key,
              FoldBuffers *out_fb)
 {
-    const FoldPlan pl = plan_fold(ctx, n, np, nbins, find_tuned(ctx, nbins, mode, n));
+    const FoldPlan pl = plan_fold(ctx, n, np, nbins, find_tuned(ctx, nbins, mode, n), mode == kModeFold);
     FoldBuffers fb{};
     const size_t need = carve_fold(nullptr, pl, n, 1, nbins, fb);
     int rc = ensure_ws(ctx, need);
     if (rc) return rc;
     carve_fold(ctx->ws, pl, n, 1, nbins, fb);
     cudaError_t e = launch_prep(times, flux, nullptr, n, 1, n, nullptr, t0, fb.smp, fb.partial, pl.G,
-                                fb.stats, ctx->status_dev, ctx->stream, pl.chunk);
+                                fb.stats, ctx->status_dev, ctx->stream, pl.chunk, pl.packed);
     if (e != cudaSuccess) return cuda_err(ctx, e, "prep kernels");
     p.smp = fb.smp;
     p.lc_off = nullptr;
@@ -485,7 +545,7 @@ int run_fold(gpfc_ctx *ctx, const double *times, const float *flux, int64_t n, c
         if (e != cudaSuccess) return cuda_err(ctx, e, "cudaMemsetAsync");
     }
     KernelTimer timer(ctx);
-    e = launch_fold(p, mode, pl.grid, ctx->stream);
+    e = pl.packed ? launch_fold_pack(p, pl.grid, ctx->stream) : launch_fold(p, mode, pl.grid, ctx->stream);
     if (e != cudaSuccess) return cuda_err(ctx, e, "fold kernel");
     timer.stop();
     if (out_fb) *out_fb = fb;
@@ -555,7 +615,7 @@ cudaError_t timed_fold(gpfc_ctx *ctx, cudaStream_t sf, Launch launch)
 // does not fit.
 bool fused_plan(gpfc_ctx *ctx, int64_t n, int64_t np, int nbins, FoldPlan &pl)
 {
-    pl = plan_fold(ctx, n, np, nbins, find_tuned(ctx, nbins, kModeFold, n));
+    pl = plan_fold(ctx, n, np, nbins, find_tuned(ctx, nbins, kModeFold, n), false);
     int bps = search_blocks_per_sm(nbins, pl.warps, pl.layout, pl.tile, pl.streams);
     if (bps < 1 && !ctx->fold_cfg.tile && pl.tile > 512) {
         // the scorer staging did not fit beside 1024-sample tiles: halve the tiles
@@ -604,7 +664,7 @@ int run_search_box_fused(gpfc_ctx *ctx, const double *times, const float *flux, 
     carve_fused(ctx->ws, pl, n, nbins, B);
     const bool want_best = best_index || best_score;
     cudaError_t e = launch_prep(times, flux, nullptr, n, 1, n, nullptr, t0, B.fb.smp, B.fb.partial, pl.G,
-                                B.fb.stats, ctx->status_dev, ctx->stream, pl.chunk);
+                                B.fb.stats, ctx->status_dev, ctx->stream, pl.chunk, pl.packed);
     if (e == cudaSuccess && want_best) e = cudaMemsetAsync(B.fb.key, 0, sizeof(unsigned long long), ctx->stream);
     if (e != cudaSuccess) return cuda_err(ctx, e, "prep kernels");
     FoldParams p{};
@@ -654,12 +714,12 @@ static int chunk_shape(const gpfc_ctx *ctx, const FoldPlan &pl, int64_t nk, Fold
 {
     p.warps = pl.warps;
     p.streams = pl.streams;
-    if (pl.layout == kLayoutRed32 && ctx->fold_cfg.warps == 0 && ctx->fold_cfg.streams == 0) {
+    if (pl.packed || (pl.layout == kLayoutRed32 && ctx->fold_cfg.warps == 0 && ctx->fold_cfg.streams == 0)) {
         const int64_t per_sm = (nk + (int64_t)32 * ctx->num_sms - 1) / ((int64_t)32 * ctx->num_sms);
         const int w = (int)std::max<int64_t>(1, std::min<int64_t>(pl.warps, per_sm));
         if (w < pl.warps) {
             p.warps = w;
-            p.streams = std::max(1, std::min(kMaxRedWarps / w, pl.warps * pl.streams / w));
+            p.streams = std::max(1, std::min(kMaxRedWarps / w, pl.warps * pl.streams / w));  // (one word: unused)
         }
     }
     p.ntasks = (nk + 32 * p.warps - 1) / (32 * p.warps);
@@ -687,7 +747,7 @@ int run_search_box_warp(gpfc_ctx *ctx, const double *times, const float *flux, i
                         int64_t np, int32_t nbins, double t0, const gpfc_box_params *bp, float *score,
                         int64_t *best_index, float *best_score)
 {
-    const FoldPlan pl = plan_fold(ctx, n, np, nbins, find_tuned(ctx, nbins, kModeFold, n));
+    const FoldPlan pl = plan_fold(ctx, n, np, nbins, find_tuned(ctx, nbins, kModeFold, n), true);
     const int64_t chunk = std::min<int64_t>(np, (int64_t)pl.grid * pl.ppc);
     FoldBuffers fb{};
     int rc = ensure_ws(ctx, box_warp_bytes(pl, n, np, nbins));
@@ -703,7 +763,7 @@ int run_search_box_warp(gpfc_ctx *ctx, const double *times, const float *flux, i
     }
     const bool want_best = best_index || best_score;
     cudaError_t e = launch_prep(times, flux, nullptr, n, 1, n, nullptr, t0, fb.smp, fb.partial, pl.G, fb.stats,
-                                ctx->status_dev, ctx->stream, pl.chunk);
+                                ctx->status_dev, ctx->stream, pl.chunk, pl.packed);
     if (e == cudaSuccess && want_best) e = cudaMemsetAsync(fb.key, 0, sizeof(unsigned long long), ctx->stream);
     if (e != cudaSuccess) return cuda_err(ctx, e, "prep kernels");
     KernelTimer timer(ctx);
@@ -727,7 +787,7 @@ int run_search_box_warp(gpfc_ctx *ctx, const double *times, const float *flux, i
         p.counts = cc[b];
         p.status = ctx->status_dev;
         const int grid = chunk_shape(ctx, pl, nk, p);
-        return timed_fold(ctx, sf, [&] { return launch_fold(p, kModeFold, grid, sf); });
+        return timed_fold(ctx, sf, [&] { return launch_plan(pl, p, grid, sf); });
     };
     auto box = [&](int64_t i, int b, cudaStream_t sb) {
         const int64_t k0 = i * chunk, nk = std::min<int64_t>(chunk, np - k0);
@@ -779,7 +839,7 @@ int run_search_cnn(gpfc_ctx *ctx, const double *times, const float *flux, int64_
                    int64_t np, int32_t nbins, double t0, const gpfc_cnn_weights *wt, float *score,
                    int64_t *best_index, float *best_score)
 {
-    const FoldPlan pl = plan_fold(ctx, n, np, nbins, find_tuned(ctx, nbins, kModeFold, n));
+    const FoldPlan pl = plan_fold(ctx, n, np, nbins, find_tuned(ctx, nbins, kModeFold, n), true);
     const int64_t wave = (int64_t)pl.grid * pl.ppc;
     const int64_t chunk = std::min<int64_t>(np, wave);
     const int64_t half = (chunk + 1) / 2;
@@ -809,7 +869,7 @@ int run_search_cnn(gpfc_ctx *ctx, const double *times, const float *flux, int64_
     unsigned long long *key = w.take<unsigned long long>(1);
 
     cudaError_t e = launch_prep(times, flux, nullptr, n, 1, n, nullptr, t0, fb.smp, fb.partial, pl.G, fb.stats,
-                                ctx->status_dev, ctx->stream, pl.chunk);
+                                ctx->status_dev, ctx->stream, pl.chunk, pl.packed);
     if (e == cudaSuccess) e = launch_cnn_prep(cnn_src(wt), dev, ctx->stream);
     if (e != cudaSuccess) return cuda_err(ctx, e, "prep kernels");
     KernelTimer timer(ctx);
@@ -835,7 +895,8 @@ int run_search_cnn(gpfc_ctx *ctx, const double *times, const float *flux, int64_
         p.folded = cf[b];
         p.counts = cc[b];
         p.status = ctx->status_dev;
-        return launch_fold(p, kModeFold, chunk_shape(ctx, pl, nk, p), sf);
+        const int grid = chunk_shape(ctx, pl, nk, p);
+        return launch_plan(pl, p, grid, sf);
     };
     auto cnn = [&](int64_t i, int b, cudaStream_t sb) {
         const int64_t k0 = i * chunk, nk = std::min<int64_t>(chunk, np - k0);
@@ -889,6 +950,7 @@ int tune_fold(gpfc_ctx *ctx, const double *times, const float *flux, int64_t n, 
     struct Cand {
         gpfc_fold_config cfg;
         int resident;
+        bool packed;
     };
     std::vector<Cand> cands;
     int best_res = 0;
@@ -903,18 +965,22 @@ int tune_fold(gpfc_ctx *ctx, const double *times, const float *flux, int64_t n, 
                 const int bps = fold_blocks_per_sm(nbins, w, layout, tile);
                 if (bps < 1) continue;
                 const int res = 32 * w * bps;
-                cands.push_back(Cand{gpfc_fold_config{w, layout, 0, tile, bps}, res});
+                cands.push_back(Cand{gpfc_fold_config{w, layout, 0, tile, bps}, res, false});
                 best_res = std::max(best_res, res);
             }
         }
     }
+    if (mode == kModeFold && pack_ok(ctx, nbins)) cands.push_back(Cand{gpfc_fold_config{}, best_res, true});
+    auto plan_of = [&](const Cand &c) {
+        return c.packed ? plan_packed(ctx, n, P, nbins, 1) : plan_with(ctx, n, P, nbins, c.cfg);
+    };
     if (cands.empty()) return set_err(ctx, GPFC_ENOTSUP, "no fold launch config fits nbins = %d", nbins);
     // workspace: the largest carve of any candidate plus the sample score buffer
     size_t need = 0;
     for (const Cand &c : cands) {
         if (2 * c.resident < best_res) continue;
         FoldBuffers fb{};
-        need = std::max(need, carve_fold(nullptr, plan_with(ctx, n, P, nbins, c.cfg), n, 1, nbins, fb));
+        need = std::max(need, carve_fold(nullptr, plan_of(c), n, 1, nbins, fb));
     }
     int rc = ensure_ws(ctx, need + (size_t)P * sizeof(float) + 512);
     if (rc) return rc;
@@ -922,16 +988,17 @@ int tune_fold(gpfc_ctx *ctx, const double *times, const float *flux, int64_t n, 
     bool prepped = false;
     float best_ms = 0.f;
     gpfc_fold_config best{};
+    bool best_packed = false;
     for (const Cand &c : cands) {
         if (2 * c.resident < best_res) continue;
-        const FoldPlan pl = plan_with(ctx, n, P, nbins, c.cfg);
+        const FoldPlan pl = plan_of(c);
         FoldBuffers fb{};
         carve_fold(ctx->ws, pl, n, 1, nbins, fb);  // the sample scratch sits at the same place for all
         cudaError_t e = cudaSuccess;
-        if (!prepped) {
+        if (!prepped || c.packed) {  // (the one-word fold's candidate, the last, has its own form of the flux)
             // the longest chunk, so the fixed-point flux fits every candidate's chunks
             e = launch_prep(times, flux, nullptr, n, 1, n, nullptr, NAN, fb.smp, fb.partial, pl.G, fb.stats,
-                            ctx->status_dev, ctx->stream, 65520);
+                            ctx->status_dev, ctx->stream, kPackChunk, c.packed);
             if (e != cudaSuccess) return cuda_err(ctx, e, "prep kernels");
             prepped = true;
         }
@@ -959,9 +1026,10 @@ int tune_fold(gpfc_ctx *ctx, const double *times, const float *flux, int64_t n, 
             p.w_max = bp->w_max;
             p.sigma_user = bp->sigma > 0.0 ? (float)bp->sigma : 0.f;
         }
-        e = launch_fold(p, mode, pl.grid, ctx->stream);  // warm-up
+        auto fold = [&] { return pl.packed ? launch_fold_pack(p, pl.grid, ctx->stream) : launch_fold(p, mode, pl.grid, ctx->stream); };
+        e = fold();  // warm-up
         if (e == cudaSuccess) e = cudaEventRecord(ctx->ev_start, ctx->stream);
-        for (int r = 0; r < 2 && e == cudaSuccess; ++r) e = launch_fold(p, mode, pl.grid, ctx->stream);
+        for (int r = 0; r < 2 && e == cudaSuccess; ++r) e = fold();
         if (e == cudaSuccess) e = cudaEventRecord(ctx->ev_stop, ctx->stream);
         if (e == cudaSuccess) e = cudaEventSynchronize(ctx->ev_stop);
         float ms = 0.f;
@@ -972,6 +1040,7 @@ int tune_fold(gpfc_ctx *ctx, const double *times, const float *flux, int64_t n, 
         if (best_ms == 0.f || ms < best_ms) {
             best_ms = ms;
             best = gpfc_fold_config{pl.warps, pl.layout, 0, pl.tile, pl.bps};
+            best_packed = pl.packed != 0;
         }
     }
     ctx->timed = false;
@@ -981,9 +1050,10 @@ int tune_fold(gpfc_ctx *ctx, const double *times, const float *flux, int64_t n, 
         if (t.nbins == nbins && t.mode == mode && t.lg == lg) {
             t.cfg = best;
             t.ms = best_ms;
+            t.packed = best_packed;
             found = true;
         }
-    if (!found) ctx->tuned.push_back(gpfc_ctx::Tuned{nbins, mode, lg, best, best_ms});
+    if (!found) ctx->tuned.push_back(gpfc_ctx::Tuned{nbins, mode, lg, best, best_ms, best_packed});
     if (out) *out = best;
     return GPFC_OK;
 }
@@ -1072,7 +1142,7 @@ cudaError_t enqueue_batched(gpfc_ctx *ctx, const BatchArgs &A, const FoldPlan &p
                                       B.task_off, ctx->status_dev, st);
     if (e == cudaSuccess)
         e = launch_prep(A.times, A.flux, B.lc_s, A.n_total, A.S, 0, A.t0s, NAN, B.fb.smp, B.fb.partial, pl.G,
-                        B.fb.stats, ctx->status_dev, st, pl.chunk);
+                        B.fb.stats, ctx->status_dev, st, pl.chunk, pl.packed);
     if (e != cudaSuccess) return e;
     FoldParams p{};
     p.smp = B.fb.smp;
@@ -1126,7 +1196,7 @@ cudaError_t enqueue_batched(gpfc_ctx *ctx, const BatchArgs &A, const FoldPlan &p
             q.slot_k = B.chunk_k[b];
             q.task_begin = i * wave;
             q.ntasks = std::min<int64_t>(T, q.task_begin + wave);
-            return launch_fold(q, kModeFold, (int)(q.ntasks - q.task_begin), sf);
+            return launch_plan(pl, q, (int)(q.ntasks - q.task_begin), sf);
         };
         auto box = [&](int64_t i, int b, cudaStream_t sb) {
             const int64_t tb = i * wave, te = std::min<int64_t>(T, tb + wave);
@@ -1176,7 +1246,7 @@ cudaError_t enqueue_batched(gpfc_ctx *ctx, const BatchArgs &A, const FoldPlan &p
         q.slot_k = B.chunk_k[b];
         q.task_begin = i * wave;
         q.ntasks = std::min<int64_t>(T, q.task_begin + wave);
-        return launch_fold(q, kModeFold, (int)(q.ntasks - q.task_begin), sf);
+        return launch_plan(pl, q, (int)(q.ntasks - q.task_begin), sf);
     };
     auto cnn = [&](int64_t i, int b, cudaStream_t sb) {
         const int64_t tb = i * wave, te = std::min<int64_t>(T, tb + wave);
@@ -1298,6 +1368,7 @@ int gpfc_create(gpfc_ctx **out, int device, void *stream)
         e = cudaHostGetDevicePointer(reinterpret_cast<void **>(&ctx->status_dev), ctx->status_host, 0);
     }
     if (e == cudaSuccess) e = static_cast<cudaError_t>(fold_register_kernels());
+    if (e == cudaSuccess) e = static_cast<cudaError_t>(fold_pack_register());
     int prio_least = 0, prio_greatest = 0;
     if (e == cudaSuccess) e = cudaDeviceGetStreamPriorityRange(&prio_least, &prio_greatest);
     if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&ctx->side[0], cudaStreamNonBlocking, prio_greatest);
@@ -1448,10 +1519,11 @@ int gpfc_workspace_size(gpfc_ctx *ctx, int64_t n, int64_t n_periods, int32_t nbi
     // the largest of a fold (gpfc_fold, the epilogue search), the warp-per-profile search
     // and the one-kernel search; planning them leaves the context's last plan as it was
     const gpfc_fold_config last = ctx->last_plan;
-    const FoldPlan pb = plan_fold(ctx, n, n_periods, nbins, find_tuned(ctx, nbins, kModeBox, n));
-    const FoldPlan pf = plan_fold(ctx, n, n_periods, nbins, find_tuned(ctx, nbins, kModeFold, n));
+    const FoldPlan pb = plan_fold(ctx, n, n_periods, nbins, find_tuned(ctx, nbins, kModeBox, n), false);
+    const FoldPlan pf = plan_fold(ctx, n, n_periods, nbins, find_tuned(ctx, nbins, kModeFold, n), true);
     FoldBuffers fb{};
-    *bytes = std::max(carve_fold(nullptr, pb, n, 1, nbins, fb), box_warp_bytes(pf, n, n_periods, nbins));
+    *bytes = std::max(carve_fold(nullptr, pb, n, 1, nbins, fb), carve_fold(nullptr, pf, n, 1, nbins, fb));
+    *bytes = std::max(*bytes, box_warp_bytes(pf, n, n_periods, nbins));
     FoldPlan ps{};
     if (fused_plan(ctx, n, n_periods, nbins, ps)) {
         FusedBuffers B{};
@@ -2081,8 +2153,9 @@ int gpfc_search_batched(gpfc_ctx *ctx, int32_t n_stars, const int64_t *lc_offset
     if (e != cudaSuccess) return cuda_err(ctx, e, "cudaStreamIsCapturing");
     const bool capturing = cs != cudaStreamCaptureStatusNone;
     const int64_t n_avg = n_total / n_stars;
-    const gpfc_fold_config *tuned = find_tuned(ctx, nbins, mode, n_avg);
-    if (!tuned && ctx->autotune && !capturing) {
+    const gpfc_ctx::Tuned *tuned = find_tuned(ctx, nbins, mode, n_avg);
+    const bool pack = mode == kModeFold && pack_ok(ctx, nbins);
+    if (!tuned && ctx->autotune && !capturing && !pack) {
         // tune on the first star (its offsets are read back once)
         int64_t off[2] = {0, 0};
         e = cudaMemcpyAsync(off, lc_offsets, sizeof(off), cudaMemcpyDeviceToHost, ctx->stream);
@@ -2096,14 +2169,14 @@ int gpfc_search_batched(gpfc_ctx *ctx, int32_t n_stars, const int64_t *lc_offset
             tuned = find_tuned(ctx, nbins, mode, n_avg);
         }
     }
-    FoldPlan pl = plan_fold(ctx, n_avg, n_periods_total, nbins, tuned);
-    if (A.box_warp && ctx->box_path != GPFC_BOX_WARP) {
+    FoldPlan pl = plan_fold(ctx, n_avg, n_periods_total, nbins, tuned, mode == kModeFold, n_stars);
+    if (A.box_warp && ctx->box_path != GPFC_BOX_WARP && !(pl.packed && ctx->box_path == GPFC_BOX_AUTO)) {
         // the one-kernel search, with the tuned fold config if its block fits, else the
         // default one
-        FoldPlan ps = pl;
+        FoldPlan ps = pl.packed ? plan_fold(ctx, n_avg, n_periods_total, nbins, tuned, false) : pl;
         int bps = search_blocks_per_sm(nbins, ps.warps, ps.layout, ps.tile, ps.streams);
         if (bps < 1) {
-            ps = plan_fold(ctx, n_avg, n_periods_total, nbins, nullptr);
+            ps = plan_fold(ctx, n_avg, n_periods_total, nbins, nullptr, false);
             bps = search_blocks_per_sm(nbins, ps.warps, ps.layout, ps.tile, ps.streams);
         }
         // a block numbers the rows of its tasks in 32-bit tickets

@@ -240,10 +240,11 @@ constexpr int32_t kThMixed = INT32_MIN;  // per-group high word marker: the samp
 // word of tau is the same for all 16 (it changes every 2^32 units, ~256 d). The fold
 // skips its per-group bin-collision check on flagged groups when the period allows it,
 // and forms their phases with one th * F_lo product per group. The same pass writes the
-// fixed-point flux xq = rint(x 2^qexp) when the scratch has room for it.
+// fixed-point flux xq = rint(x 2^qexp) when the scratch has room for it, with pack_chunk > 0 as
+// the one-word fold's increment xq + 2^S + L.
 // grid = (G, stars).
 __global__ void prep_flags_kernel(const int64_t *lc_off, int64_t n, SampleScratch smp,
-                                  const StarStats *stats)
+                                  const StarStats *stats, int pack_chunk)
 {
     const int s = blockIdx.y;
     int64_t b, e;
@@ -252,6 +253,7 @@ __global__ void prep_flags_kernel(const int64_t *lc_off, int64_t n, SampleScratc
     const int64_t base = scratch_start(b, s);
     const long long d0 = stats[s].dtau0;
     const int64_t ngroups = (len + 255) / 256 * 16;  // every flag byte of the star's region
+    const uint32_t add = pack_chunk > 0 ? pack_word(len, pack_chunk).add() : 0u;
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < ngroups;
          q += (int64_t)gridDim.x * blockDim.x) {
         const int64_t j0 = q * 16;
@@ -285,7 +287,8 @@ __global__ void prep_flags_kernel(const int64_t *lc_off, int64_t n, SampleScratc
             // even); zero past the star's end
             const double sc = ldexp(1.0, stats[s].qexp);
             for (int k = 0; k < 16; ++k)
-                smp.xq[base + j0 + k] = j0 + k < len ? __double2int_rn((double)smp.x[base + j0 + k] * sc) : 0;
+                smp.xq[base + j0 + k] =
+                    j0 + k < len ? (int32_t)((uint32_t)__double2int_rn((double)smp.x[base + j0 + k] * sc) + add) : 0;
         }
     }
 }
@@ -293,7 +296,7 @@ __global__ void prep_flags_kernel(const int64_t *lc_off, int64_t n, SampleScratc
 cudaError_t launch_prep(const double *times, const float *flux, const int64_t *lc_off, int64_t n,
                         int nstars, int64_t max_len, const double *t0s, double t0, SampleScratch smp,
                         double *partial, int G, StarStats *stats, uint32_t *status, cudaStream_t st,
-                        int chunk)
+                        int chunk, bool packed)
 {
     (void)max_len;
     dim3 grid(G, nstars);
@@ -302,7 +305,7 @@ cudaError_t launch_prep(const double *times, const float *flux, const int64_t *l
     prep_quant_kernel<<<grid, 256, 0, st>>>(times, flux, lc_off, n, t0s, t0, partial, pmin, smp, stats,
                                             status);
     prep_sigma_kernel<<<nstars, 32, 0, st>>>(partial, pmin, G, nstars, chunk < 16 ? 16 : chunk, stats);
-    prep_flags_kernel<<<grid, 256, 0, st>>>(lc_off, n, smp, stats);
+    prep_flags_kernel<<<grid, 256, 0, st>>>(lc_off, n, smp, stats, packed ? chunk : 0);
     return cudaGetLastError();
 }
 

@@ -210,6 +210,31 @@ __device__ __forceinline__ void report_error(uint32_t *status, uint32_t bits)
     if (status) atomicOr(status, bits);
 }
 
+// The star-dependent constants of the one-word fold's words (fold_pack.cu): the bound L of
+// |xq|, the shift S of the count and the largest count M a segment may leave in a bin.
+struct PackWord {
+    uint32_t L, M;
+    int S;
+    __device__ uint32_t add() const { return (1u << S) + L; }  // a sample's increment is xq + add()
+};
+
+__device__ __forceinline__ PackWord pack_word(int64_t nsamp, int chunk)
+{
+    PackWord w;
+    const uint32_t lmax = (uint32_t)max((int64_t)1, min((int64_t)chunk, nsamp));
+    w.L = 2147483647u / lmax;
+    w.M = 0;
+    w.S = 31;
+    for (int S = 31; S >= 16; --S) {
+        const uint32_t m = min((uint32_t)(((1ull << S) - 1ull) / (2ull * w.L)), (uint32_t)((1ull << (32 - S)) - 1ull));
+        if (m > w.M) {
+            w.M = m;
+            w.S = S;
+        }
+    }
+    return w;
+}
+
 // Sortable 64-bit key for (score, index): larger score wins, ties -> smaller index,
 // NaN never wins (maps below every number).
 __device__ __forceinline__ unsigned long long argmax_key(float s, long long k)

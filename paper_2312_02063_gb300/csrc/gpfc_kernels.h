@@ -40,7 +40,8 @@ struct SampleScratch {
     uint32_t *tau_lo;   // low 32 bits of tau
     int32_t *tau_hi;    // high 32 bits of tau
     float *x;           // flux - f_ref (FP32)
-    int32_t *xq;        // rint(x 2^qexp): the fixed-point flux of the reduction layout
+    int32_t *xq;        // rint(x 2^qexp): the fixed-point flux of the reduction layout (for the
+                        // one-word fold, with 2^S + L added)
     int32_t *thg;       // one word per 16 samples: tau_hi of the group's first sample
     uint8_t *flags;     // one byte per 16 samples: regular-cadence group (see prep)
 };
@@ -134,8 +135,20 @@ int fold_register_kernels();
 cudaError_t launch_prep(const double *times, const float *flux, const int64_t *lc_off, int64_t n,
                         int nstars, int64_t max_len, const double *t0s, double t0, SampleScratch smp,
                         double *partial, int G, StarStats *stats, uint32_t *status, cudaStream_t st,
-                        int chunk = 65520);
+                        int chunk = 65520, bool packed = false);
 cudaError_t launch_fold(const FoldParams &p, int mode, int grid, cudaStream_t st);
+// The reduction layout's fold with sum and count in one word (kModeFold, fold_pack.cu):
+// p.warps period groups of 32, p.chunk = kPackChunk, p.tile and p.streams unused. The block's
+// shared memory, the most groups a block holds (0: none fits) and the kernels' registration.
+constexpr int kPackMaxGroups = 6;
+constexpr int kPackChunk = 65520;
+constexpr int kPackSegs = 4;                  // segments of a star whose words go to slots
+constexpr int kPackPlanes = 3 + kPackSegs - 1;  // 32-bit words of workspace (ws_sc) per bin and period of a
+                                                // resident block: totals (3) and slots
+size_t fold_pack_smem(int nbins, int groups);
+int fold_pack_groups(int nbins);
+int fold_pack_register();
+cudaError_t launch_fold_pack(const FoldParams &p, int grid, cudaStream_t st);
 // Shared memory of a kModeSearch block (0 if it does not fit or warps + 1 > 4).
 size_t search_smem_bytes(int nbins, int warps, int layout, int tile, int streams = 1);
 int search_blocks_per_sm(int nbins, int warps, int layout, int tile, int streams = 1);
