@@ -1494,6 +1494,375 @@ __device__ __forceinline__ void score_row(const BoxCoopParams &p, int64_t r, int
     }
 }
 
+// ------------------------------------------------------------------ box-SNR by maximum, then exactly
+
+// The separate scorer (box_coop_kernel). The walk above keeps each start's best box by
+// cross-multiplied comparisons: two compares to a mask (4 cycles each per warp and scheduler) and
+// three bit selects (2 each) per pair of boxes, and the ALU bounds it. Here a warp first takes
+// only the maximum of v = D / sqrt(q) over each start's boxes, with an approximate reciprocal
+// square root (nine instructions for two boxes), and then replays the walk's own comparisons on
+// the few starts and boxes whose v lies within kNear of the profile's largest. v is off by a few
+// 2^-23, the walk's products by 2^-23: a box further below the largest can neither win the walk
+// nor decide which of the near ones does, so the box, and every output, is the walk's. Profiles
+// with more than kMaxNearStarts near starts (a flat one: every box 0) go through the walk itself.
+// What bounds it now: instruction issue. 29,184 profiles of 256 bins, widths 1..108: see
+// kCoopBlocks.
+constexpr float kNear = 1e-5f;
+constexpr int kMaxNearStarts = 8;
+
+// (sum, count) pairs of one profile staged by a warp, circularly continued past its end, at
+// index b + b / 8 (so b's that differ by 8 lie in different banks): a walk of w_max bins from
+// any start needs no wrap, and eight steps from a multiple of 8 are at fixed offsets. The replay's
+// prefixes follow.
+__host__ __device__ inline int scan_bins(int nbins, int w_max) { return nbins + w_max + kCoopR; }
+__host__ __device__ inline int scan_pairs(int nbins, int w_max)
+{
+    return coop_pairs(scan_bins(nbins, w_max)) + w_max + 2 * kCoopR;
+}
+
+__device__ __forceinline__ float rsqrt_approx(float x)
+{
+    float r;
+    asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+    return r;
+}
+__device__ __forceinline__ unsigned long long f2fma(unsigned long long a, unsigned long long b, unsigned long long c)
+{
+    unsigned long long d;
+    asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(d) : "l"(a), "l"(b), "l"(c));
+    return d;
+}
+
+// mx[r] = largest v of the boxes of start s0 + r and w_min..w_max bins (-inf if none is valid).
+// QCHECK as in box_walk. The prefix A and every D and q are box_walk's, operation by operation.
+template <bool QCHECK>
+__device__ __forceinline__ void box_scan8(const float2 *B, int s0, int w_min, int w_max, float Stot, float Ntot,
+                                          float (&mx)[kCoopR])
+{
+    constexpr int R = kCoopR;
+    const float2 *b8 = B + s0 + (s0 >> 3);  // s0 is a multiple of 8: step t is b8[t + t / 8]
+    float bA[R] = {}, bN[R] = {};
+    float runA = 0.f, runN = 0.f;
+    auto step = [&](float2 v) {
+        runA = fmaf(Stot, v.y, fmaf(-Ntot, v.x, runA));
+        runN += v.y;
+    };
+    auto eval = [&](int r, bool ok) {
+        const float nin = runN - bN[r];
+        const float q = nin * (Ntot - nin);
+        const float v = (runA - bA[r]) * rsqrt_approx(q);
+        mx[r] = fmaxf(mx[r], ok && (!QCHECK || q >= 1.f) ? v : -INFINITY);
+    };
+#pragma unroll
+    for (int r = 0; r < R; ++r) mx[r] = -INFINITY;
+    const bool plain = w_min == 1 && w_max >= R;  // (the usual case: no width test anywhere)
+    // start r is entered at t = r
+#pragma unroll
+    for (int t = 0; t < R; ++t) {
+        bA[t] = runA;
+        bN[t] = runN;
+        step(b8[t]);
+        if (plain) {
+#pragma unroll
+            for (int r = 0; r <= t; ++r) eval(r, true);
+        } else {
+#pragma unroll
+            for (int r = 0; r <= t; ++r) {
+                const int w = t - r + 1;
+                eval(r, (w >= w_min) & (w <= w_max));
+            }
+        }
+    }
+    const int tend = R - 1 + w_max;  // exclusive
+    // steps at which every start's box is valid
+    const int ta = min(max(R, w_min + R - 2), tend), tb = max(ta, min(w_max, tend));
+    int t = R;
+    auto edge = [&](int t1) {
+#pragma unroll 1
+        for (; t < t1; ++t) {
+            step(b8[t + (t >> 3)]);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int w = t - r + 1;
+                eval(r, (w >= w_min) & (w <= w_max));
+            }
+        }
+    };
+    if (!plain) edge(min(tb, (ta + 7) & ~7));
+    unsigned long long nbN2[R / 2], cN2[R / 2], nbA2[R / 2];
+    const unsigned long long minus1 = f2pack(-1.f, -1.f);
+#pragma unroll
+    for (int h = 0; h < R / 2; ++h) {
+        nbN2[h] = f2pack(-bN[2 * h], -bN[2 * h + 1]);
+        cN2[h] = f2pack(Ntot + bN[2 * h], Ntot + bN[2 * h + 1]);
+        nbA2[h] = f2pack(-bA[2 * h], -bA[2 * h + 1]);
+    }
+    auto full = [&](float2 v) {  // one step, every start's box valid
+        step(v);
+        const unsigned long long RN2 = f2pack(runN, runN), RA2 = f2pack(runA, runA);
+#pragma unroll
+        for (int h = 0; h < R / 2; ++h) {
+            const unsigned long long q2 = f2mul(f2add(RN2, nbN2[h]), f2fma(RN2, minus1, cN2[h]));
+            float q0, q1, v0, v1;
+            f2unpack(q2, q0, q1);
+            f2unpack(f2mul(f2add(RA2, nbA2[h]), f2pack(rsqrt_approx(q0), rsqrt_approx(q1))), v0, v1);
+            if (QCHECK) {
+                v0 = q0 >= 1.f ? v0 : -INFINITY;
+                v1 = q1 >= 1.f ? v1 : -INFINITY;
+            }
+            // (an empty box has D = 0 and q = 0: 0 x inf is NaN, which a maximum passes over)
+            mx[2 * h] = fmaxf(mx[2 * h], v0);
+            mx[2 * h + 1] = fmaxf(mx[2 * h + 1], v1);
+        }
+    };
+#pragma unroll 1
+    for (; t + 8 <= tb; t += 8) {
+        const float2 *b = b8 + t + (t >> 3);
+        float2 v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = b[u];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) full(v[u]);
+    }
+    if (plain) {
+#pragma unroll 1
+        for (; t < tb; ++t) full(b8[t + (t >> 3)]);
+        // start r's last box ends at step w_max - 1 + r
+#pragma unroll
+        for (int u = 0; u < R - 1; ++u) {
+            step(b8[t + u + ((t + u) >> 3)]);
+#pragma unroll
+            for (int r = u + 1; r < R; ++r) eval(r, true);
+        }
+    } else {
+        edge(tend);
+    }
+}
+
+// The walk's best box of start s among those of v >= near, by box_walk's comparisons in its
+// order (32 widths at a time), merged into (bv, bkey) by its rule. `pre` is room for the
+// prefixes (A, N) after each step of the start's block of eight.
+__device__ __forceinline__ void box_replay(const float2 *B, float2 *pre, int s, int w_min, int w_max, float Stot,
+                                           float Ntot, float near, int lane, float &bv, int &bkey)
+{
+    const int s0 = s & ~(kCoopR - 1), r = s - s0;
+    const float2 *b8 = B + s0 + (s0 >> 3);
+    const int nsteps = r + w_max;
+    float runA = 0.f, runN = 0.f;
+    __syncwarp();
+    for (int t = 0; t < nsteps; t += 8) {  // (up to seven steps past the end: staged bins, unused)
+        float2 v[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) v[u] = b8[t + (t >> 3) + u];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            runA = fmaf(Stot, v[u].y, fmaf(-Ntot, v[u].x, runA));
+            runN += v[u].y;
+            if (lane == 0) pre[t + u] = make_float2(runA, runN);
+        }
+    }
+    __syncwarp();
+    const float2 b = r > 0 ? pre[r - 1] : make_float2(0.f, 0.f);
+    float rE = -INFINITY, rq = 1.f;
+    int rw = -1;
+    for (int w0 = 1; w0 <= w_max; w0 += 32) {
+        const int w = w0 + lane;
+        const float2 e = pre[min(r + w, nsteps) - 1];
+        const float nin = e.y - b.y;
+        const float q = nin * (Ntot - nin);
+        const float D = e.x - b.x;
+        const float E = D * fabsf(D);
+        unsigned cand = __ballot_sync(0xffffffffu, w <= w_max && w >= w_min && q >= 1.f && D * rsqrt_approx(q) >= near);
+        while (cand) {
+            const int l = __ffs((int)cand) - 1;
+            cand &= cand - 1;
+            const float Ej = __shfl_sync(0xffffffffu, E, l), qj = __shfl_sync(0xffffffffu, q, l);
+            if (Ej * rq > rE * qj) {
+                rE = Ej;
+                rq = qj;
+                rw = w0 + l;
+            }
+        }
+    }
+    if (rw >= 0) {
+        const float vr = rE >= 0.f ? sqrtf(rE / rq) : -sqrtf(-rE / rq);
+        const int key = (rw << 12) | s;
+        const bool take = (vr > bv) | ((vr == bv) & (key < bkey));
+        bv = take ? vr : bv;
+        bkey = take ? key : bkey;
+    }
+}
+
+// a + b as a pair (TwoSum)
+__device__ __forceinline__ void two_sum(float a, float b, float &s, float &e)
+{
+    s = a + b;
+    const float bb = s - a;
+    e = (a - (s - bb)) + (b - bb);
+}
+
+// What the FP64 re-evaluation of a profile's best box needs.
+struct BoxWinner {
+    float sth, stl, sih, sil;  // total and in-box sums, double-float
+    uint32_t nt, ni;
+    int key;                   // w << 12 | s, or 0x7fffffff
+};
+
+// The best box of row r of p's profile buffer, by the calling warp, staged in Bw.
+__device__ __forceinline__ BoxWinner scan_row(const BoxCoopParams &p, int64_t r, float2 *Bw, int lane)
+{
+    const int nbins = p.nbins;
+    const float *srow = p.sums ? p.sums + (size_t)r * nbins : nullptr;
+    const float *mrow = p.means ? p.means + (size_t)r * nbins : nullptr;
+    const int32_t *crow = p.counts + (size_t)r * nbins;
+    float Stot = 0.f, Ntot = 0.f;
+    int nnz = 0;
+    __syncwarp();  // the previous profile's readers are done
+    float mref = 0.f;
+    if (mrow) {
+        // means in: centre them on the profile's count-weighted mean. Its sum is a double-float
+        // (products split by an FMA, TwoSum): FP64 runs at one warp instruction per 64 cycles.
+        float nh = 0.f, nl = 0.f;
+        int den = 0;
+        for (int b = lane; b < nbins; b += 32) {
+            const int32_t c = crow[b];
+            if (c > 0) {
+                const float m = mrow[b], cf = (float)c, pr = m * cf;
+                float e;
+                two_sum(nh, pr, nh, e);
+                nl += e + fmaf(m, cf, -pr);
+                den += c;
+            }
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            const float oh = __shfl_xor_sync(0xffffffffu, nh, o), ol = __shfl_xor_sync(0xffffffffu, nl, o);
+            float e;
+            two_sum(nh, oh, nh, e);
+            nl += ol + e;
+            den += __shfl_xor_sync(0xffffffffu, den, o);
+        }
+        if (den > 0) {  // num / den: the rounded quotient and its remainder's
+            const float d = (float)den, q = nh / d;
+            mref = q + (fmaf(-q, d, nh) + nl) / d;
+        }
+    }
+    // 256 bins at a time, every load issued before any is used: one L2 round trip per
+    // 256 bins
+    const int ext = scan_bins(nbins, p.w_max) - nbins;  // bins continued past the end
+    for (int b0 = 0; b0 < nbins; b0 += 256) {
+        float vv[8];
+        int32_t cv[8];
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int b = b0 + 32 * u + lane;
+            cv[u] = b < nbins ? crow[b] : 0;
+            vv[u] = b < nbins ? (mrow ? mrow[b] : srow[b]) : 0.f;
+        }
+#pragma unroll
+        for (int u = 0; u < 8; ++u) {
+            const int b = b0 + 32 * u + lane;
+            if (b < nbins) {
+                const float c = (float)max(cv[u], 0);
+                const float sv = mrow ? (c > 0.f ? (vv[u] - mref) * c : 0.f) : vv[u];
+                for (int x = b; x < nbins + ext; x += nbins) Bw[x + (x >> 3)] = make_float2(sv, c);
+                Stot += sv;
+                Ntot += c;
+                nnz += c > 0.f;
+            }
+        }
+    }
+    for (int o = 16; o > 0; o >>= 1) {  // a butterfly leaves the same totals in every lane
+        Stot += __shfl_xor_sync(0xffffffffu, Stot, o);
+        Ntot += __shfl_xor_sync(0xffffffffu, Ntot, o);
+        nnz += __shfl_xor_sync(0xffffffffu, nnz, o);
+    }
+    __syncwarp();
+    // the largest v of the profile, then the starts near it
+    const bool unchecked = p.w_max < nnz;
+    float top = -INFINITY, bv = -INFINITY;
+    int bkey = 0x7fffffff;
+    int nnear = 0;
+    for (int pass0 = 0; pass0 < nbins; pass0 += 32 * kCoopR) {
+        const int s0 = pass0 + lane * kCoopR;
+        float mx[kCoopR];
+#pragma unroll
+        for (int i = 0; i < kCoopR; ++i) mx[i] = -INFINITY;
+        if (s0 < nbins) {
+            if (unchecked) box_scan8<false>(Bw, s0, p.w_min, p.w_max, Stot, Ntot, mx);
+            else box_scan8<true>(Bw, s0, p.w_min, p.w_max, Stot, Ntot, mx);
+        }
+        float big = -INFINITY;
+#pragma unroll
+        for (int i = 0; i < kCoopR; ++i) {
+            if (s0 + i >= nbins) mx[i] = -INFINITY;
+            big = fmaxf(big, mx[i]);
+        }
+        for (int o = 16; o > 0; o >>= 1) big = fmaxf(big, __shfl_xor_sync(0xffffffffu, big, o));
+        if (big == -INFINITY) continue;
+        // (a later pass with a larger top replays its own starts; those replayed before stay
+        // correct candidates: the merge keeps the larger)
+        top = fmaxf(top, big);
+        const float near = fabsf(top) < INFINITY ? top - kNear * fabsf(top) : top;
+        uint32_t mine = 0u;
+#pragma unroll
+        for (int i = 0; i < kCoopR; ++i) mine |= (mx[i] >= near ? 1u : 0u) << i;
+        int n = __popc(mine);
+        for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
+        nnear += n;
+        if (nnear > kMaxNearStarts) break;
+        unsigned lanes = __ballot_sync(0xffffffffu, mine != 0u);
+        while (lanes) {
+            const int l = __ffs((int)lanes) - 1;
+            lanes &= lanes - 1;
+            uint32_t m = __shfl_sync(0xffffffffu, mine, l);
+            while (m) {
+                const int i = __ffs((int)m) - 1;
+                m &= m - 1;
+                box_replay(Bw, Bw + coop_pairs(scan_bins(nbins, p.w_max)), pass0 + l * kCoopR + i, p.w_min, p.w_max, Stot, Ntot, near, lane, bv, bkey);
+            }
+        }
+    }
+    const PairBins B{Bw};
+    if (nnear > kMaxNearStarts) {
+        bv = -INFINITY;
+        bkey = 0x7fffffff;
+        if (unchecked)
+            box_walk<kCoopR, false>(B, nbins, p.w_min, p.w_max, Stot, Ntot, lane * kCoopR, 32 * kCoopR, bv, bkey);
+        else
+            box_walk<kCoopR, true>(B, nbins, p.w_min, p.w_max, Stot, Ntot, lane * kCoopR, 32 * kCoopR, bv, bkey);
+        for (int o = 16; o > 0; o >>= 1) {
+            const float ov = __shfl_xor_sync(0xffffffffu, bv, o);
+            const int okey = __shfl_xor_sync(0xffffffffu, bkey, o);
+            const bool take = (ov > bv) | ((ov == bv) & (okey < bkey));
+            bv = take ? ov : bv;
+            bkey = take ? okey : bkey;
+        }
+    }
+    BoxWinner W{0.f, 0.f, 0.f, 0.f, 0u, 0u, bkey};
+    if (bkey != 0x7fffffff) {
+        const int bw = bkey >> 12, bs = bkey & 4095;
+        for (int b = lane; b < nbins; b += 32) {
+            const float2 v = B.sc(b);
+            const uint32_t c = (uint32_t)v.y;
+            two_sum_acc(W.sth, W.stl, v.x);
+            W.nt += c;
+            int d = b - bs;
+            d += d < 0 ? nbins : 0;
+            if (d < bw) {
+                two_sum_acc(W.sih, W.sil, v.x);
+                W.ni += c;
+            }
+        }
+        for (int o = 16; o > 0; o >>= 1) {
+            two_sum_merge(W.sth, W.stl, __shfl_xor_sync(0xffffffffu, W.sth, o), __shfl_xor_sync(0xffffffffu, W.stl, o));
+            two_sum_merge(W.sih, W.sil, __shfl_xor_sync(0xffffffffu, W.sih, o), __shfl_xor_sync(0xffffffffu, W.sil, o));
+            W.nt += __shfl_xor_sync(0xffffffffu, W.nt, o);
+            W.ni += __shfl_xor_sync(0xffffffffu, W.ni, o);
+        }
+    }
+    return W;
+}
+
 // ---------------------------------------------------------------- fold + box-SNR in one kernel
 
 // Work of the box-SNR scorer inside a search block. Tickets number the rows of the block's
@@ -2213,30 +2582,77 @@ cudaError_t launch_fold(const FoldParams &p_in, int mode, int grid, cudaStream_t
     return cudaGetLastError();
 }
 
-__global__ void __launch_bounds__(kCoopWarps * 32, 2) box_coop_kernel(const BoxCoopParams p)
+// One profile per warp at a time. The FP64 tail of the score runs once per 32 profiles, one
+// profile a lane (a division, a square root and a dozen FP64 operations: a tail per profile
+// costs as much as a third of its search).
+__global__ void __launch_bounds__(kCoopWarps * 32, kCoopBlocks) box_coop_kernel(const BoxCoopParams p)
 {
     extern __shared__ __align__(128) uint8_t smem[];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nw = blockDim.x >> 5;
-    float2 *Bw = reinterpret_cast<float2 *>(smem) + (size_t)warp * coop_pairs(p.nbins);
-    int cur_s = -1;
-    unsigned long long cur_key = 0ull;
+    float2 *Bw = reinterpret_cast<float2 *>(smem) + (size_t)warp * scan_pairs(p.nbins, p.w_max);
+    BoxWinner mine{};
+    int64_t my_k = -1;
+    int held = 0;
+    auto finish = [&]() {
+        unsigned long long key = 0ull;
+        int s = -1;
+        if (my_k >= 0) {
+            s = p.grid_off ? star_of(p.grid_off, p.nstars, my_k) : 0;
+            float sc = -INFINITY;
+            const bool any = mine.key != 0x7fffffff;
+            if (any) {
+                float sig = p.sigma_user;
+                if (!(sig > 0.f) && p.stats) sig = p.stats[s].sigma;
+                if (!(sig > 0.f)) sig = 1.f;
+                const double St = (double)mine.sth + (double)mine.stl, Si = (double)mine.sih + (double)mine.sil;
+                const double Nt = (double)mine.nt, Ni = (double)mine.ni, No = (double)(mine.nt - mine.ni);
+                sc = (float)((St * Ni - Si * Nt) / ((double)sig * sqrt(Nt * Ni * No)));
+            }
+            p.score[my_k] = sc;
+            if (p.best_s) p.best_s[my_k] = any ? mine.key & 4095 : -1;
+            if (p.best_w) p.best_w[my_k] = any ? mine.key >> 12 : -1;
+            key = argmax_key(sc, my_k - (p.grid_off ? p.grid_off[s] : 0));
+        }
+        if (p.best_key) {
+            // one atomic per star among the lanes' profiles
+            unsigned left = __ballot_sync(0xffffffffu, my_k >= 0);
+            while (left) {
+                const int l = __ffs((int)left) - 1;
+                const int star = __shfl_sync(0xffffffffu, s, l);
+                const unsigned long long k = warp_max_u64(s == star ? key : 0ull);
+                if (lane == l && k) atomicMax(&p.best_key[star], k);
+                left &= ~__ballot_sync(0xffffffffu, s == star);
+            }
+        }
+        my_k = -1;
+        held = 0;
+    };
     for (int64_t r = (int64_t)blockIdx.x * nw + warp; r < p.rows; r += (int64_t)gridDim.x * nw) {
         const int64_t k = p.slot_k ? p.slot_k[r] : p.k_begin + r;
-        if (k >= 0) score_row(p, r, k, Bw, lane, cur_s, cur_key);
+        if (k < 0) continue;
+        const BoxWinner W = scan_row(p, r, Bw, lane);
+        if (lane == held) {
+            mine = W;
+            my_k = k;
+        }
+        if (++held == 32) finish();
     }
-    if (lane == 0 && p.best_key && cur_key) atomicMax(&p.best_key[cur_s], cur_key);
+    finish();
 }
 
-// Warps per block of the scorer: 8, fewer when 8 profiles do not fit shared memory.
-int box_coop_warps(int nbins)
+static size_t box_coop_bytes(int nbins, int w_max, int warps)
+{
+    return (size_t)warps * scan_pairs(nbins, w_max) * sizeof(float2);
+}
+
+// Warps per block of the scorer: kCoopWarps, fewer when their profiles do not fit shared memory.
+static int box_coop_warps(int nbins, int w_max)
 {
     int w = kCoopWarps;
-    while (w > 1 && (size_t)w * coop_pairs(nbins) * sizeof(float2) > kSmemLimit - 1024) --w;
+    while (w > 1 && box_coop_bytes(nbins, w_max, w) > kSmemLimit - 1024) --w;
     return w;
 }
-
-size_t box_coop_smem(int nbins) { return (size_t)box_coop_warps(nbins) * coop_pairs(nbins) * sizeof(float2); }
 
 cudaError_t box_coop_register()
 {
@@ -2246,9 +2662,9 @@ cudaError_t box_coop_register()
 cudaError_t launch_box_coop(const BoxCoopParams &p, int num_sms, cudaStream_t st)
 {
     if (p.rows <= 0) return cudaSuccess;
-    const size_t smem = box_coop_smem(p.nbins);
+    const int warps = box_coop_warps(p.nbins, p.w_max);
+    const size_t smem = box_coop_bytes(p.nbins, p.w_max, warps);
     if (smem > kSmemLimit - 1024) return cudaErrorInvalidValue;
-    const int warps = box_coop_warps(p.nbins);
     int occ = 0;
     cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, box_coop_kernel, warps * 32, smem);
     if (e != cudaSuccess) return e;

@@ -123,8 +123,8 @@ struct BoxCoopParams {
 // float2 (sum, count) slots one warp of the scorer stages per profile
 __host__ __device__ inline int coop_pairs(int nbins) { return nbins + (nbins >> 3) + 2; }
 constexpr int kCoopWarps = 8;  // warps per block of the scorer
+constexpr int kCoopBlocks = 3; // and blocks per multiprocessor its registers leave room for
 
-size_t box_coop_smem(int nbins);
 cudaError_t launch_box_coop(const BoxCoopParams &p, int num_sms, cudaStream_t st);
 
 size_t fold_smem_bytes(int nbins, int warps, int layout, int tile = kTile);
