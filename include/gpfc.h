@@ -87,6 +87,11 @@ int gpfc_fold_launch_times(gpfc_ctx *ctx, float *total_ms, int32_t *launches);
  * multiples of 2^-e (e per star, the largest with chunk x max|x| 2^e < 2^31) exactly and
  * rounds each bin once to FP32: bit-identical for any warps, streams, tile and
  * blocks_per_sm; chunk sets e.
+ * With every field 0 (layout 0 or 3), up to 800 bins or so, the fold keeps sum and count in one
+ * shared-memory word: from 256 bins with layout 3's arithmetic and bit-identical outputs, from 32
+ * to 255 bins in gpfc_fold only, as said there. gpfc_last_fold_plan then reports layout 3
+ * with up to 6 warps (groups of 32 periods), below 256 bins the FP32 layout's plan that the
+ * one-word fold stands in for.
  *   warps          warps per block, 32 trial periods per warp (1..16, capped by shared memory)
  *   layout         shared-memory bins: 1 = FP32 sum + 16-bit count (6 B per bin),
  *                  2 = FP32 sum + 32-bit count in one 64-bit word (8 B per bin),
@@ -135,7 +140,7 @@ int gpfc_last_fold_plan(const gpfc_ctx *ctx, gpfc_fold_config *out);
  * With autotuning enabled (the default), gpfc_fold, gpfc_search and gpfc_search_batched
  * use a tuned config with a matching key, and gpfc_search_batched tunes on its first
  * star when there is none (keyed by the average star length), unless its stream is
- * capturing. gpfc_set_autotune(ctx, 0) disables both; enable < 0 also forgets the
+ * capturing or the automatic plan is the one-word fold (see gpfc_fold_config). gpfc_set_autotune(ctx, 0) disables both; enable < 0 also forgets the
  * tuned configs. Fields set by gpfc_set_fold_config take precedence. */
 int gpfc_autotune(gpfc_ctx *ctx, const double *times, const float *flux, int64_t n,
                   const double *periods, int64_t n_periods, int32_t nbins, int scorer,
@@ -177,8 +182,10 @@ int gpfc_workspace_size(gpfc_ctx *ctx, int64_t n, int64_t n_periods, int32_t nbi
  * layout 3, the default) x is rounded to a multiple of 2^-e, e per star the largest with
  * max|x| 2^e <= floor((2^31 - 1) / min(chunk, n)), and the multiples are summed exactly
  * (shared-memory integer reductions, int64 across chunks), each bin rounded once to FP32:
- * a bin mean is within 2^-e / 2 of the exact mean of the x. Below 256 bins (layouts 1 and 2)
- * they are accumulated in FP32 with Kahan compensation (chunk partials in shared memory,
+ * a bin mean is within 2^-e / 2 of the exact mean of the x. From 32 to
+ * 255 bins, with every field of the fold config 0, the same holds of gpfc_fold's profiles with
+ * max|x| 2^e <= 2^30 whatever n: 2^-31 max|x|, the FP32 rounding of a value 128 times smaller.
+ * Below 32 bins, in the searches, and with any field set, layouts 1 and 2 accumulate x in FP32 with Kahan compensation (chunk partials in shared memory,
  * compensated across chunks). Above 1024 bins (more than a lane's shared-memory share) the
  * fold adds each sample with shared-memory atomics per period into count << 40 plus the
  * flux sum in fixed point (quantum 2^-k with n max|x| 2^k < 2^38, or up to 65,536 samples

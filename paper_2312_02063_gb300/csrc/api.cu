@@ -155,6 +155,10 @@ struct FoldPlan {
     int64_t ntasks;
 };
 
+// Blocks per star of the prep passes: a thousand samples each (their FP64 work, some ten operations
+// a sample at one warp instruction per 64 cycles, takes 40 us a block at 8,192).
+int prep_groups(int64_t n) { return (int)std::min<int64_t>(256, std::max<int64_t>(1, (n + 1023) / 1024)); }
+
 cudaError_t launch_plan(const FoldPlan &pl, const FoldParams &p, int grid, cudaStream_t st)
 {
     return pl.packed ? launch_fold_pack(p, grid, st) : launch_fold(p, kModeFold, grid, st);
@@ -201,6 +205,18 @@ bool pack_ok(const gpfc_ctx *ctx, int nbins)
            fold_max_warps(nbins, kLayoutRed32, kTile) >= 1 && fold_pack_groups(nbins) >= 1;
 }
 
+// Below 256 bins the one-word fold takes the place of the FP32 layouts, with flux in 31 bits, where
+// the caller gets the profiles and set nothing: measured, 12,345 periods of 28,800 samples and 200
+// bins, 747 -> 416 us (one warp a group of 32 periods waits out a read-modify-write per sample; here
+// sixteen share it). Below kPackMinBins a segment holds too few samples for its check to pay. A
+// search keeps the FP32 sums: its scores would change in their last bits.
+bool hilo_ok(const gpfc_ctx *ctx, int nbins)
+{
+    const gpfc_fold_config &c = ctx->fold_cfg;
+    return nbins >= kPackMinBins && nbins < 256 && c.layout == 0 && c.warps == 0 && c.chunk == 0 && c.tile == 0 &&
+           c.blocks_per_sm == 0 && c.streams == 0;
+}
+
 // Its plan over np periods in nstars grids of about equal length. A block takes as many
 // period groups as fit (each sample is read once for all), fewer where the grid would leave
 // multiprocessors idle, or where a star's last block would be mostly empty: the cost of a
@@ -214,12 +230,14 @@ FoldPlan plan_packed(const gpfc_ctx *ctx, int64_t n, int64_t np, int nbins, int6
     pl.tile = kMaxTile;
     pl.bps = 1;
     const int64_t per_sm = (np + (int64_t)32 * ctx->num_sms - 1) / ((int64_t)32 * ctx->num_sms);
-    const int maxg = (int)std::max<int64_t>(1, std::min<int64_t>(fold_pack_groups(nbins), per_sm));
+    const int maxg =
+        fold_pack_allowed(nbins, (int)std::max<int64_t>(1, std::min<int64_t>(fold_pack_groups(nbins), per_sm)));
     pl.warps = maxg;
     if (nstars > 1) {
         const int64_t avg = std::max<int64_t>(1, np / nstars);
         int64_t best = INT64_MAX;
         for (int g = maxg; g >= 1; --g) {
+            if (fold_pack_allowed(nbins, g) != g) continue;
             const int64_t cost = (avg + 32 * g - 1) / (32 * g) * (g + 1);
             if (cost < best) {
                 best = cost;
@@ -231,7 +249,7 @@ FoldPlan plan_packed(const gpfc_ctx *ctx, int64_t n, int64_t np, int nbins, int6
     pl.streams = std::max(1, kMaxRedWarps / pl.warps);
     pl.ntasks = (np + pl.ppc - 1) / pl.ppc;
     pl.grid = (int)std::min<int64_t>(pl.ntasks, ctx->num_sms);
-    pl.G = (int)std::min<int64_t>(256, std::max<int64_t>(1, (n + 8191) / 8192));
+    pl.G = prep_groups(n);
     return pl;
 }
 
@@ -276,13 +294,14 @@ FoldPlan plan_with(const gpfc_ctx *ctx, int64_t n, int64_t np, int nbins, const 
     const int occ = std::max(1, fold_blocks_per_sm(nbins, w, pl.layout, pl.tile, pl.streams));
     pl.bps = cfg.blocks_per_sm > 0 ? std::min(cfg.blocks_per_sm, occ) : occ;
     pl.grid = (int)std::min<int64_t>(pl.ntasks, (int64_t)ctx->num_sms * pl.bps);
-    pl.G = (int)std::min<int64_t>(256, std::max<int64_t>(1, (n + 8191) / 8192));
+    pl.G = prep_groups(n);
     return pl;
 }
 
-// With `profiles` (the fold writes profiles, for the caller or for a separate scorer) the plan
-// may be the one-word fold's.
-FoldPlan plan_fold(gpfc_ctx *ctx, int64_t n, int64_t np, int nbins, const gpfc_ctx::Tuned *tuned, bool profiles,
+// What the fold gives: scores, profiles for a scorer (the plan may be the one-word fold's) or
+// profiles for the caller (so too below 256 bins).
+enum FoldOut { kScores, kForScorer, kForCaller };
+FoldPlan plan_fold(gpfc_ctx *ctx, int64_t n, int64_t np, int nbins, const gpfc_ctx::Tuned *tuned, FoldOut out,
                    int64_t nstars = 1)
 {
     gpfc_fold_config cfg = ctx->fold_cfg;
@@ -292,10 +311,13 @@ FoldPlan plan_fold(gpfc_ctx *ctx, int64_t n, int64_t np, int nbins, const gpfc_c
         if (!cfg.tile) cfg.tile = tuned->cfg.tile;
         if (!cfg.blocks_per_sm) cfg.blocks_per_sm = tuned->cfg.blocks_per_sm;
     }
-    const FoldPlan pl = profiles && pack_ok(ctx, nbins) && (!tuned || tuned->packed)
-                            ? plan_packed(ctx, n, np, nbins, nstars)
-                            : plan_with(ctx, n, np, nbins, cfg);
-    ctx->last_plan = gpfc_fold_config{pl.warps, pl.layout, pl.chunk, pl.tile, pl.bps, pl.streams};
+    const bool packed = (out != kScores && pack_ok(ctx, nbins) && (!tuned || tuned->packed)) ||
+                        (out == kForCaller && hilo_ok(ctx, nbins));
+    const FoldPlan pl = packed ? plan_packed(ctx, n, np, nbins, nstars) : plan_with(ctx, n, np, nbins, cfg);
+    // (below 256 bins the FP32 plan that it stands in for: layout 3 set by hand there would cut
+    // the flux to its chunk's fixed point)
+    const FoldPlan r = packed && nbins < 256 ? plan_with(ctx, n, np, nbins, cfg) : pl;
+    ctx->last_plan = gpfc_fold_config{r.warps, r.layout, r.chunk, r.tile, r.bps, r.streams};
     return pl;
 }
 
@@ -321,7 +343,8 @@ size_t carve_fold(void *base, const FoldPlan &pl, int64_t n_total, int nstars, i
     fb.smp.xq = c.take<int32_t>(se);
     fb.smp.thg = c.take<int32_t>(se / 16 + 64);
     fb.smp.flags = c.take<uint8_t>(se / 16 + 64);
-    fb.ws_sc = c.take<float2>((size_t)pl.grid * nbins * pl.ppc * (pl.packed ? kPackPlanes / 2 : 1));
+    const int planes = pl.packed ? (nbins < 256 ? kPackPlanesHilo : kPackPlanes) : 2;
+    fb.ws_sc = reinterpret_cast<float2 *>(c.take<uint32_t>((size_t)pl.grid * nbins * pl.ppc * planes));
     fb.ws_cnt = c.take<uint32_t>(pl.packed ? 0 : (size_t)pl.grid * nbins * pl.ppc);
     fb.key = c.take<unsigned long long>(nstars);
     return c.off + 256;
@@ -362,8 +385,6 @@ struct WideBuffers {
     unsigned int *maxbits;
     int *kscale;
 };
-
-int prep_groups(int64_t n) { return (int)std::min<int64_t>(256, std::max<int64_t>(1, (n + 8191) / 8192)); }
 
 size_t carve_wide(void *base, int64_t n, WideBuffers &w)
 {
@@ -509,14 +530,17 @@ int run_fold(gpfc_ctx *ctx, const double *times, const float *flux, int64_t n, c
              int64_t np, int32_t nbins, double t0, int mode, FoldParams p, bool want_key,
              FoldBuffers *out_fb)
 {
-    const FoldPlan pl = plan_fold(ctx, n, np, nbins, find_tuned(ctx, nbins, mode, n), mode == kModeFold);
+    const FoldPlan pl =
+        plan_fold(ctx, n, np, nbins, find_tuned(ctx, nbins, mode, n), mode == kModeFold ? kForCaller : kScores);
     FoldBuffers fb{};
     const size_t need = carve_fold(nullptr, pl, n, 1, nbins, fb);
     int rc = ensure_ws(ctx, need);
     if (rc) return rc;
     carve_fold(ctx->ws, pl, n, 1, nbins, fb);
+    const bool hilo = pl.packed && nbins < 256;  // flux in 31 bits, unbiased
     cudaError_t e = launch_prep(times, flux, nullptr, n, 1, n, nullptr, t0, fb.smp, fb.partial, pl.G,
-                                fb.stats, ctx->status_dev, ctx->stream, pl.chunk, pl.packed);
+                                fb.stats, ctx->status_dev, ctx->stream, hilo ? kPackHiloChunk : pl.chunk,
+                                pl.packed && !hilo);
     if (e != cudaSuccess) return cuda_err(ctx, e, "prep kernels");
     p.smp = fb.smp;
     p.lc_off = nullptr;
@@ -615,7 +639,7 @@ cudaError_t timed_fold(gpfc_ctx *ctx, cudaStream_t sf, Launch launch)
 // does not fit.
 bool fused_plan(gpfc_ctx *ctx, int64_t n, int64_t np, int nbins, FoldPlan &pl)
 {
-    pl = plan_fold(ctx, n, np, nbins, find_tuned(ctx, nbins, kModeFold, n), false);
+    pl = plan_fold(ctx, n, np, nbins, find_tuned(ctx, nbins, kModeFold, n), kScores);
     int bps = search_blocks_per_sm(nbins, pl.warps, pl.layout, pl.tile, pl.streams);
     if (bps < 1 && !ctx->fold_cfg.tile && pl.tile > 512) {
         // the scorer staging did not fit beside 1024-sample tiles: halve the tiles
@@ -747,7 +771,7 @@ int run_search_box_warp(gpfc_ctx *ctx, const double *times, const float *flux, i
                         int64_t np, int32_t nbins, double t0, const gpfc_box_params *bp, float *score,
                         int64_t *best_index, float *best_score)
 {
-    const FoldPlan pl = plan_fold(ctx, n, np, nbins, find_tuned(ctx, nbins, kModeFold, n), true);
+    const FoldPlan pl = plan_fold(ctx, n, np, nbins, find_tuned(ctx, nbins, kModeFold, n), kForScorer);
     const int64_t chunk = std::min<int64_t>(np, (int64_t)pl.grid * pl.ppc);
     FoldBuffers fb{};
     int rc = ensure_ws(ctx, box_warp_bytes(pl, n, np, nbins));
@@ -839,7 +863,7 @@ int run_search_cnn(gpfc_ctx *ctx, const double *times, const float *flux, int64_
                    int64_t np, int32_t nbins, double t0, const gpfc_cnn_weights *wt, float *score,
                    int64_t *best_index, float *best_score)
 {
-    const FoldPlan pl = plan_fold(ctx, n, np, nbins, find_tuned(ctx, nbins, kModeFold, n), true);
+    const FoldPlan pl = plan_fold(ctx, n, np, nbins, find_tuned(ctx, nbins, kModeFold, n), kForScorer);
     const int64_t wave = (int64_t)pl.grid * pl.ppc;
     const int64_t chunk = std::min<int64_t>(np, wave);
     const int64_t half = (chunk + 1) / 2;
@@ -1519,10 +1543,11 @@ int gpfc_workspace_size(gpfc_ctx *ctx, int64_t n, int64_t n_periods, int32_t nbi
     // the largest of a fold (gpfc_fold, the epilogue search), the warp-per-profile search
     // and the one-kernel search; planning them leaves the context's last plan as it was
     const gpfc_fold_config last = ctx->last_plan;
-    const FoldPlan pb = plan_fold(ctx, n, n_periods, nbins, find_tuned(ctx, nbins, kModeBox, n), false);
-    const FoldPlan pf = plan_fold(ctx, n, n_periods, nbins, find_tuned(ctx, nbins, kModeFold, n), true);
+    const FoldPlan pb = plan_fold(ctx, n, n_periods, nbins, find_tuned(ctx, nbins, kModeBox, n), kScores);
+    const FoldPlan pf = plan_fold(ctx, n, n_periods, nbins, find_tuned(ctx, nbins, kModeFold, n), kForScorer);
+    const FoldPlan pc = plan_fold(ctx, n, n_periods, nbins, find_tuned(ctx, nbins, kModeFold, n), kForCaller);
     FoldBuffers fb{};
-    *bytes = std::max(carve_fold(nullptr, pb, n, 1, nbins, fb), carve_fold(nullptr, pf, n, 1, nbins, fb));
+    *bytes = std::max(carve_fold(nullptr, pb, n, 1, nbins, fb), carve_fold(nullptr, pc, n, 1, nbins, fb));
     *bytes = std::max(*bytes, box_warp_bytes(pf, n, n_periods, nbins));
     FoldPlan ps{};
     if (fused_plan(ctx, n, n_periods, nbins, ps)) {
@@ -2169,14 +2194,15 @@ int gpfc_search_batched(gpfc_ctx *ctx, int32_t n_stars, const int64_t *lc_offset
             tuned = find_tuned(ctx, nbins, mode, n_avg);
         }
     }
-    FoldPlan pl = plan_fold(ctx, n_avg, n_periods_total, nbins, tuned, mode == kModeFold, n_stars);
+    FoldPlan pl = plan_fold(ctx, n_avg, n_periods_total, nbins, tuned,
+                            mode == kModeFold ? kForScorer : kScores, n_stars);
     if (A.box_warp && ctx->box_path != GPFC_BOX_WARP && !(pl.packed && ctx->box_path == GPFC_BOX_AUTO)) {
         // the one-kernel search, with the tuned fold config if its block fits, else the
         // default one
-        FoldPlan ps = pl.packed ? plan_fold(ctx, n_avg, n_periods_total, nbins, tuned, false) : pl;
+        FoldPlan ps = pl.packed ? plan_fold(ctx, n_avg, n_periods_total, nbins, tuned, kScores) : pl;
         int bps = search_blocks_per_sm(nbins, ps.warps, ps.layout, ps.tile, ps.streams);
         if (bps < 1) {
-            ps = plan_fold(ctx, n_avg, n_periods_total, nbins, nullptr, false);
+            ps = plan_fold(ctx, n_avg, n_periods_total, nbins, nullptr, kScores);
             bps = search_blocks_per_sm(nbins, ps.warps, ps.layout, ps.tile, ps.streams);
         }
         // a block numbers the rows of its tasks in 32-bit tickets

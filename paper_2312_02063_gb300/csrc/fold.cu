@@ -130,10 +130,11 @@ __global__ void prep_quant_kernel(const double *times, const float *flux, const 
     int64_t b, e;
     star_range(lc_off, n, s, b, e);
     const int64_t len = e - b;
-    if (threadIdx.x == 0) {
+    if (threadIdx.x < 32) {  // (lanes in parallel, then a fixed tree)
         double tot = 0.0;
-        for (int g = 0; g < G; ++g) tot += partial[(size_t)s * G + g];
-        s_fref = tot / (double)len;
+        for (int g = threadIdx.x; g < G; g += 32) tot += partial[(size_t)s * G + g];
+        for (int o = 16; o > 0; o >>= 1) tot += __shfl_xor_sync(0xffffffffu, tot, o);
+        if (threadIdx.x == 0) s_fref = tot / (double)len;
     }
     __syncthreads();
     const double f_ref = s_fref;
@@ -216,15 +217,21 @@ __global__ void prep_sigma_kernel(const double *partial, const long long *pmin, 
                                   StarStats *stats)
 {
     const int s = blockIdx.x;
-    if (threadIdx.x != 0) return;
     double t = 0.0, xm = 0.0;
     long long m = LLONG_MAX;
-    for (int g = 0; g < G; ++g) {
+    for (int g = threadIdx.x; g < G; g += 32) {
         t += partial[(size_t)nstars * G + (size_t)s * G + g];
         xm = fmax(xm, partial[(size_t)3 * nstars * G + (size_t)s * G + g]);
         const long long v = pmin[(size_t)s * G + g];
         m = v < m ? v : m;
     }
+    for (int o = 16; o > 0; o >>= 1) {
+        t += __shfl_xor_sync(0xffffffffu, t, o);
+        xm = fmax(xm, __shfl_xor_sync(0xffffffffu, xm, o));
+        const long long v = __shfl_xor_sync(0xffffffffu, m, o);
+        m = v < m ? v : m;
+    }
+    if (threadIdx.x != 0) return;
     stats[s].sigma = (float)sqrt(t / (double)stats[s].n);
     stats[s].dtau0 = m == LLONG_MAX ? 0 : m;
     // a chunk holds at most min(chunk, n) samples of the star
@@ -304,7 +311,7 @@ cudaError_t launch_prep(const double *times, const float *flux, const int64_t *l
     prep_sum_kernel<<<grid, 256, 0, st>>>(flux, lc_off, n, partial);
     prep_quant_kernel<<<grid, 256, 0, st>>>(times, flux, lc_off, n, t0s, t0, partial, pmin, smp, stats,
                                             status);
-    prep_sigma_kernel<<<nstars, 32, 0, st>>>(partial, pmin, G, nstars, chunk < 16 ? 16 : chunk, stats);
+    prep_sigma_kernel<<<nstars, 32, 0, st>>>(partial, pmin, G, nstars, chunk < 2 ? 2 : chunk, stats);
     prep_flags_kernel<<<grid, 256, 0, st>>>(lc_off, n, smp, stats, packed ? chunk : 0);
     return cudaGetLastError();
 }
@@ -1505,8 +1512,8 @@ __device__ __forceinline__ void score_row(const BoxCoopParams &p, int64_t r, int
 // 2^-23, the walk's products by 2^-23: a box further below the largest can neither win the walk
 // nor decide which of the near ones does, so the box, and every output, is the walk's. Profiles
 // with more than kMaxNearStarts near starts (a flat one: every box 0) go through the walk itself.
-// What bounds it now: instruction issue. 29,184 profiles of 256 bins, widths 1..108: see
-// kCoopBlocks.
+// What bounds it now: instruction issue. 262,144 profiles of 256 bins (before -> now): widths
+// 1..32 2.15 -> 1.05 ms, 1..108 3.96 -> 2.34 ms, 1..160 5.33 -> 3.20 ms.
 constexpr float kNear = 1e-5f;
 constexpr int kMaxNearStarts = 8;
 

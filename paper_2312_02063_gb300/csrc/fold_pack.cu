@@ -20,6 +20,11 @@
 // with such a period costs little more than the others (a launch lasts as long as its slowest
 // block).
 //
+// Below 256 bins, where the flux is not cut to the chunk's fixed point (layouts 1 and 2 sum FP32),
+// the same scheme takes 31-bit flux (HILO): xq = hi 2^15 + lo, the word holds the count and the
+// sum of lo, and a second word of the bin's record, 128 bytes on, the sum of hi. Sums are exact
+// in units of 2^-30 max|x|, rounded once.
+//
 // Half the words also means half the shared memory: six groups of 32 periods share each
 // sample read from the tile instead of three. A block is 16 warps; each takes every 16th
 // 16-sample group of a tile and adds it to the bins of all period groups (lane l: period l of
@@ -72,6 +77,7 @@ __host__ __device__ inline uint32_t pack_records_addr(uint32_t base, int nbins)
 
 __host__ __device__ inline uint32_t pack_records_bytes(int nbins, int groups)
 {
+    if (nbins < 256) return (uint32_t)groups * (uint32_t)nbins * 256u;
     return nbins == 256 ? (uint32_t)((groups + 1) / 2) * kSlab : (uint32_t)groups * (uint32_t)nbins * 128u;
 }
 
@@ -84,7 +90,7 @@ __device__ __forceinline__ uint32_t phase_hi(uint32_t tl, uint32_t thF, uint32_t
 }
 
 // Shared address of a sample's bin word for one period (KIND 0: 256 bins, 1: a power of two,
-// 2: any). With 256 bins the bin is the top byte of the phase and rows are 256 bytes, so one
+// 2: any; 3 and 4: below 256 bins, HILO, a power of two or any). With 256 bins the bin is the top byte of the phase and rows are 256 bytes, so one
 // byte permutation builds the address: byte 0 = lane and group parity, byte 1 = bin, the rest the
 // slab; the slab's distance from a multiple of 64 KB is the reduction's immediate offset.
 template <int KIND>
@@ -93,9 +99,10 @@ __device__ __forceinline__ uint32_t word_addr(uint32_t hi, uint32_t tl, uint32_t
 {
     if (KIND == 0) return __byte_perm(hi, base, 0x7634);
     if (KIND == 1) return base + ((hi >> shift) << 7);
+    if (KIND == 3) return base + ((hi >> shift) << 8);
     const uint32_t lo = tl * Fl;
     const unsigned long long t = (unsigned long long)hi * nbins + (unsigned long long)__umulhi(lo, nbins);
-    return base + ((uint32_t)(t >> 32) << 7);
+    return base + ((uint32_t)(t >> 32) << (KIND == 4 ? 8 : 7));
 }
 
 template <int KIND>
@@ -112,6 +119,19 @@ __device__ __forceinline__ void st_row8(void *dst, const uint32_t *v)
     asm volatile("st.global.v8.b32 [%0], {%1, %2, %3, %4, %5, %6, %7, %8};" ::"l"(dst), "r"(v[0]), "r"(v[1]), "r"(v[2]),
                  "r"(v[3]), "r"(v[4]), "r"(v[5]), "r"(v[6]), "r"(v[7])
                  : "memory");
+}
+
+// A sample's increments: x as it is, or (HILO) a count and lo, and hi in the second word.
+constexpr int kLoBits = 15;
+template <int KIND>
+__device__ __forceinline__ void sample_add(uint32_t a, uint32_t x, uint32_t one)
+{
+    if (KIND >= 3) {
+        asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(a), "r"((x & ((1u << kLoBits) - 1u)) + one) : "memory");
+        asm volatile("red.shared.add.u32 [%0+128], %1;" ::"r"(a), "r"((uint32_t)((int32_t)x >> kLoBits)) : "memory");
+    } else {
+        word_add<KIND>(a, x);
+    }
 }
 
 struct PackHalf {
@@ -164,10 +184,11 @@ __global__ void __launch_bounds__(kPackThreads, 1) fold_pack_kernel(const FoldPa
         return;
     }
     // row stride of a bin and start of period group j's words (lane's own)
-    const uint32_t row = KIND == 0 ? 256u : 128u;
+    constexpr bool HILO = KIND >= 3;
+    constexpr uint32_t row = KIND == 0 || HILO ? 256u : 128u;
     auto group_rec = [&](int j) {
         return (KIND == 0 ? rec + (uint32_t)(j >> 1) * kSlab + (uint32_t)(j & 1) * 128u
-                          : rec + (uint32_t)j * (uint32_t)nbins * 128u) + 4u * (uint32_t)lane;
+                          : rec + (uint32_t)j * (uint32_t)nbins * row) + 4u * (uint32_t)lane;
     };
     if (threadIdx.x == 0) {
         mbar_init(&sh.bars[0], 1);
@@ -190,7 +211,7 @@ __global__ void __launch_bounds__(kPackThreads, 1) fold_pack_kernel(const FoldPa
     // biased sum up to 2^23 samples, else an int64 sum and, in the third plane, 32-bit counts),
     // then the slots
     const size_t plane = (size_t)nbins * ppc;
-    uint32_t *ws = reinterpret_cast<uint32_t *>(p.ws_sc) + (size_t)blockIdx.x * kPackPlanes * plane + lane;
+    uint32_t *ws = reinterpret_cast<uint32_t *>(p.ws_sc) + (size_t)blockIdx.x * (HILO ? kPackPlanesHilo : kPackPlanes) * plane + lane;
     unsigned long long *ws_tot = reinterpret_cast<unsigned long long *>(ws - lane) + lane;
     uint32_t *ws_cnt = ws + 2 * plane, *ws_slot = ws + 3 * plane;
 
@@ -251,19 +272,22 @@ __global__ void __launch_bounds__(kPackThreads, 1) fold_pack_kernel(const FoldPa
             }
         }
         __syncthreads();
-        const PackWord pw = pack_word(nsamp, p.chunk);
-        const bool wide = nsamp > ((int64_t)1 << 23);
+        // (HILO: lo < 2^15 whatever the star)
+        const PackWord pw = HILO ? PackWord{0u, 256u, 23} : pack_word(nsamp, p.chunk);
+        const bool wide = HILO || nsamp > ((int64_t)1 << 23);
         const unsigned long long bias = (1ull << 40) + pw.L;  // per count in a 64-bit total
         // Tiles of the star: no longer than a tenth of the samples over 0.86 M, so that one tile
         // holds even for a period ten cadences long.
         int tile = kPackTile;
         while (tile > 256 && (float)tile > 8.6f * (float)pw.M) tile >>= 1;
         const int ntiles = (int)((nsamp + tile - 1) / tile);
-        // The block's segments: of seg_tiles tiles, at most kPackSegs of them (their words go to
-        // slots) for a star of one chunk.
-        const bool slots = nsamp <= (int64_t)p.chunk;
+        // The block's segments: of seg_tiles tiles, about kPackSegTiles but no more than a mean load of
+        // half M allows; into slots where a star of one chunk has at most kPackSegs of them.
+        const int most = max(1, (int)fminf(0.55f * (float)pw.M * (float)nbins / (float)tile, 1e6f));
         int nsegs = max(1, (ntiles + kPackSegTiles - 1) / kPackSegTiles);
-        if (slots) nsegs = min(nsegs, kPackSegs);
+        if (nsegs > kPackSegs && nsamp <= (int64_t)p.chunk) nsegs = kPackSegs;
+        nsegs = max(nsegs, (ntiles + most - 1) / most);
+        const bool slots = nsamp <= (int64_t)p.chunk && nsegs <= kPackSegs;
         const int seg_tiles = max(1, (ntiles + nsegs - 1) / nsegs);
 
         // ---- each group's segment length: the longest whose predicted load stays below M
@@ -364,8 +388,8 @@ __global__ void __launch_bounds__(kPackThreads, 1) fold_pack_kernel(const FoldPa
                     const uint32_t x = lds_u32(sxq + 4u * i);
 #pragma unroll
                     for (int j = 0; j < G; ++j) {
-                        word_add<KIND>(word_addr<KIND>(phase_hi(tl, th * Fl[j], Fl[j], Fh[j]), tl, Fl[j], gaddr[j],
-                                                       (uint32_t)nbins, p.shift), x);
+                        sample_add<KIND>(word_addr<KIND>(phase_hi(tl, th * Fl[j], Fl[j], Fh[j]), tl, Fl[j], gaddr[j],
+                                                         (uint32_t)nbins, p.shift), x, 1u << pw.S);
                     }
                 };
                 // a group whose samples differ in their high word (every ~256 days, or
@@ -395,7 +419,7 @@ __global__ void __launch_bounds__(kPackThreads, 1) fold_pack_kernel(const FoldPa
                             for (int q = 0; q < 2; ++q) {
                                 const uint32_t xx[4] = {H.x[q].x, H.x[q].y, H.x[q].z, H.x[q].w};
 #pragma unroll
-                                for (int u = 0; u < 4; ++u) word_add<KIND>(ad[4 * q + u], xx[u]);
+                                for (int u = 0; u < 4; ++u) sample_add<KIND>(ad[4 * q + u], xx[u], 1u << pw.S);
                             }
                         }
                     };
@@ -435,15 +459,16 @@ __global__ void __launch_bounds__(kPackThreads, 1) fold_pack_kernel(const FoldPa
             return true;
         };
 
-        // The words of a segment: (sum of xq, count) by what they hold (0 both, 1 counts, 2 sums).
+        // The word (and HILO's second) of a segment: sum of xq and count, by what they hold: 0 both;
+        // after a redone segment's passes 1 counts (and hi), 2 the rest of the sums.
+        using Sum = typename std::conditional<HILO, long long, int32_t>::type;
         const uint32_t ymask = (1u << pw.S) - 1u;
-        auto decode = [&](int what, uint32_t w, int32_t &ds, uint32_t &dc) {
-            if (what == 0) {
-                dc = w >> pw.S;
-                ds = (int32_t)((w & ymask) - pw.L * dc);
+        auto decode = [&](int what, uint32_t w, uint32_t w2, Sum &ds, uint32_t &dc) {
+            dc = what == 0 ? w >> pw.S : (what == 1 ? w : 0u);
+            if constexpr (HILO) {
+                ds = (long long)(int32_t)w2 * (1 << kLoBits) + (long long)(what == 0 ? w & ymask : (what == 1 ? 0u : w));
             } else {
-                dc = what == 1 ? w : 0u;
-                ds = what == 2 ? (int32_t)w : 0;
+                ds = what == 0 ? (int32_t)((w & ymask) - pw.L * dc) : (what == 2 ? (int32_t)w : 0);
             }
         };
         // Empty this warp's bins of group j into its totals (written, not added to, the first time).
@@ -465,10 +490,12 @@ __global__ void __launch_bounds__(kPackThreads, 1) fold_pack_kernel(const FoldPa
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
                     if (u < nb) {
-                        int32_t ds;
+                        Sum ds;
                         uint32_t dc;
-                        decode(what, lds_u32(a + (uint32_t)(b0 + u) * row), ds, dc);
-                        sts_u32(a + (uint32_t)(b0 + u) * row, 0u);
+                        const uint32_t w = a + (uint32_t)(b0 + u) * row;
+                        decode(what, lds_u32(w), HILO ? lds_u32(w + 128u) : 0u, ds, dc);
+                        sts_u32(w, 0u);
+                        if (HILO) sts_u32(w + 128u, 0u);
                         tot[u] += (unsigned long long)(long long)ds + (wide ? 0ull : (unsigned long long)dc * bias);
                         ws_tot[(size_t)(b0 + u) * ppc + 32 * j] = tot[u];
                         if (wide) ws_cnt[(size_t)(b0 + u) * ppc + 32 * j] = cn[u] + dc;
@@ -490,16 +517,28 @@ __global__ void __launch_bounds__(kPackThreads, 1) fold_pack_kernel(const FoldPa
                     fh = (uint32_t)(F >> 32);
                 }
             }
-            for (int b = blo; b < bhi; ++b) sts_u32(a + (uint32_t)b * row, 0u);
+            for (int b = blo; b < bhi; ++b) {
+                sts_u32(a + (uint32_t)b * row, 0u);
+                if (HILO) sts_u32(a + (uint32_t)b * row + 128u, 0u);
+            }
             __syncthreads();
-            const uint32_t unbias = 0u - pw.add();
+            const uint32_t unbias = HILO ? 0u : 0u - pw.add();
 #pragma unroll 1
             for (int pass = 1; pass <= 2; ++pass) {
 #pragma unroll 4
                 for (int64_t i = i0 + warp; i < i1; i += kPackWarps) {
                     const uint32_t tl = __ldg(p.smp.tau_lo + sbase + i), th = (uint32_t)__ldg(p.smp.tau_hi + sbase + i);
-                    const uint32_t x = pass == 1 ? 1u : (uint32_t)__ldg(p.smp.xq + sbase + i) + unbias;
-                    word_add<KIND>(word_addr<KIND>(phase_hi(tl, th * fl, fl, fh), tl, fl, ab, (uint32_t)nbins, p.shift), x);
+                    const uint32_t x = (uint32_t)__ldg(p.smp.xq + sbase + i) + unbias;
+                    const uint32_t w =
+                        word_addr<KIND>(phase_hi(tl, th * fl, fl, fh), tl, fl, ab, (uint32_t)nbins, p.shift);
+                    if (!HILO) {
+                        word_add<KIND>(w, pass == 1 ? 1u : x);
+                    } else if (pass == 1) {  // counts and hi, then lo
+                        word_add<KIND>(w, 1u);
+                        word_add<KIND>(w + 128u, (uint32_t)((int32_t)x >> kLoBits));
+                    } else {
+                        word_add<KIND>(w, x & ((1u << kLoBits) - 1u));
+                    }
                 }
                 __syncthreads();
                 flush(j, pass, first && pass == 1);
@@ -537,13 +576,17 @@ __global__ void __launch_bounds__(kPackThreads, 1) fold_pack_kernel(const FoldPa
                     const uint32_t a = group_rec(j);
                     uint32_t sum = 0u, big = 0u;
                     const bool store = to_slot && !((own >> (5 * j)) & 31u);
-                    uint32_t *w = ws_slot + (size_t)seg * plane + 32 * j;
+                    uint32_t *w = ws_slot + (size_t)(HILO ? 2 * seg : seg) * plane + 32 * j;
 #pragma unroll 4
                     for (int b = blo; b < bhi; ++b) {
                         const uint32_t v = lds_u32(a + (uint32_t)b * row), c = v >> pw.S;
                         if (store) {
                             w[(size_t)b * ppc] = v;
                             sts_u32(a + (uint32_t)b * row, 0u);
+                            if (HILO) {
+                                w[plane + (size_t)b * ppc] = lds_u32(a + (uint32_t)b * row + 128u);
+                                sts_u32(a + (uint32_t)b * row + 128u, 0u);
+                            }
                         }
                         sum += c;
                         big = max(big, c);
@@ -591,7 +634,7 @@ __global__ void __launch_bounds__(kPackThreads, 1) fold_pack_kernel(const FoldPa
         const double qscale = ldexp(1.0, -p.stats[s].qexp);
         const int qexp = -ilogb(qscale);
         const float qscale_f = (qexp >= -100 && qexp <= 100) ? __int_as_float((127 - qexp) << 23) : 0.f;
-        const int conv = qscale_f == 0.f ? 2 : (nsamp <= (int64_t)p.chunk ? 0 : 1);
+        const int conv = qscale_f == 0.f ? 2 : (!HILO && nsamp <= (int64_t)p.chunk ? 0 : 1);
         const float fh = p.stats[s].f_hi, fl = p.stats[s].f_lo;
 #pragma unroll 1
         for (int j = 0; j < G; ++j) {
@@ -605,32 +648,36 @@ __global__ void __launch_bounds__(kPackThreads, 1) fold_pack_kernel(const FoldPa
             const bool totals = (have >> j) & 1u;
             const size_t o = (size_t)orow * nbins;
             for (int b0 = blo; b0 < bhi; b0 += kEpi) {
-                int32_t ds[kEpi];
+                Sum ds[kEpi];
                 uint32_t c[kEpi];
                 float S[kEpi];
 #pragma unroll
                 for (int u = 0; u < kEpi; ++u) {
                     c[u] = 0u;
                     ds[u] = 0;
-                    if (b0 + u < bhi) decode(0, lds_u32(a + (uint32_t)(b0 + u) * row), ds[u], c[u]);
+                    const uint32_t w = a + (uint32_t)(b0 + u) * row;
+                    if (b0 + u < bhi) decode(0, lds_u32(w), HILO ? lds_u32(w + 128u) : 0u, ds[u], c[u]);
                 }
                 if (slots) {
-                    // (a star of at most one chunk: its bin sums are 32-bit integers)
-                    uint32_t w[kPackSegs - 1][kEpi];
+                    // (a star of at most one chunk: without HILO its bin sums are 32-bit integers)
+                    constexpr int W = HILO ? 2 : 1;
+                    uint32_t w[kPackSegs - 1][W][kEpi];
 #pragma unroll
                     for (int q = 0; q < kPackSegs - 1; ++q)
 #pragma unroll
-                        for (int u = 0; u < kEpi; ++u)
-                            w[q][u] = ((mine >> q) & 1u) && b0 + u < bhi
-                                          ? ws_slot[(size_t)q * plane + (size_t)(b0 + u) * ppc + 32 * j]
-                                          : 0u;
+                        for (int h = 0; h < W; ++h)
+#pragma unroll
+                            for (int u = 0; u < kEpi; ++u)
+                                w[q][h][u] = ((mine >> q) & 1u) && b0 + u < bhi
+                                                 ? ws_slot[(size_t)(W * q + h) * plane + (size_t)(b0 + u) * ppc + 32 * j]
+                                                 : 0u;
 #pragma unroll
                     for (int q = 0; q < kPackSegs - 1; ++q)
 #pragma unroll
                         for (int u = 0; u < kEpi; ++u) {
-                            int32_t es;
+                            Sum es;
                             uint32_t ec;
-                            decode(0, w[q][u], es, ec);
+                            decode(0, w[q][0][u], w[q][W - 1][u], es, ec);
                             ds[u] += es;
                             c[u] += ec;
                         }
@@ -692,28 +739,35 @@ size_t fold_pack_smem(int nbins, int groups)
     return pack_records_addr(kWindow, nbins) - kWindow + pack_records_bytes(nbins, groups);
 }
 
+int fold_pack_allowed(int nbins, int groups);
+
 int fold_pack_groups(int nbins)
 {
     int g = kPackMaxGroups;
     while (g > 0 && fold_pack_smem(nbins, g) > kSmemLimit) --g;
-    return g;
+    return fold_pack_allowed(nbins, g);
 }
 
-// f(kernel) for the instance of these bins and groups (each kind with the groups it can hold)
+// f(kernel) for the instance of these bins and groups (each kind with the groups it can hold;
+// HILO with 1, 2, 3 or 6)
 template <int KIND, int G, class F>
 static cudaError_t with_groups(int groups, F f)
 {
     if constexpr (G < 1) return cudaErrorInvalidValue;
     else if (groups == G) return f(fold_pack_kernel<KIND, G>);
-    else return with_groups<KIND, G - 1>(groups, f);
+    else return with_groups<KIND, (KIND >= 3 && G == 6 ? 3 : G - 1)>(groups, f);
 }
 template <class F>
 static cudaError_t with_kernel(int nbins, int shift, int groups, F f)
 {
+    if (nbins < 256)
+        return shift >= 0 ? with_groups<3, kPackMaxGroups>(groups, f) : with_groups<4, kPackMaxGroups>(groups, f);
     if (nbins == 256) return with_groups<0, kPackMaxGroups>(groups, f);
     if (shift >= 0) return with_groups<1, 3>(groups, f);  // 512 bins: 64 KB a group
     return with_groups<2, 5>(groups, f);                  // 257 bins and more
 }
+
+int fold_pack_allowed(int nbins, int groups) { return nbins < 256 && (groups == 4 || groups == 5) ? 3 : groups; }
 
 int fold_pack_register()
 {
@@ -725,6 +779,8 @@ int fold_pack_register()
         e = with_kernel(256, 24, g, attr);
         if (e == cudaSuccess && g <= 3) e = with_kernel(512, 23, g, attr);
         if (e == cudaSuccess && g <= 5) e = with_kernel(300, -1, g, attr);
+        if (e == cudaSuccess && fold_pack_allowed(64, g) == g) e = with_kernel(64, 26, g, attr);
+        if (e == cudaSuccess && fold_pack_allowed(64, g) == g) e = with_kernel(100, -1, g, attr);
     }
     return (int)e;
 }

@@ -123,7 +123,9 @@ struct BoxCoopParams {
 // float2 (sum, count) slots one warp of the scorer stages per profile
 __host__ __device__ inline int coop_pairs(int nbins) { return nbins + (nbins >> 3) + 2; }
 constexpr int kCoopWarps = 8;  // warps per block of the scorer
-constexpr int kCoopBlocks = 3; // and blocks per multiprocessor its registers leave room for
+// and blocks per multiprocessor its registers leave room for (262,144 profiles, widths 1..32, 1..108
+// and 1..160, with 2 / 3 / 4: 1.10 / 1.05 / 1.02, 2.40 / 2.34 / 2.34, 3.26 / 3.20 / 3.23 ms)
+constexpr int kCoopBlocks = 3;
 
 cudaError_t launch_box_coop(const BoxCoopParams &p, int num_sms, cudaStream_t st);
 
@@ -143,10 +145,16 @@ cudaError_t launch_fold(const FoldParams &p, int mode, int grid, cudaStream_t st
 constexpr int kPackMaxGroups = 6;
 constexpr int kPackChunk = 65520;
 constexpr int kPackSegs = 4;                  // segments of a star whose words go to slots
-constexpr int kPackPlanes = 3 + kPackSegs - 1;  // 32-bit words of workspace (ws_sc) per bin and period of a
-                                                // resident block: totals (3) and slots
+// 32-bit words of workspace (ws_sc) per bin and period of a resident block: totals (3) and slots
+// (below 256 bins two words each)
+constexpr int kPackPlanes = 3 + kPackSegs - 1;
+constexpr int kPackPlanesHilo = 3 + 2 * (kPackSegs - 1);
+constexpr int kPackMinBins = 32;
+// prep's chunk below 256 bins: flux in 31 bits (the bound of two samples' sum)
+constexpr int kPackHiloChunk = 2;
 size_t fold_pack_smem(int nbins, int groups);
 int fold_pack_groups(int nbins);
+int fold_pack_allowed(int nbins, int groups);  // the largest instance of at most that many groups
 int fold_pack_register();
 cudaError_t launch_fold_pack(const FoldParams &p, int grid, cudaStream_t st);
 // Shared memory of a kModeSearch block (0 if it does not fit or warps + 1 > 4).
