@@ -104,147 +104,174 @@ struct LoadH3 {  // B(k = profile, n = fd) from the fc1 operand tiles: high + lo
 
 struct LdDZ1T {  // dW(fc1): A(j, profile)
     const float *dZ1;
-    __device__ float operator()(int64_t j, int64_t k) const { return dZ1[k * 256 + j]; }
+    __device__ float operator()(uint32_t j, uint32_t k) const { return dZ1[(size_t)k * 256 + j]; }
 };
 struct LdH3T {  // dW(fc1): B(feature fd, profile) = h3 (high + low terms)
     const uint8_t *h3t;
-    __device__ float operator()(int64_t fd, int64_t k) const { return LoadH3{h3t}((int)k, (int)fd); }
+    __device__ float operator()(uint32_t fd, uint32_t k) const { return LoadH3{h3t}((int)k, (int)fd); }
 };
 struct LdDZ1 {  // dh3: A(profile, j)
     const float *dZ1;
-    __device__ float operator()(int64_t k, int64_t j) const { return dZ1[k * 256 + j]; }
+    __device__ float operator()(uint32_t k, uint32_t j) const { return dZ1[(size_t)k * 256 + j]; }
 };
 struct LdW1T {  // dh3: B(fd, j) = fc1.w[j][pt_feature(fd)]
     const float *w;
-    __device__ float operator()(int64_t fd, int64_t j) const { return w[j * 2048 + pt_feature((int)fd)]; }
+    __device__ float operator()(uint32_t fd, uint32_t j) const { return w[j * 2048 + pt_feature((int)fd)]; }
 };
 template <int COUT, int L>
 struct LdDa {  // conv weight gradient: A(co, (profile b, position l))
     const float *da;
-    __device__ float operator()(int64_t co, int64_t k) const { return da[((k / L) * COUT + co) * L + (k % L)]; }
+    __device__ float operator()(uint32_t co, uint32_t k) const { return da[((size_t)(k / L) * COUT + co) * L + (k % L)]; }
 };
 template <int CIN, int L>
 struct LdHim {  // conv weight gradient: B((ci, tap), (b, l)) = h[b][ci][(l + tap - 2) mod L]
     const uint16_t *h;
-    __device__ float operator()(int64_t n, int64_t k) const
+    __device__ float operator()(uint32_t n, uint32_t k) const
     {
         const int ci = (int)(n / 5), tap = (int)(n % 5), l = (int)(k % L);
-        return bf2f(h[((k / L) * CIN + ci) * L + ((l + tap - 2 + L) % L)]);
+        return bf2f(h[((size_t)(k / L) * CIN + ci) * L + ((l + tap - 2 + L) % L)]);
     }
 };
 template <int COUT, int L>
 struct LdDaShift {  // conv input gradient: A((b, m), (co, tap)) = da[b][co][(m - tap + 2) mod L]
     const float *da;
-    __device__ float operator()(int64_t r, int64_t k) const
+    __device__ float operator()(uint32_t r, uint32_t k) const
     {
         const int m = (int)(r % L), co = (int)(k / 5), tap = (int)(k % 5);
-        return da[((r / L) * COUT + co) * L + ((m - tap + 2 + L) % L)];
+        return da[((size_t)(r / L) * COUT + co) * L + ((m - tap + 2 + L) % L)];
     }
 };
 template <int CIN>
 struct LdWT {  // conv input gradient: B(ci, (co, tap)) = W[co][ci][tap]
     const float *W;
-    __device__ float operator()(int64_t ci, int64_t k) const { return W[((k / 5) * CIN + ci) * 5 + (k % 5)]; }
+    __device__ float operator()(uint32_t ci, uint32_t k) const { return W[((k / 5) * CIN + ci) * 5 + (k % 5)]; }
 };
 
 // ------------------------------------------------------------------ ReLU + max-pool backward
 
-// da[k][c][2l+s] = g[k][c][l] if element 2l+s was the (first) maximum of relu(a) over the
-// pair and a > 0 there; else 0. With FROM_H3, g is dh3 in the device feature order.
-template <int C, int L, bool FROM_H3>
-__global__ void poolrelu_bwd_kernel(const float *a, const float *g, float *da, int64_t B)
+// One profile at a time per block. da[k][c][2l+s] = g[k][l][c] if element 2l+s was the (first)
+// maximum of relu(a) over the pair and a > 0 there; else 0. g is a GEMM's result, position-major
+// (the device feature order for dh3): it goes through shared memory, a's and da's four positions
+// a thread straight. The bias gradient is summed on the way, in a thread's registers across the
+// block's profiles (its channels do not change), so da is not read again for it; and the first
+// layer's weight gradient
+//   dW[c][t] += sum_l da[c][l] x[(l + t - 2) mod L]
+// too (CONV1), whose da is then never stored. Partials per block: [C] or, CONV1, [C][5], [C].
+// Bound by memory: 4,096 profiles move 168 MB a layer (CONV1 105 MB).
+template <int C, int L, bool CONV1>
+__global__ void __launch_bounds__(256, 3) poolrelu_bwd_kernel(const float *a, const float *g, const float *x,
+                                                              float *da, int64_t B, float *part)
 {
-    const int64_t total = B * C * (L / 2);
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
-        const int lp = (int)(e % (L / 2));
-        const int64_t kc = e / (L / 2);
-        const int c = (int)(kc % C);
-        const int64_t k = kc / C;
-        const float u = a[(kc * L) + 2 * lp], v = a[(kc * L) + 2 * lp + 1];
-        const bool second = fmaxf(v, 0.f) > fmaxf(u, 0.f);
-        const float gg = FROM_H3 ? g[k * 2048 + lp * 64 + c] : g[kc * (L / 2) + lp];
-        da[kc * L + 2 * lp] = (!second && u > 0.f) ? gg : 0.f;
-        da[kc * L + 2 * lp + 1] = (second && v > 0.f) ? gg : 0.f;
-    }
-}
-
-// ------------------------------------------------------------------ conv backward
-
-// One profile at a time per block: weight-gradient partials (kept in registers across the
-// block's profiles) and, with DGRAD, the input gradient
-//   dW[co][ci][t] += sum_l da[co][l] h[ci][(l + t - 2) mod L],  db[co] += sum_l da[co][l]
-//   dh[ci][l] = sum_{co,t} da[co][(l - t + 2) mod L] W[co][ci][t]
-template <int CIN, int COUT, int L, bool DGRAD, bool XF32>
-__global__ void __launch_bounds__(256) conv_bwd_kernel(const float *da, const void *hin, const float *W,
-                                                       float *dh, float *part, int64_t B)
-{
-    constexpr int NW = COUT * CIN * 5;
-    constexpr int PER = (NW + 255) / 256;
-    extern __shared__ float sm[];
-    float *da_s = sm;                 // [COUT][L]
-    float *h_s = da_s + COUT * L;     // [CIN][L]
-    float *W_s = h_s + CIN * L;       // [COUT][CIN][5]
+    static_assert(C * L == 4096 && L % 4 == 0, "four float4 a thread");
+    constexpr int LP = L / 2, GS = C + 1;  // row stride in shared memory: no bank conflicts along l
+    constexpr int T = L / 4;               // threads of a channel
+    __shared__ float gs[LP * GS];
+    __shared__ float xs[CONV1 ? L : 1];
+    __shared__ float red[CONV1 ? 8 * 4 * 6 : 1];
     const int t = threadIdx.x;
-    if (DGRAD)
-        for (int i = t; i < NW; i += 256) W_s[i] = rbf(W[i]);
-    float acc[PER];
+    float accb[4] = {0.f, 0.f, 0.f, 0.f};
+    float accw[4][5];
 #pragma unroll
-    for (int i = 0; i < PER; ++i) acc[i] = 0.f;
-    float accb = 0.f;
+    for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int q = 0; q < 5; ++q) accw[i][q] = 0.f;
     for (int64_t k = blockIdx.x; k < B; k += gridDim.x) {
-        __syncthreads();
-        for (int i = t; i < COUT * L; i += 256) da_s[i] = da[(size_t)k * COUT * L + i];
-        for (int i = t; i < CIN * L; i += 256) {
-            if (XF32) h_s[i] = static_cast<const float *>(hin)[(size_t)k * CIN * L + i];
-            else h_s[i] = bf2f(static_cast<const uint16_t *>(hin)[(size_t)k * CIN * L + i]);
+        const float4 *ak = reinterpret_cast<const float4 *>(a + k * 4096);
+        const float4 *gk = reinterpret_cast<const float4 *>(g + k * 2048);
+        float4 v[4], w[2];
+#pragma unroll
+        for (int i = 0; i < 2; ++i) w[i] = gk[t + 256 * i];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) v[i] = ak[t + 256 * i];
+        __syncthreads();  // the profile before has been read
+#pragma unroll
+        for (int i = 0; i < 2; ++i) {
+            const int e = 4 * (t + 256 * i), lp = e / C, c = e % C;
+            float *d = gs + lp * GS + c;
+            d[0] = w[i].x;
+            d[1] = w[i].y;
+            d[2] = w[i].z;
+            d[3] = w[i].w;
         }
+        if (CONV1) xs[t] = x[k * L + t];
         __syncthreads();
 #pragma unroll
-        for (int i = 0; i < PER; ++i) {
-            const int o = t + 256 * i;
-            if (o < NW) {
-                const int co = o / (CIN * 5), ci = (o / 5) % CIN, tap = o % 5;
-                const float *dr = da_s + co * L;
-                const float *hr = h_s + ci * L;
-                float s = 0.f;
-                for (int l = 0; l < L; ++l) s = fmaf(dr[l], hr[(l + tap - 2 + L) % L], s);
-                acc[i] += s;
-            }
-        }
-        if (t < COUT) {
-            float s = 0.f;
-            for (int l = 0; l < L; ++l) s += da_s[t * L + l];
-            accb += s;
-        }
-        if (DGRAD) {
-            for (int o = t; o < CIN * L; o += 256) {
-                const int ci = o / L, l = o % L;
-                float s = 0.f;
-                for (int co = 0; co < COUT; ++co)
+        for (int i = 0; i < 4; ++i) {
+            const int e = t + 256 * i, c = e / T, l = 4 * (e % T);
+            const float g0 = gs[(l / 2) * GS + c], g1 = gs[(l / 2 + 1) * GS + c];
+            const bool s0 = fmaxf(v[i].y, 0.f) > fmaxf(v[i].x, 0.f), s1 = fmaxf(v[i].w, 0.f) > fmaxf(v[i].z, 0.f);
+            float4 d;
+            d.x = (!s0 && v[i].x > 0.f) ? g0 : 0.f;
+            d.y = (s0 && v[i].y > 0.f) ? g0 : 0.f;
+            d.z = (!s1 && v[i].z > 0.f) ? g1 : 0.f;
+            d.w = (s1 && v[i].w > 0.f) ? g1 : 0.f;
+            accb[i] += (d.x + d.y) + (d.z + d.w);
+            if (CONV1) {
+                float xx[8];
 #pragma unroll
-                    for (int tap = 0; tap < 5; ++tap)
-                        s = fmaf(da_s[co * L + (l - tap + 2 + L) % L], W_s[(co * CIN + ci) * 5 + tap], s);
-                dh[(size_t)k * CIN * L + o] = s;
+                for (int q = 0; q < 8; ++q) xx[q] = xs[(l + q - 2) & (L - 1)];
+#pragma unroll
+                for (int q = 0; q < 5; ++q)
+                    accw[i][q] +=
+                        fmaf(d.x, xx[q], d.y * xx[q + 1]) + fmaf(d.z, xx[q + 2], d.w * xx[q + 3]);
+            } else {
+                reinterpret_cast<float4 *>(da + k * 4096)[e] = d;
             }
         }
     }
-    float *pp = part + (size_t)blockIdx.x * (NW + COUT);
+    // a channel's threads are T consecutive ones
+    constexpr int TW = T < 32 ? T : 32;
+    auto fold = [&](float s) {
 #pragma unroll
-    for (int i = 0; i < PER; ++i) {
-        const int o = t + 256 * i;
-        if (o < NW) pp[o] = acc[i];
+        for (int o = TW / 2; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        return s;
+    };
+    if (CONV1) {  // two warps a channel
+        static_assert(!CONV1 || T == 64, "two warps a channel");
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int q = 0; q < 6; ++q) {
+                const float s = fold(q < 5 ? accw[i][q < 5 ? q : 0] : accb[i]);
+                if ((t & 31) == 0) red[((t >> 5) * 4 + i) * 6 + q] = s;
+            }
+        __syncthreads();
+        if (t < C * 6) {
+            const int c = t / 6, q = t % 6, wp = 2 * (c & 3), i = c >> 2;
+            const float s = red[(wp * 4 + i) * 6 + q] + red[((wp + 1) * 4 + i) * 6 + q];
+            part[(size_t)blockIdx.x * (C * 6) + (q < 5 ? c * 5 + q : C * 5 + c)] = s;
+        }
+    } else {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float s = fold(accb[i]);
+            if (t % TW == 0) part[(size_t)blockIdx.x * C + (t + 256 * i) / T] = s;
+        }
     }
-    if (t < COUT) pp[NW + t] = accb;
 }
 
-// out[i] (+)= sum_b part[b][off + i] for i < n, in block order (deterministic)
-__global__ void reduce_parts_kernel(const float *part, int nblk, int stride, int off, int n, float *out)
+// out[i] = sum_b part[b][i] for i < n: a warp per output, its lanes the blocks in a fixed order
+// (one thread per output waits out 304 dependent FP64 additions, 30 us); the row's outputs lie in
+// up to three arrays of n0, n1 and n - n0 - n1.
+__global__ void __launch_bounds__(256) reduce_parts_kernel(const float *part, int nblk, int n, float *out0, int n0,
+                                                           float *out1, int n1, float *out2)
 {
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    const int i = blockIdx.x * 8 + (threadIdx.x >> 5);
     if (i >= n) return;
     double s = 0.0;
-    for (int b = 0; b < nblk; ++b) s += (double)part[(size_t)b * stride + off + i];
-    out[i] = (float)s;
+    for (int b = threadIdx.x & 31; b < nblk; b += 32) s += (double)part[(size_t)b * n + i];
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (threadIdx.x & 31) return;
+    if (i < n0) out0[i] = (float)s;
+    else if (i < n0 + n1) out1[i - n0] = (float)s;
+    else out2[i - n0 - n1] = (float)s;
+}
+
+static void reduce_parts(const float *part, int nblk, float *out0, int n0, float *out1, int n1, float *out2, int n2,
+                         cudaStream_t st)
+{
+    const int n = n0 + n1 + n2;
+    reduce_parts_kernel<<<(n + 7) / 8, 256, 0, st>>>(part, nblk, n, out0, n0, out1, n1, out2);
 }
 
 // ------------------------------------------------------------------ Adam
@@ -294,49 +321,30 @@ CnnSaved CnnSaved::layout(int64_t B)
 
 // ------------------------------------------------------------------ backward launches
 
-template <int CIN, int COUT, int L, bool DGRAD, bool XF32>
-static cudaError_t run_conv_bwd(const float *da, const void *hin, const float *W, float *dh, float *part,
-                                int64_t B, int nblk, float *gw, float *gb, cudaStream_t st)
-{
-    const size_t smem = (size_t)(COUT * L + CIN * L + (DGRAD ? COUT * CIN * 5 : 0)) * 4;
-    cudaError_t e = cudaFuncSetAttribute(conv_bwd_kernel<CIN, COUT, L, DGRAD, XF32>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    conv_bwd_kernel<CIN, COUT, L, DGRAD, XF32><<<nblk, 256, smem, st>>>(da, hin, W, dh, part, B);
-    constexpr int NW = COUT * CIN * 5;
-    reduce_parts_kernel<<<(NW + 255) / 256, 256, 0, st>>>(part, nblk, NW + COUT, 0, NW, gw);
-    reduce_parts_kernel<<<1, 64, 0, st>>>(part, nblk, NW + COUT, NW, COUT, gb);
-    return cudaGetLastError();
-}
-
-// per-block partial sums over the profiles of da[b][c][l] for each channel c (bias gradients)
-template <int C, int L>
-__global__ void __launch_bounds__(256) bias_grad_kernel(const float *da, int64_t B, float *part)
-{
-    __shared__ float acc[C];
-    for (int c = threadIdx.x; c < C; c += blockDim.x) acc[c] = 0.f;
-    __syncthreads();
-    for (int64_t k = blockIdx.x; k < B; k += gridDim.x) {
-        for (int c = threadIdx.x >> 5; c < C; c += blockDim.x >> 5) {
-            float s = 0.f;
-            for (int l = threadIdx.x & 31; l < L; l += 32) s += da[(k * C + c) * L + l];
-            for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-            if ((threadIdx.x & 31) == 0) acc[c] += s;
-        }
-    }
-    __syncthreads();
-    for (int c = threadIdx.x; c < C; c += blockDim.x) part[(size_t)blockIdx.x * C + c] = acc[c];
-}
-
-// out(m, n) = sum over splits s (in order) of part[s][m][n], stored by st(m, n, value)
+// out(m, n) = sum over splits s of part[s][m][n], stored by st(m, n, value). A block takes 32
+// outputs, its eight warps every eighth split each, added up in a fixed order (a thread per output
+// leaves all but 40 blocks' worth of the chip idle for 152 dependent FP64 additions: 130 us for
+// conv3's 64 x 160).
 template <class ST>
-__global__ void reduce_splits_kernel(const float *part, int splits, int64_t rows, int64_t cols, ST st)
+__global__ void __launch_bounds__(256) reduce_splits_kernel(const float *part, int splits, int64_t rows, int cols,
+                                                            ST st)
 {
+    __shared__ double red[8][32];
     const int64_t total = rows * cols;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (int64_t)gridDim.x * blockDim.x) {
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    for (int64_t e0 = (int64_t)blockIdx.x * 32; e0 < total; e0 += (int64_t)gridDim.x * 32) {
+        const int64_t e = e0 + lane;
         double v = 0.0;
-        for (int s = 0; s < splits; ++s) v += (double)part[(size_t)s * total + e];
-        st(e / cols, e % cols, (float)v);
+        if (e < total)
+            for (int s = w; s < splits; s += 8) v += (double)part[(size_t)s * total + e];
+        red[w][lane] = v;
+        __syncthreads();
+        if (w == 0 && e < total) {
+#pragma unroll
+            for (int q = 1; q < 8; ++q) v += red[q][lane];
+            st(e / cols, e % cols, (float)v);
+        }
+        __syncthreads();
     }
 }
 struct StWf1 {  // dW(fc1)[j][fd] -> PyTorch order
@@ -348,12 +356,6 @@ struct StRowMajor {
     int64_t ld;
     __device__ void operator()(int64_t r, int64_t c, float v) const { g[r * ld + c] = v; }
 };
-template <int C, int L>
-struct StDh {  // input gradient [(b, m)][ci] -> [b][ci][m]
-    float *dh;
-    __device__ void operator()(int64_t r, int64_t ci, float v) const { dh[((r / L) * C + ci) * L + (r % L)] = v; }
-};
-
 // The tensor-core GEMMs of one backward pass: (rows of A and of the output, rows of B = N,
 // K, N tile, split-K count). Operands and partials share three workspace buffers.
 struct BwdGemmShape {
@@ -393,12 +395,8 @@ size_t cnn_backward_ws_bytes(int64_t B, int nblk, int num_sms)
     size_t o = 0;
     auto take = [&](size_t bytes) { o = ((o + 255) & ~(size_t)255) + bytes; };
     take((size_t)B * 256 * 4);         // dZ1
-    take((size_t)B * 2048 * 4);        // dH3
-    take((size_t)B * 64 * 64 * 4);     // da3
-    take((size_t)B * 32 * 64 * 4);     // dh2
-    take((size_t)B * 32 * 128 * 4);    // da2
-    take((size_t)B * 16 * 128 * 4);    // dh1
-    take((size_t)B * 16 * 256 * 4);    // da1
+    take((size_t)B * 2048 * 4);        // dH3, then dh2 and dh1
+    take((size_t)B * 64 * 64 * 4);     // da3, then da2
     take((size_t)nblk * (16 * 5 + 16) * 4);  // conv1 weight/bias partials
     take((size_t)nblk * 64 * 4);       // bias partials
     take((size_t)nblk * 513 * 4);      // head partials
@@ -410,15 +408,17 @@ size_t cnn_backward_ws_bytes(int64_t B, int nblk, int num_sms)
     return o + 256;
 }
 
-// pack A and B of GEMM `which`, run it and hand its partials to `store`
+// Pack A and B of GEMM `which`, run it and hand its partials to `store`; or, where `whole` is
+// given and the GEMM's K is not split, leave them where they are: *whole is the row-major result
+// (else it is what `store` wrote).
 template <class LA, class LB, class ST>
-static cudaError_t bwd_gemm(int which, int64_t B, int num_sms, LA la, LB lb, ST store, uint8_t *pa, uint8_t *pb,
-                            float *part, cudaStream_t st)
+static cudaError_t bwd_gemm(int which, int64_t B, int num_sms, LA la, LB lb, ST store, const float **whole,
+                            uint8_t *pa, uint8_t *pb, float *part, cudaStream_t st)
 {
     const BwdGemmShape s = bwd_shape(which, B, num_sms);
     const int64_t kch = (s.K + 63) / 64;
-    const int64_t ga = std::min<int64_t>(65535, ((s.M + 127) / 128 * 128 * kch * 8 + 255) / 256);
-    const int64_t gb = std::min<int64_t>(65535, ((s.N + s.bn - 1) / s.bn * s.bn * kch * 8 + 255) / 256);
+    const int64_t ga = std::min<int64_t>(65535, (s.M + 127) / 128 * kch);
+    const int64_t gb = std::min<int64_t>(65535, (s.N + s.bn - 1) / s.bn * kch);
     pack_tiles_kernel<<<(int)ga, 256, 0, st>>>(s.M, 128, s.K, la, pa);
     pack_tiles_kernel<<<(int)gb, 256, 0, st>>>(s.N, s.bn, s.K, lb, pb);
     TcGemm g{};
@@ -434,9 +434,13 @@ static cudaError_t bwd_gemm(int which, int64_t B, int num_sms, LA la, LB lb, ST 
     g.part = part;
     cudaError_t e = launch_tcgemm(g, num_sms, st);
     if (e != cudaSuccess) return e;
+    if (whole && s.splits == 1) {
+        *whole = part;
+        return cudaSuccess;
+    }
     const int64_t total = s.M * g.ldp;
-    reduce_splits_kernel<<<(int)std::min<int64_t>(4096, (total + 255) / 256), 256, 0, st>>>(part, s.splits, s.M,
-                                                                                              g.ldp, store);
+    reduce_splits_kernel<<<(int)std::min<int64_t>(8192, (total + 31) / 32), 256, 0, st>>>(part, s.splits, s.M,
+                                                                                            (int)g.ldp, store);
     return cudaGetLastError();
 }
 
@@ -453,12 +457,8 @@ cudaError_t launch_cnn_backward(const CnnSrc &w, const uint8_t *saved, int64_t B
         return p;
     };
     float *dZ1 = reinterpret_cast<float *>(take((size_t)B * 256 * 4));
-    float *dH3 = reinterpret_cast<float *>(take((size_t)B * 2048 * 4));
-    float *da3 = reinterpret_cast<float *>(take((size_t)B * 64 * 64 * 4));
-    float *dh2 = reinterpret_cast<float *>(take((size_t)B * 32 * 64 * 4));
-    float *da2 = reinterpret_cast<float *>(take((size_t)B * 32 * 128 * 4));
-    float *dh1 = reinterpret_cast<float *>(take((size_t)B * 16 * 128 * 4));
-    float *da1 = reinterpret_cast<float *>(take((size_t)B * 16 * 256 * 4));
+    float *dh = reinterpret_cast<float *>(take((size_t)B * 2048 * 4));
+    float *da = reinterpret_cast<float *>(take((size_t)B * 64 * 64 * 4));
     float *cpart = reinterpret_cast<float *>(take((size_t)nblk * (16 * 5 + 16) * 4));
     float *bpart = reinterpret_cast<float *>(take((size_t)nblk * 64 * 4));
     float *hpart = reinterpret_cast<float *>(take((size_t)nblk * 513 * 4));
@@ -471,40 +471,38 @@ cudaError_t launch_cnn_backward(const CnnSrc &w, const uint8_t *saved, int64_t B
 
     const float *z1 = reinterpret_cast<const float *>(saved + S.z1);
     head_bwd_kernel<<<nblk, 256, 0, st>>>(z1, dlogit, w.wf2, B, dZ1, hpart);
-    reduce_parts_kernel<<<1, 256, 0, st>>>(hpart, nblk, 513, 0, 256, g.wf2);
-    reduce_parts_kernel<<<1, 256, 0, st>>>(hpart, nblk, 513, 256, 256, g.bf1);
-    reduce_parts_kernel<<<1, 32, 0, st>>>(hpart, nblk, 513, 512, 1, g.bf2);
+    reduce_parts(hpart, nblk, g.wf2, 256, g.bf1, 256, g.bf2, 1, st);
     // dW(fc1)[256][2048] = dZ1^T h3; dh3[B][2048] = dZ1 W1
-    cudaError_t e = bwd_gemm(0, B, sms, LdDZ1T{dZ1}, LdH3T{saved + S.h3t}, StWf1{g.wf1}, pa, pb, gpart, st);
-    if (e == cudaSuccess) e = bwd_gemm(1, B, sms, LdDZ1{dZ1}, LdW1T{w.wf1}, StRowMajor{dH3, 2048}, pa, pb, gpart, st);
-    if (e != cudaSuccess) return e;
-    const int eb = 256;
-    const int egrid = (int)std::min<int64_t>((B * 64 * 32 + eb - 1) / eb, 65535);
-    poolrelu_bwd_kernel<64, 64, true><<<egrid, eb, 0, st>>>(reinterpret_cast<const float *>(saved + S.a3), dH3,
-                                                              da3, B);
-    // conv3: dW[64][160] and dh2, bias by reduction
-    e = bwd_gemm(2, B, sms, LdDa<64, 64>{da3}, LdHim<32, 64>{reinterpret_cast<const uint16_t *>(saved + S.h2)},
-                 StRowMajor{g.w3, 160}, pa, pb, gpart, st);
+    const float *gp = dh;  // a GEMM's result for the layer below
+    cudaError_t e = bwd_gemm(0, B, sms, LdDZ1T{dZ1}, LdH3T{saved + S.h3t}, StWf1{g.wf1}, nullptr, pa, pb, gpart, st);
     if (e == cudaSuccess)
-        e = bwd_gemm(3, B, sms, LdDaShift<64, 64>{da3}, LdWT<32>{w.w3}, StDh<32, 64>{dh2}, pa, pb, gpart, st);
+        e = bwd_gemm(1, B, sms, LdDZ1{dZ1}, LdW1T{w.wf1}, StRowMajor{dh, 2048}, &gp, pa, pb, gpart, st);
     if (e != cudaSuccess) return e;
-    bias_grad_kernel<64, 64><<<nblk, 256, 0, st>>>(da3, B, bpart);
-    reduce_parts_kernel<<<1, 64, 0, st>>>(bpart, nblk, 64, 0, 64, g.b3);
-    poolrelu_bwd_kernel<32, 128, false><<<egrid, eb, 0, st>>>(reinterpret_cast<const float *>(saved + S.a2), dh2,
-                                                                da2, B);
-    // conv2: dW[32][80] and dh1, bias by reduction
-    e = bwd_gemm(4, B, sms, LdDa<32, 128>{da2}, LdHim<16, 128>{reinterpret_cast<const uint16_t *>(saved + S.h1)},
-                 StRowMajor{g.w2, 80}, pa, pb, gpart, st);
+    // conv3: da3 and bias, dW[64][160] and dh2
+    poolrelu_bwd_kernel<64, 64, false>
+        <<<nblk, 256, 0, st>>>(reinterpret_cast<const float *>(saved + S.a3), gp, nullptr, da, B, bpart);
+    reduce_parts(bpart, nblk, g.b3, 64, nullptr, 0, nullptr, 0, st);
+    e = bwd_gemm(2, B, sms, LdDa<64, 64>{da}, LdHim<32, 64>{reinterpret_cast<const uint16_t *>(saved + S.h2)},
+                 StRowMajor{g.w3, 160}, nullptr, pa, pb, gpart, st);
+    gp = dh;
     if (e == cudaSuccess)
-        e = bwd_gemm(5, B, sms, LdDaShift<32, 128>{da2}, LdWT<16>{w.w2}, StDh<16, 128>{dh1}, pa, pb, gpart, st);
+        e = bwd_gemm(3, B, sms, LdDaShift<64, 64>{da}, LdWT<32>{w.w3}, StRowMajor{dh, 32}, &gp, pa, pb, gpart, st);
     if (e != cudaSuccess) return e;
-    bias_grad_kernel<32, 128><<<nblk, 256, 0, st>>>(da2, B, bpart);
-    reduce_parts_kernel<<<1, 64, 0, st>>>(bpart, nblk, 32, 0, 32, g.b2);
-    poolrelu_bwd_kernel<16, 256, false><<<egrid, eb, 0, st>>>(reinterpret_cast<const float *>(saved + S.a1), dh1,
-                                                                da1, B);
+    // conv2: da2 and bias, dW[32][80] and dh1
+    poolrelu_bwd_kernel<32, 128, false>
+        <<<nblk, 256, 0, st>>>(reinterpret_cast<const float *>(saved + S.a2), gp, nullptr, da, B, bpart);
+    reduce_parts(bpart, nblk, g.b2, 32, nullptr, 0, nullptr, 0, st);
+    e = bwd_gemm(4, B, sms, LdDa<32, 128>{da}, LdHim<16, 128>{reinterpret_cast<const uint16_t *>(saved + S.h1)},
+                 StRowMajor{g.w2, 80}, nullptr, pa, pb, gpart, st);
+    gp = dh;
+    if (e == cudaSuccess)
+        e = bwd_gemm(5, B, sms, LdDaShift<32, 128>{da}, LdWT<16>{w.w2}, StRowMajor{dh, 16}, &gp, pa, pb, gpart, st);
+    if (e != cudaSuccess) return e;
     // conv1 (16 x 5 weights) on CUDA cores
-    e = run_conv_bwd<1, 16, 256, false, true>(da1, saved + S.x, w.w1, nullptr, cpart, B, nblk, g.w1, g.b1, st);
-    if (e != cudaSuccess) return e;
+    poolrelu_bwd_kernel<16, 256, true>
+        <<<nblk, 256, 0, st>>>(reinterpret_cast<const float *>(saved + S.a1), gp,
+                               reinterpret_cast<const float *>(saved + S.x), nullptr, B, cpart);
+    reduce_parts(cpart, nblk, g.w1, 80, g.b1, 16, nullptr, 0, st);
     return cudaGetLastError();
 }
 

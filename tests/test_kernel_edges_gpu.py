@@ -181,3 +181,26 @@ def test_detrending_of_short_and_odd_segments(ctx, lengths):
         if len(r["times"]):
             err = np.abs(fo.cpu().numpy().astype(np.float64) - r["flux"]) / np.abs(r["flux"])
             assert err.max() <= FLUX_RTOL
+
+
+@pytest.mark.parametrize("batch", [2, 130, 609, 2561])
+def test_gradients_of_a_batch_are_the_sum_of_its_halves(ctx, batch):
+    """The GEMMs of a large batch are not split over K, those of a small one are, into other pieces:
+    the gradients of the whole batch against its halves' sum. FP32 sums in another order, and a rare
+    BF16 rounding of a gradient that this moves across a tie: 1e-4 of a tensor's norm."""
+    import paper_2312_02063_gb300 as g
+    prof, lab = lcsynth.profiles_mixed(batch, seed=3)
+    wd = {k: _dev(ctx, v) for k, v in lcsynth.cnn_init(3, bias_scale=0.05).items()}
+    f = _dev(ctx, prof)
+    logit, saved = g.gpfc_cnn_forward_train(ctx, f, wd)
+    _, dl = g.gpfc_bce_with_logits(ctx, logit, _dev(ctx, lab.astype(np.float32)))
+    whole = g.gpfc_cnn_backward(ctx, dl, wd, saved)
+    h = batch // 2
+    parts = []
+    for a, b in ((0, h), (h, batch)):
+        _, sv = g.gpfc_cnn_forward_train(ctx, f[a:b].contiguous(), wd)
+        parts.append(g.gpfc_cnn_backward(ctx, dl[a:b].contiguous(), wd, sv))
+    ctx.sync()
+    for n in g.CNN_PARAM_NAMES:
+        w, s = whole[n].double(), parts[0][n].double() + parts[1][n].double()
+        assert float((w - s).norm()) <= 1e-4 * float(s.norm()) + 1e-12, n
