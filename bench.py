@@ -35,8 +35,8 @@ UNIT = "sample·period folds/s"
 NBINS = 256
 N_PERIODS = 250_000  # default; --n-periods changes it (small cases for profiling)
 W_MAX = int(math.ceil(0.42 * NBINS))  # 108: widths up to the longest injected duty cycle
-SM_FOLD_UPDATES_PER_CLK = 16          # the pipe model: 128 B/clk / (4 B + 4 B of reductions)
-# DRAM bytes (read + write) of the fold kernel's 18 launches of one 250,000-period search of
+SM_FOLD_UPDATES_PER_CLK = 32          # the pipe model: 128 B/clk / one 4-byte reduction
+# DRAM bytes (read + write) of the fold kernel's launches of one 250,000-period search of
 # the same light curve in steady state (no cache flush, one ncu pass), per period:
 # profiles/dram_traffic_steady_state_kepler62835.md
 SEARCH_DRAM_BYTES_PER_PERIOD = (0.403456e6 + 206.749696e6) / 250000
@@ -569,9 +569,9 @@ def run_gpu(args, rank, world, local_rank):
         model_gups = sms * SM_FOLD_UPDATES_PER_CLK * smax * 1e6 / 1e9
         # the fold's binding pipe, measured here: lane-private shared-memory updates of the
         # fold's 8-byte bin record at full occupancy (16 warps x 32 bins per SM), as two
-        # no-return reductions (the default fold's record) and as a 64-bit read-modify-write
-        # (the FP32 layout's record), and both at the fold's own footprint (256 bins x 3
-        # period groups per SM)
+        # no-return reductions (the two-word record; the one-word fold takes one, so its peak is
+        # twice that) and as a 64-bit read-modify-write (the FP32 layout's record), and both at
+        # 256 bins x 3 period groups per SM
         probe = {}
         for key, cfg, op in (("red8_full", (8, 32, 16, 1), 1), ("red8_fold_footprint", (8, 256, 3, 1), 1),
                              ("rmw8_full", (8, 32, 16, 1), 0), ("rmw8_fold_footprint", (8, 256, 3, 1), 0)):
@@ -579,7 +579,7 @@ def run_gpu(args, rank, world, local_rank):
             probe[key] = {"gupdates_per_s": ups / 1e9, "updates_per_clk_sm": upc,
                           "config": f"{cfg[0]}-byte record, {'two 32-bit reductions' if op else 'load + store'}, "
                                     f"{cfg[1]} bins x {cfg[2]} warps per SM"}
-        peak_gups = probe["red8_full"]["gupdates_per_s"]
+        peak_gups = 2.0 * probe["red8_full"]["gupdates_per_s"]
         kmean = statistics.mean(kernel_ms)
         # the search kernel's own launch (fold + box-SNR): all n * N_PERIODS updates of a step
         # over its duration
@@ -601,7 +601,7 @@ def run_gpu(args, rank, world, local_rank):
                        "l2": "flushed between timed steps (256 MB write outside the events)",
                        "parallelism": "replicas" if world > 1 else "single"},
             "periods_scored_per_s": world * N_PERIODS / (ms_per_step * 1e-3),
-            "roofline": {"bound": "smem", "kernel": "fold_kernel (reduction layout, 3 period groups, 12 sample streams across them)",
+            "roofline": {"bound": "smem", "kernel": "fold_pack_kernel (one word per bin and period, 6 period groups, 16 warps across them)",
                          "achieved": achieved,
                          "peak": peak_gups, "unit": "Gupdates/s", "frac": achieved / peak_gups,
                          "traffic": None if SEARCH_DRAM_BYTES_PER_PERIOD is None
@@ -611,13 +611,13 @@ def run_gpu(args, rank, world, local_rank):
                                           "by periods and divided by the launches of a step",
                          "kernel_ms": fold_step_ms / launches, "launches_per_step": launches,
                          "search_ms": kmean,
-                         "peak_basis": "measured in this run by gpfc_probe_smem_rmw: lane-private updates of "
-                                       "the fold's 8-byte record (32-bit sum and count words) by two "
-                                       "red.shared.add.u32, 16 warps x 32 bins per SM, "
-                                       f"{probe['red8_full']['updates_per_clk_sm']:.2f} updates/clk/SM",
+                         "peak_basis": "measured in this run by gpfc_probe_smem_rmw: lane-private "
+                                       "red.shared.add.u32, two per update of an 8-byte record, 16 warps x 32 "
+                                       f"bins per SM, {probe['red8_full']['updates_per_clk_sm']:.2f} updates/clk/SM; "
+                                       "twice that for the fold's one reduction per update",
                          "peak_model": model_gups,
                          "peak_model_basis": f"{sms} SMs x {SM_FOLD_UPDATES_PER_CLK} updates/clk (128 B/clk over "
-                                             f"8 B of reductions per update) x {smax:.0f} MHz ({src} sm_max_mhz)",
+                                             f"one 4-byte reduction per update) x {smax:.0f} MHz ({src} sm_max_mhz)",
                          "probe": probe},
             "cpu_baseline": cpu,
             "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": h2d, "d2h_bytes_per_step": d2h,

@@ -140,8 +140,8 @@ int gpfc_last_fold_plan(const gpfc_ctx *ctx, gpfc_fold_config *out);
  * With autotuning enabled (the default), gpfc_fold, gpfc_search and gpfc_search_batched
  * use a tuned config with a matching key, and gpfc_search_batched tunes on its first
  * star when there is none (keyed by the average star length), unless its stream is
- * capturing or the automatic plan is the one-word fold (see gpfc_fold_config). gpfc_set_autotune(ctx, 0) disables both; enable < 0 also forgets the
- * tuned configs. Fields set by gpfc_set_fold_config take precedence. */
+ * capturing or the automatic plan is the one-word fold (see gpfc_fold_config).
+ * gpfc_set_autotune(ctx, 0) disables both; enable < 0 also forgets the tuned configs. Fields set by gpfc_set_fold_config take precedence. */
 int gpfc_autotune(gpfc_ctx *ctx, const double *times, const float *flux, int64_t n,
                   const double *periods, int64_t n_periods, int32_t nbins, int scorer,
                   const void *scorer_params, gpfc_fold_config *out);

@@ -90,9 +90,10 @@ __device__ __forceinline__ uint32_t phase_hi(uint32_t tl, uint32_t thF, uint32_t
 }
 
 // Shared address of a sample's bin word for one period (KIND 0: 256 bins, 1: a power of two,
-// 2: any; 3 and 4: below 256 bins, HILO, a power of two or any). With 256 bins the bin is the top byte of the phase and rows are 256 bytes, so one
-// byte permutation builds the address: byte 0 = lane and group parity, byte 1 = bin, the rest the
-// slab; the slab's distance from a multiple of 64 KB is the reduction's immediate offset.
+// 2: any; 3 and 4: below 256 bins, HILO, a power of two or any). With 256 bins the bin is the top
+// byte of the phase and rows are 256 bytes, so one byte permutation builds the address: byte 0 =
+// lane and group parity, byte 1 = bin, the rest the slab; the slab's distance from a multiple of
+// 64 KB is the reduction's immediate offset.
 template <int KIND>
 __device__ __forceinline__ uint32_t word_addr(uint32_t hi, uint32_t tl, uint32_t Fl, uint32_t base, uint32_t nbins,
                                               int shift)
@@ -211,7 +212,8 @@ __global__ void __launch_bounds__(kPackThreads, 1) fold_pack_kernel(const FoldPa
     // biased sum up to 2^23 samples, else an int64 sum and, in the third plane, 32-bit counts),
     // then the slots
     const size_t plane = (size_t)nbins * ppc;
-    uint32_t *ws = reinterpret_cast<uint32_t *>(p.ws_sc) + (size_t)blockIdx.x * (HILO ? kPackPlanesHilo : kPackPlanes) * plane + lane;
+    constexpr int kPlanes = HILO ? kPackPlanesHilo : kPackPlanes;
+    uint32_t *ws = reinterpret_cast<uint32_t *>(p.ws_sc) + (size_t)blockIdx.x * kPlanes * plane + lane;
     unsigned long long *ws_tot = reinterpret_cast<unsigned long long *>(ws - lane) + lane;
     uint32_t *ws_cnt = ws + 2 * plane, *ws_slot = ws + 3 * plane;
 
@@ -282,7 +284,7 @@ __global__ void __launch_bounds__(kPackThreads, 1) fold_pack_kernel(const FoldPa
         while (tile > 256 && (float)tile > 8.6f * (float)pw.M) tile >>= 1;
         const int ntiles = (int)((nsamp + tile - 1) / tile);
         // The block's segments: of seg_tiles tiles, about kPackSegTiles but no more than a mean load of
-        // half M allows; into slots where a star of one chunk has at most kPackSegs of them.
+        // about half M allows; into slots where a star of one chunk has at most kPackSegs of them.
         const int most = max(1, (int)fminf(0.55f * (float)pw.M * (float)nbins / (float)tile, 1e6f));
         int nsegs = max(1, (ntiles + kPackSegTiles - 1) / kPackSegTiles);
         if (nsegs > kPackSegs && nsamp <= (int64_t)p.chunk) nsegs = kPackSegs;
@@ -739,8 +741,6 @@ size_t fold_pack_smem(int nbins, int groups)
     return pack_records_addr(kWindow, nbins) - kWindow + pack_records_bytes(nbins, groups);
 }
 
-int fold_pack_allowed(int nbins, int groups);
-
 int fold_pack_groups(int nbins)
 {
     int g = kPackMaxGroups;
@@ -767,6 +767,7 @@ static cudaError_t with_kernel(int nbins, int shift, int groups, F f)
     return with_groups<2, 5>(groups, f);                  // 257 bins and more
 }
 
+// (4 and 5 have no HILO instance: a grid of that few periods a multiprocessor takes 3)
 int fold_pack_allowed(int nbins, int groups) { return nbins < 256 && (groups == 4 || groups == 5) ? 3 : groups; }
 
 int fold_pack_register()
