@@ -204,3 +204,29 @@ def test_gradients_of_a_batch_are_the_sum_of_its_halves(ctx, batch):
     for n in g.CNN_PARAM_NAMES:
         w, s = whole[n].double(), parts[0][n].double() + parts[1][n].double()
         assert float((w - s).norm()) <= 1e-4 * float(s.norm()) + 1e-12, n
+
+
+# two rows of 32-bit words up to 65,536 samples, 64-bit words above; final bins about the 31 that a warp
+# finishes at a time
+@pytest.mark.parametrize("n,kind,nbins,merged", [
+    (16383, "regular", 2048, 30), (16384, "regular", 1025, 31), (16385, "gaps", 3000, 32), (40000, "equal", 4096, 61),
+    (65536, "regular", 4096, 62), (65537, "gaps", 4096, 63), (9000, "gaps", 1030, 2)])
+def test_fine_bins_and_their_merging(ctx, n, kind, nbins, merged):
+    import paper_2312_02063_gb300 as g
+    rng = np.random.default_rng(n)
+    t = np.arange(n) * CADENCE + (3.3 * (np.arange(n) // 911) if kind == "gaps" else 0.0)
+    if kind == "equal":
+        t = np.full(n, 7.25)
+    f = (1.0 + rng.normal(0.0, 3e-4, n)).astype(np.float32)
+    p = np.r_[10 * CADENCE, rng.uniform(0.2, 1.0, 6), 17 * CADENCE]
+    args = [_dev(ctx, x) for x in (t, f, p)]
+    folded, counts = g.gpfc_fold(ctx, *args, nbins, 0.0)
+    eq = g.gpfc_fold_equal_count(ctx, *args, merged, nbins, 0.0)
+    ctx.sync()
+    mean_o, cnt_o, _ = oracle.fold(t, f, p, nbins, 0.0)
+    fo, co = folded.cpu().numpy().astype(np.float64), counts.cpu().numpy()
+    np.testing.assert_array_equal(co, cnt_o)
+    nz = cnt_o > 0
+    assert np.all(np.abs(fo[nz] - mean_o[nz]) <= MEAN_RTOL * np.abs(mean_o[nz]))
+    eq_o, _ = oracle.fold_equal_count(t, f, p, nbins, merged, 0.0)
+    assert np.all(np.abs(eq.cpu().numpy() - eq_o) <= MEAN_RTOL * np.abs(eq_o))
