@@ -14,8 +14,7 @@
 // follows a run past the chunk's end until it closes; qualifying runs go to the candidate
 // list of the cluster's first block (the first kPkCap of them; the best peak and the count are
 // exact in any case). What bounds it: FP64 instructions (one per warp and scheduler every 64
-// cycles), five a period; one block takes 0.60 ms for 250,000 periods, see kPkCluster for a
-// cluster of sixteen.
+// cycles), five a period; one block takes 0.60 ms for 250,000 periods, a cluster of sixteen 0.09 ms.
 #include <cmath>
 #include <cooperative_groups.h>
 #include <cstdint>
