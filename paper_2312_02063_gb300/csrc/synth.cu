@@ -22,7 +22,8 @@
 //  * flux: x is summed as integers, rint(x 2^e) with |x| 2^e <= 2^22 (an FP32 add with a large
 //    constant rounds it), by shared-memory reductions: the low 11 bits, the rest and the count
 //    each have a word per bin. Integer sums are exact and independent of their order; sum and
-//    sum of squares (a 64-bit integer per lane) also give the flux standard deviation.
+//    sum of squares (a 64-bit integer per lane, emptied into FP64 with the bin words) also give the
+//    flux standard deviation.
 // 4,096 curves of 65,536 samples: 12.5 ms with FP64 phases, fmod, moments and a 32-shuffle
 // merge of equal bins per sample; now 1.17 ms.
 #include <cmath>
@@ -167,7 +168,9 @@ __device__ __noinline__ long long tau_fp64(int i, double cadence)
 // the others' samples; 1,024 where there are too few light curves to fill the SMs that way.
 constexpr int kSynthThreads = 256, kSynthWide = 1024;
 
-constexpr int kSynthSpan = 1 << 19;  // samples between emptyings of the 32-bit bin words
+// Samples between emptyings of the 32-bit bin words and of a lane's squares (2,048 of 2^44 at most: a
+// warp's share of a whole light curve passes 2^64 from 2^24 cadences).
+constexpr int kSynthSpan = 1 << 19;
 
 template <bool POW2, int THREADS>
 __global__ void __launch_bounds__(THREADS) synth_fold_kernel(SynthParams P, int shift)
@@ -194,11 +197,12 @@ __global__ void __launch_bounds__(THREADS) synth_fold_kernel(SynthParams P, int 
         const uint32_t step_i = lp.step_i, sfl = (uint32_t)lp.step_f, sfh = (uint32_t)(lp.step_f >> 32), tguard = lp.tguard;
         const uint64_t step20 = lp.step20;
         const float sigma = lp.sigma, scale = lp.scale;
-        unsigned long long m2 = 0ull;          // sum of squares of this lane's integers
+        double m2 = 0.0;                       // sum of squares of this lane's integers
         long long tot = 0;                     // bin tid: sum and count
         uint32_t cnt = 0u;
         for (int64_t span = 0; span < n; span += kSynthSpan) {
             const int i_end = (int)min((int64_t)n, span + kSynthSpan);
+            unsigned long long sq = 0ull;
             for (int64_t base = span + 128 * warp; base < i_end; base += 128 * nw) {
                 const int i0 = (int)base + 4 * lane;  // this lane's four samples
                 if (i0 >= i_end) break;               // (no warp-wide operation below)
@@ -251,7 +255,7 @@ __global__ void __launch_bounds__(THREADS) synth_fold_kernel(SynthParams P, int 
                         }
                         // rint(x 2^e): the sum with 3 2^22 has a unit in its last place of 1
                         const int xq = __float_as_int(fmaf(x, scale, 12582912.0f)) - 0x4B400000;
-                        m2 += (unsigned long long)((long long)xq * (long long)xq);
+                        sq += (unsigned long long)((long long)xq * (long long)xq);
                         const unsigned long long phi = (unsigned long long)tl * Fl +
                                                        ((unsigned long long)(th * Fl + tl * Fh) << 32);
                         const uint32_t bin = POW2 ? (uint32_t)(phi >> 32) >> shift
@@ -262,6 +266,7 @@ __global__ void __launch_bounds__(THREADS) synth_fold_kernel(SynthParams P, int 
                     }
                 }
             }
+            m2 += (double)sq;
             __syncthreads();
             if (tid < nb) {
                 tot += ((long long)(int32_t)s_hi[tid] << 11) + (long long)s_lo[tid];
@@ -284,7 +289,7 @@ __global__ void __launch_bounds__(THREADS) synth_fold_kernel(SynthParams P, int 
             }
             if (lane == 0) {
                 if (warp < 8) s_m1[warp] = tot;  // (256 bins: the first eight warps)
-                s_m2[warp] = (double)m2;
+                s_m2[warp] = m2;
             }
             __syncthreads();
             if (tid == 0) {

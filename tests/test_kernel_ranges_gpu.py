@@ -1,0 +1,50 @@
+"""Ranges beyond the usual ones: long generated curves, flux with outliers or that is no number, resonant and
+irregular times, wide profiles, large scales, and the workspace. Times are compared on the same GPU in the same
+process, with room for noise."""
+import numpy as np
+import pytest
+import torch
+
+import lcsynth
+import oracle
+
+pytestmark = pytest.mark.gpu
+CADENCE = 29.4 / 1440.0
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    import paper_2312_02063_gb300 as g
+    c = g.Context(0)
+    yield c
+    c.close()
+
+
+def _dev(ctx, a):
+    return torch.from_numpy(np.ascontiguousarray(a)).to(ctx.device)
+
+
+# ---------------------------------------------------------------- generated profiles
+
+def test_flux_std_of_a_long_sinusoid(ctx):
+    """2^27 cadences whose squares sum to more than 64 bits of the integers they are added as. The
+    expected value is that of whole cycles; a part of one among 10^5 changes it by 1e-6."""
+    import paper_2312_02063_gb300 as g
+    amp, sigma = 0.0019, 1e-6
+    sp = dict(g.TRAINING_SET, n_cadences=1 << 27, cadence=1 / 1440.0, depth_min=amp, depth_max=amp, sigma_min=sigma,
+              sigma_max=sigma)
+    _, counts, _, _, std = g.gpfc_synth_profiles(ctx, 5, 3, 1, 256, sp, want_std=True)  # curve 3: a sinusoid
+    ctx.sync()
+    assert int(counts.sum().item()) == 1 << 27
+    assert abs(float(std[0]) / (amp * amp / 2 + sigma * sigma) ** 0.5 - 1.0) <= 1e-5
+
+
+@pytest.mark.parametrize("n_cad,nbins", [(300, 256), (5003, 37), (131073, 200)])
+def test_flux_std_does_not_depend_on_the_batch(ctx, n_cad, nbins):
+    import paper_2312_02063_gb300 as g
+    sp = dict(lcsynth.TRAINING_SET, n_cadences=n_cad)
+    many = g.gpfc_synth_profiles(ctx, 9, 40, 640, nbins, sp, want_std=True)[4]
+    for j in (0, 1, 3, 639):
+        one = g.gpfc_synth_profiles(ctx, 9, 40 + j, 1, nbins, sp, want_std=True)[4]
+        ctx.sync()
+        assert abs(float(one[0]) / float(many[j]) - 1.0) <= 2.0 ** -23
