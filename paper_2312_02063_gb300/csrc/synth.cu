@@ -19,13 +19,14 @@
 //    period; both know how far they can be off, and a sample that close to a rounding or box
 //    edge (one in some 10^5) is decided by the FP64 formula itself, so every bin, count and
 //    membership is that of the formula.
-//  * flux: x is summed as integers, rint(x 2^e) with |x| 2^e <= 2^22 (an FP32 add with a large
-//    constant rounds it), by shared-memory reductions: the low 11 bits, the rest and the count
-//    each have a word per bin. Integer sums are exact and independent of their order; sum and
-//    sum of squares (a 64-bit integer per lane, emptied into FP64 with the bin words) also give the
-//    flux standard deviation.
+//  * flux: x is summed as integers, rint(x 2^e) with |x| 2^e < 2^29 (exact where |x| 2^e is 2^24 or
+//    more), by shared-memory reductions: the low 15 bits, the rest and the count each have a word
+//    per bin. Integer sums are exact and independent of their order; sum and sum of squares (of
+//    the upper 26 bits, a 64-bit integer per lane, emptied into FP64 with the bin words) also give
+//    the flux standard deviation.
+//  * a sinusoid's phase is fixed point too, and its flux a sum of FP32 pairs.
 // 4,096 curves of 65,536 samples: 12.5 ms with FP64 phases, fmod, moments and a 32-shuffle
-// merge of equal bins per sample; now 1.17 ms.
+// merge of equal bins per sample; now 1.32 ms.
 #include <cmath>
 #include <cstdint>
 
@@ -67,13 +68,14 @@ struct LcParams {
     int kind;        // 0 transit, 1 noise, 2 sinusoid, 3 eclipsing binary
     int fixed;       // the fixed-point phases below hold for every sample
     double period, epoch, duration, fold_period;
-    float sigma, depth, depth2, amp;
+    float sigma, depth, depth2, amp, amp_lo;  // (amp + amp_lo: to FP64's precision)
     uint32_t Fl, Fh;  // fold frequency, rint(2^40 / fold_period)
     uint32_t Gl, Gh;  // light curve's own frequency, rint(2^40 / period)
     uint32_t off;     // epoch / period in 2^-32 cycles
     uint32_t half;    // half the duration in 2^-32 cycles
     uint32_t guard;   // bound of the phase's error in 2^-32 cycles
     float cyc;        // 2^-24 / period: cycles per unit of tau
+    float drift;      // cycles per 2^16 units of tau that 2^-40 (Gh 2^32 + Gl) falls short by
     float scale;      // 2^e
     int e;
     // the cadence in units of tau: integer part, fraction in 2^-64; and in 2^-20 (64-bit)
@@ -110,12 +112,13 @@ __device__ LcParams lc_params(uint64_t seed, int64_t j, const gpfc_synth_params 
     p.depth = (float)depth;
     p.depth2 = (float)depth2;
     p.amp = (float)amp;
+    p.amp_lo = (float)(amp - (double)p.amp);
     const unsigned long long F = (unsigned long long)__double2ll_rn(__ddiv_rn(1099511627776.0, p.fold_period));
     p.Fl = (uint32_t)F;
     p.Fh = (uint32_t)(F >> 32);
     // |x| < 5.78 sigma (the largest Box-Muller radius for u >= 2^-24) plus the signal
     const double xmax = 5.78 * sigma + (p.kind == 2 ? amp : (p.kind == 0 ? depth : (p.kind == 3 ? depth + depth2 : 0.0)));
-    p.e = max(-100, min(100, 21 - ilogb(xmax)));
+    p.e = max(-100, min(100, 28 - ilogb(xmax)));
     p.scale = (float)ldexp(1.0, p.e);
     // fixed-point phase of the light curve's own period: off by at most 2^-25 d of tau, half a
     // unit of 2^-40 c/d over T, and a few units of 2^-32 cycles
@@ -123,6 +126,7 @@ __device__ LcParams lc_params(uint64_t seed, int64_t j, const gpfc_synth_params 
     const unsigned long long G = (unsigned long long)__double2ll_rn(1099511627776.0 * freq);
     p.Gl = (uint32_t)G;
     p.Gh = (uint32_t)(G >> 32);
+    p.drift = (float)((freq - (double)G * 9.094947017729282e-13) * 0.00390625);
     p.off = (uint32_t)__double2ll_rn(p.epoch * freq * 4294967296.0);
     const double half = 0.5 * p.duration * freq;
     p.half = (uint32_t)__double2ll_rn(fmin(half, 0.5) * 4294967296.0);
@@ -164,18 +168,53 @@ __device__ __noinline__ long long tau_fp64(int i, double cadence)
     return __double2ll_rn(__dmul_rn(__dmul_rn((double)i, cadence), 16777216.0));
 }
 
+// sin(2 pi (u 2^-32 + du)), |du| small, as lead + mid + rest: u is reduced to within an eighth of a
+// cycle of a quarter; there the sine is a = 2 pi f and the cosine 1 - a^2 / 2, up to a rest below 0.1,
+// from the Taylor series (next terms below 2e-9 for |a| <= pi / 4).
+__device__ __forceinline__ void sin_cycles(uint32_t u, float du, float &lead, float &mid, float &rest)
+{
+    const uint32_t quarter = (u + (1u << 29)) >> 30;
+    const int32_t v = (int32_t)(u - (quarter << 30));
+    const int32_t vh = v & ~63;  // (24 bits: exact in FP32)
+    const float f = (float)vh * 2.3283064365386963e-10f, fl = fmaf((float)(v - vh), 2.3283064365386963e-10f, du);
+    const float a = 6.2831855f * f;
+    const float al = fmaf(6.2831855f, f, -a) + fmaf(-1.7484556e-7f, f, 6.2831855f * fl);
+    const float q = a * a;
+    // sin a - a, and cos a - (1 - q / 2) with what q is short of a^2
+    const float s = a * q * fmaf(q, fmaf(q, fmaf(q, 2.7557319e-6f, -1.9841270e-4f), 8.3333333e-3f), -0.16666667f);
+    const float c = fmaf(q * q, fmaf(q, fmaf(q, fmaf(q, -2.7557319e-7f, 2.4801587e-5f), -1.3888889e-3f), 4.1666667e-2f),
+                         -0.5f * fmaf(a, a, -q));
+    const bool cosine = quarter & 1u;
+    lead = cosine ? 1.f : a;
+    mid = cosine ? -0.5f * q : 0.f;
+    rest = cosine ? fmaf(-al, a + s, c) : fmaf(al, fmaf(-0.5f, q, 1.f + c), s);
+    if (quarter & 2u) {
+        lead = -lead;
+        mid = -mid;
+        rest = -rest;
+    }
+}
+
+// a + b as a pair (TwoSum)
+__device__ __forceinline__ float two_sum(float a, float b, float &e)
+{
+    const float s = a + b, bb = s - a;
+    e = (a - (s - bb)) + (b - bb);
+    return s;
+}
+
 // Threads per light curve: 256, so that several blocks share an SM and one's set-up overlaps
 // the others' samples; 1,024 where there are too few light curves to fill the SMs that way.
 constexpr int kSynthThreads = 256, kSynthWide = 1024;
 
-// Samples between emptyings of the 32-bit bin words and of a lane's squares (2,048 of 2^44 at most: a
-// warp's share of a whole light curve passes 2^64 from 2^24 cadences).
-constexpr int kSynthSpan = 1 << 19;
+// Samples between emptyings of the 32-bit bin words (|hi| <= 2^14 and lo < 2^15 a sample: sums up to
+// 2^31 and below 2^32) and of a lane's squares (512 of 2^52 at most).
+constexpr int kSynthSpan = 1 << 17;
 
 template <bool POW2, int THREADS>
 __global__ void __launch_bounds__(THREADS) synth_fold_kernel(SynthParams P, int shift)
 {
-    __shared__ uint32_t s_lo[256], s_hi[256], s_cnt[256];  // sum = hi 2^11 + lo, hi signed
+    __shared__ uint32_t s_lo[256], s_hi[256], s_cnt[256];  // sum = hi 2^15 + lo, hi signed
     __shared__ LcParams s_lp;
     __shared__ long long s_m1[8];
     __shared__ double s_m2[32];
@@ -197,7 +236,7 @@ __global__ void __launch_bounds__(THREADS) synth_fold_kernel(SynthParams P, int 
         const uint32_t step_i = lp.step_i, sfl = (uint32_t)lp.step_f, sfh = (uint32_t)(lp.step_f >> 32), tguard = lp.tguard;
         const uint64_t step20 = lp.step20;
         const float sigma = lp.sigma, scale = lp.scale;
-        double m2 = 0.0;                       // sum of squares of this lane's integers
+        double m2 = 0.0;                       // sum of squares of this lane's integers, over 2^6
         long long tot = 0;                     // bin tid: sum and count
         uint32_t cnt = 0u;
         for (int64_t span = 0; span < n; span += kSynthSpan) {
@@ -227,7 +266,7 @@ __global__ void __launch_bounds__(THREADS) synth_fold_kernel(SynthParams P, int 
                         const uint32_t fr = (uint32_t)tr & 0xFFFFFu;
                         if (!fixed || fr - tguard > 0xFFFFFu - 2u * tguard) tau = tau_fp64(i, P.sp.cadence);
                         const uint32_t tl = (uint32_t)(unsigned long long)tau, th = (uint32_t)((unsigned long long)tau >> 32);
-                        float x = sigma * (m ? rad * sn : rad * cs);
+                        float x = sigma * (m ? rad * sn : rad * cs), xl = 0.f;
                         if (kind != 1) {
                             const uint32_t ph = (uint32_t)(((unsigned long long)tl * Gl +
                                                             ((unsigned long long)(th * Gl + tl * Gh) << 32)) >> 32);
@@ -245,23 +284,31 @@ __global__ void __launch_bounds__(THREADS) synth_fold_kernel(SynthParams P, int 
                                     if (in) x -= lp.depth2;
                                 }
                             } else if (fixed) {
-                                // phase in cycles, with the part of the time below the unit of tau
+                                // phase with the part of the time below the unit of tau
                                 const float dt = (float)((int32_t)fr - (1 << 19)) * 9.5367431640625e-07f;
-                                x += lp.amp * sinpif(2.0f * fmaf(dt, lp.cyc, (float)su * 2.3283064365386963e-10f));
+                                const float t16 = (float)((th << 16) | (tl >> 16));  // tau / 2^16 < 2^26
+                                float lead, mid, rest, e0, e1;
+                                sin_cycles((uint32_t)su, fmaf(dt, lp.cyc, t16 * lp.drift), lead, mid, rest);
+                                // the products and their sum with what FP32 cuts off, xl
+                                const float p0 = lp.amp * lead, p1 = lp.amp * mid;
+                                x = two_sum(two_sum(p0, p1, e0), fmaf(lp.amp, rest, fmaf(lp.amp_lo, lead + mid, x)), e1);
+                                xl = (e0 + e1) + (fmaf(lp.amp, lead, -p0) + fmaf(lp.amp, mid, -p1));
                             } else {
                                 const double t = __dmul_rn((double)i, P.sp.cadence);
-                                x += (float)((double)lp.amp * sinpi(2.0 * (t - lp.epoch) / lp.period));
+                                x += (float)(((double)lp.amp + (double)lp.amp_lo) *
+                                             sinpi(2.0 * (t - lp.epoch) / lp.period));
                             }
                         }
-                        // rint(x 2^e): the sum with 3 2^22 has a unit in its last place of 1
-                        const int xq = __float_as_int(fmaf(x, scale, 12582912.0f)) - 0x4B400000;
-                        sq += (unsigned long long)((long long)xq * (long long)xq);
+                        int xq = __float2int_rn(x * scale);
+                        if (kind == 2) xq += __float2int_rn(xl * scale);
+                        const int x26 = (xq + 4) >> 3;
+                        sq += (unsigned long long)((long long)x26 * (long long)x26);
                         const unsigned long long phi = (unsigned long long)tl * Fl +
                                                        ((unsigned long long)(th * Fl + tl * Fh) << 32);
                         const uint32_t bin = POW2 ? (uint32_t)(phi >> 32) >> shift
                                                   : (uint32_t)__umul64hi(phi, (unsigned long long)nb);
-                        atomicAdd(&s_lo[bin], (uint32_t)xq & 2047u);
-                        atomicAdd(&s_hi[bin], (uint32_t)(xq >> 11));
+                        atomicAdd(&s_lo[bin], (uint32_t)xq & 32767u);
+                        atomicAdd(&s_hi[bin], (uint32_t)(xq >> 15));
                         atomicAdd(&s_cnt[bin], 1u);
                     }
                 }
@@ -269,7 +316,7 @@ __global__ void __launch_bounds__(THREADS) synth_fold_kernel(SynthParams P, int 
             m2 += (double)sq;
             __syncthreads();
             if (tid < nb) {
-                tot += ((long long)(int32_t)s_hi[tid] << 11) + (long long)s_lo[tid];
+                tot += ((long long)(int32_t)s_hi[tid] << 15) + (long long)s_lo[tid];
                 cnt += s_cnt[tid];
                 s_lo[tid] = s_hi[tid] = s_cnt[tid] = 0u;
             }
@@ -298,7 +345,7 @@ __global__ void __launch_bounds__(THREADS) synth_fold_kernel(SynthParams P, int 
                 for (int w = 0; w < min(nw, 8); ++w) a += s_m1[w];
                 for (int w = 0; w < nw; ++w) b2 += s_m2[w];
                 const double nn = (double)n, mu = (double)a / nn;
-                P.sigma_out[q] = (float)(sqrt(fmax(b2 / nn - mu * mu, 0.0)) * unit);
+                P.sigma_out[q] = (float)(sqrt(fmax(64.0 * b2 / nn - mu * mu, 0.0)) * unit);
             }
         }
         if (tid == 0 && P.label) P.label[q] = kind == 0 ? 1.f : 0.f;

@@ -48,3 +48,30 @@ def test_flux_std_does_not_depend_on_the_batch(ctx, n_cad, nbins):
         one = g.gpfc_synth_profiles(ctx, 9, 40 + j, 1, nbins, sp, want_std=True)[4]
         ctx.sync()
         assert abs(float(one[0]) / float(many[j]) - 1.0) <= 2.0 ** -23
+
+
+# noise of a few parts in ten, deep signals on quiet stars, few samples a bin. Off by at most half a
+# unit in the last place of a mean between 1 and 2 and one rounding of the largest sample
+@pytest.mark.parametrize("sigma,depth,n_cad", [((0.05, 0.3), (3e-5, 2e-3), 20000), ((1e-7, 1e-6), (0.3, 0.9), 400),
+                                               ((1e-4, 1e-3), (0.3, 0.9), 6000)])
+def test_generated_profiles_of_wide_ranges(ctx, sigma, depth, n_cad):
+    import paper_2312_02063_gb300 as g
+    sp = dict(lcsynth.TRAINING_SET, n_cadences=n_cad, sigma_min=sigma[0], sigma_max=sigma[1], depth_min=depth[0],
+              depth_max=depth[1])
+    f, c, _, per, std = g.gpfc_synth_profiles(ctx, 31, 0, 36, 256, sp, want_period=True, want_std=True)
+    ctx.sync()
+    f, c, per, std = (x.cpu().numpy() for x in (f, c, per, std))
+    err = []
+    for j in range(36):
+        t, flux, _, P = lcsynth.training_light_curve(31, j, sp)
+        assert per[j] == P
+        b = oracle.bins(oracle.quantise_times(t, 0.0), oracle.quantise_periods(np.array([P])), 256)[0]
+        cnt = np.bincount(b, minlength=256)
+        np.testing.assert_array_equal(c[j], cnt)
+        nz = cnt > 0
+        mean = 1.0 + np.bincount(b, weights=flux - 1.0, minlength=256)[nz] / cnt[nz]
+        e = np.abs(f[j][nz].astype(np.float64) - mean)
+        assert e.max() <= 2.0 ** -24 + 2.0 ** -25 * np.abs(flux - 1.0).max(), j
+        err.append(e)
+        assert abs(std[j] / np.std(flux) - 1.0) <= 2.0 ** -22
+    assert np.sqrt((np.concatenate(err) ** 2).mean()) <= 2.0 ** -23 / 12 ** 0.5
