@@ -39,6 +39,7 @@ struct gpfc_ctx {
     };
     std::vector<Tuned> tuned;
     bool autotune = true;
+    int peak_clusters = 0;  // clusters of the decision's blocks that the device holds at a time
     // CUDA graph of the last batched search, replayed when the same call comes again
     bool use_graph = true;
     cudaStream_t cap_stream = nullptr;
@@ -1393,6 +1394,7 @@ int gpfc_create(gpfc_ctx **out, int device, void *stream)
     }
     if (e == cudaSuccess) e = static_cast<cudaError_t>(fold_register_kernels());
     if (e == cudaSuccess) e = static_cast<cudaError_t>(fold_pack_register());
+    if (e == cudaSuccess) ctx->peak_clusters = peaks_register();
     int prio_least = 0, prio_greatest = 0;
     if (e == cudaSuccess) e = cudaDeviceGetStreamPriorityRange(&prio_least, &prio_greatest);
     if (e == cudaSuccess) e = cudaStreamCreateWithPriority(&ctx->side[0], cudaStreamNonBlocking, prio_greatest);
@@ -2004,7 +2006,7 @@ int gpfc_peaks(gpfc_ctx *ctx, const float *score, const double *periods, int32_t
     p.summary = reinterpret_cast<PeakSummaryDev *>(summary);
     p.peaks = max_peaks > 0 ? reinterpret_cast<PeakDev *>(peaks) : nullptr;
     KernelTimer timer(ctx);
-    cudaError_t e = launch_peaks(p, ctx->num_sms, ctx->stream);
+    cudaError_t e = launch_peaks(p, ctx->num_sms, ctx->peak_clusters, ctx->stream);
     if (e != cudaSuccess) return cuda_err(ctx, e, "decision kernel");
     timer.stop();
     return GPFC_OK;

@@ -39,7 +39,10 @@ struct PeakParams {
     PeakDev *peaks;           // [S][max_peaks] or NULL
 };
 
-cudaError_t launch_peaks(const PeakParams &p, int num_sms, cudaStream_t st);
+// Allow the cluster kernel on the current device (function attributes are a device's own): how many
+// clusters it holds at a time, 0 if it cannot run there.
+int peaks_register();
+cudaError_t launch_peaks(const PeakParams &p, int num_sms, int clusters, cudaStream_t st);
 
 // Detection statistics of a detector on labelled scores (gpfc_roc).
 constexpr int kRocMaxFpr = 16;

@@ -24,6 +24,22 @@ def _dev(ctx, a):
     return torch.from_numpy(np.ascontiguousarray(a)).to(ctx.device)
 
 
+def _ms(ctx, call, reps=5):
+    """Least time of a call, after two warm-up calls."""
+    for _ in range(2):
+        call()
+    ctx.sync()
+    a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+    best = float("inf")
+    for _ in range(reps):
+        a.record()
+        call()
+        b.record()
+        torch.cuda.synchronize()
+        best = min(best, a.elapsed_time(b))
+    return best
+
+
 # ---------------------------------------------------------------- generated profiles
 
 def test_flux_std_of_a_long_sinusoid(ctx):
@@ -75,3 +91,17 @@ def test_generated_profiles_of_wide_ranges(ctx, sigma, depth, n_cad):
         err.append(e)
         assert abs(std[j] / np.std(flux) - 1.0) <= 2.0 ** -22
     assert np.sqrt((np.concatenate(err) ** 2).mean()) <= 2.0 ** -23 / 12 ** 0.5
+
+
+def test_decision_of_several_stars_takes_no_longer_than_of_many(ctx):
+    """19 stars of 16,384 periods: a block each, not clusters that take turns."""
+    import paper_2312_02063_gb300 as g
+    rng = np.random.default_rng(6)
+    n = 16384
+
+    def of(stars):
+        s = _dev(ctx, rng.normal(0, 1, stars * n).astype(np.float32))
+        p = _dev(ctx, np.tile(np.linspace(0.2, 30.0, n), stars))
+        off = _dev(ctx, (np.arange(stars + 1) * n).astype(np.int64))
+        return _ms(ctx, lambda: g.gpfc_peaks(ctx, s, p, off, max_peaks=4), reps=20)
+    assert of(19) <= 1.25 * of(60)
