@@ -2046,6 +2046,7 @@ int gpfc_detrend(gpfc_ctx *ctx, const double *times, const float *flux, const ui
     int rc = take_latched(ctx);
     if (rc) return rc;
     const int G = (int)std::min<int64_t>(4 * (int64_t)ctx->num_sms, std::max<int64_t>(1, (n + 2047) / 2048));
+    p.group = (int)std::min<size_t>(p.n_sp, std::max<size_t>(1, kDtScratch / (kDtPointBytes * n)));
     auto carve = [&](void *base) {
         Carver c(base);
         p.partial = c.take<double>(2 * G);
@@ -2055,20 +2056,16 @@ int gpfc_detrend(gpfc_ctx *ctx, const double *times, const float *flux, const ui
         p.seg_start = c.take<int64_t>(n + 1);
         p.seg_keep = c.take<int64_t>(n);
         p.seg_off = c.take<int64_t>(n);
-        const size_t k = (size_t)p.n_sp * n;
+        const size_t k = (size_t)p.group * n;
         p.basis = c.take<double4>(k);
         p.interval = c.take<int32_t>(k);
-        p.first = c.take<int32_t>(k + p.n_sp + 1);
-        p.inv6 = c.take<double>(6 * k);
-        p.part14 = c.take<double>(14 * k);
-        p.G4 = c.take<double>(4 * k);
-        p.LB = c.take<double>(4 * k);
+        p.first = c.take<int32_t>(k + p.group + 1);
+        p.band = c.take<double>(8 * k);
         p.rhs = c.take<double>(k);
         p.coef = c.take<double>(k);
-        p.trend = c.take<double>(k);
         p.used = c.take<uint8_t>(k);
         p.used2 = c.take<uint8_t>(k);
-        p.bic = c.take<double>(k);
+        for (double *&q : p.best) q = p.group < p.n_sp ? c.take<double>(n) : nullptr;
         p.det = c.take<float>(n);
         return c.off + 256;
     };

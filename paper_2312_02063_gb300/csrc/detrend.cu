@@ -22,8 +22,10 @@
 //
 // Layout: every per-point scratch array is indexed by the point's own index, and a
 // segment's p <= n_s coefficients live at the indices of its own points, so segments
-// never share scratch; each candidate spacing has its own copy. Every reduction runs in a
-// fixed order: the results do not depend on scheduling.
+// never share scratch; each candidate spacing fitted at the same time has its own copy, 122 bytes a
+// point (arrays whose lifetimes do not meet share it). Spacings go through in groups of as many
+// copies as kDtScratch holds, one at least. Every reduction runs in a fixed order: the results do
+// not depend on scheduling or grouping.
 //
 // What bounds it: FP64 instructions, one per warp and scheduler every 64 cycles whatever the
 // number of active lanes, and the serial factorisation. So each (segment, spacing) is a block of
@@ -182,6 +184,13 @@ __device__ __forceinline__ double dt_rcp(double d)
     return x;
 }
 
+// BIC of the segment that starts at point a with the group's spacing c (infinite: skipped), in the
+// place of its matrix, which is done with.
+__device__ __forceinline__ double &dt_bic(const DetrendParams &p, int c, int64_t a)
+{
+    return p.band[8 * ((size_t)c * p.n + a)];
+}
+
 // One end's elimination state: the last three rows' pivots and multipliers.
 // A row i of a symmetric band matrix (half width 3), left-looking: with the eliminated rows i - k,
 //   c_k = g(i, i-k) - sum over eliminated columns left of it,  l_k = c_k / d_{i-k},
@@ -334,33 +343,40 @@ __device__ bool dt_solve(double *G, double *r, double *L, double *x, int n, int 
     return true;
 }
 
-// The clipped fit of one segment with one knot spacing: a block each.
+// Knot intervals whose sums a block holds at a time: enough for most segments (a quarter of a
+// mission at half a day); longer ones go through in tiles, three intervals summed again for each.
+constexpr int kDtRows = kDtThreads;
+
+// The clipped fit of one segment with one knot spacing (of the group's): a block each.
 __global__ void __launch_bounds__(kDtThreads) dt_fit_kernel(DetrendParams p)
 {
+    __shared__ double s_part[14 * (kDtRows + 3)];
     __shared__ double red[kDtThreads / 32];
     __shared__ int s_m, s_ok, s_changed, s_cnt[kDtThreads / 32];
     __shared__ double s_lambda;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int64_t nseg = *p.n_seg;
-    for (int64_t item = blockIdx.x; item < nseg * p.n_sp; item += gridDim.x) {
-        const int64_t s = item / p.n_sp;
-        const int c = (int)(item - s * p.n_sp);
+    for (int64_t item = blockIdx.x; item < nseg * p.group; item += gridDim.x) {
+        const int64_t s = item / p.group;
+        const int c = (int)(item - s * p.group);
         const int64_t a = p.seg_start[s], b = p.seg_start[s + 1];
         const int ns = (int)(b - a);
+        const size_t o = (size_t)c * p.n + a;  // this candidate's copy of the segment's scratch
         if (ns <= 2 * (int64_t)p.edge) {
-            if (tid == 0) p.bic[(size_t)c * p.n + s] = INFINITY;
+            if (tid == 0) dt_bic(p, c, a) = INFINITY;
             continue;
         }
         const double *t = p.t + a;
         const float *f = p.f + a;
-        const size_t o = (size_t)c * p.n + a;  // this candidate's copy of the segment's scratch
         double4 *N = p.basis + o;
-        double *iv = p.inv6 + 6 * o, *P14 = p.part14 + 14 * o, *G = p.G4 + 4 * o, *LB = p.LB + 4 * o;
-        double *rhs = p.rhs + o, *coef = p.coef + o, *trend = p.trend + o;
+        // the knot intervals' reciprocal differences (at most ns - 3 intervals of 6) are used up before
+        // the matrix is formed, its factor before the fit is evaluated
+        double *G = p.band + 8 * o, *LB = G + 4 * (size_t)ns, *iv = G, *trend = LB;
+        double *rhs = p.rhs + o, *coef = p.coef + o;
         int32_t *iv_of = p.interval + o, *first = p.first + o + (int64_t)c;  // [intervals + 1] <= ns + 1
         uint8_t *used = p.used + o, *used2 = p.used2 + o;
         const double t0 = t[0], t1 = t[ns - 1];
-        const double sp = p.sp[c], inv_sp = 1.0 / sp;
+        const double sp = p.sp[p.sp0 + c], inv_sp = 1.0 / sp;
         __syncthreads();  // every thread has left the previous item
         if (tid == 0) {
             // interior knots t0 + sp i < t1 (at most 2^30, and no more than make ns coefficients
@@ -425,23 +441,6 @@ __global__ void __launch_bounds__(kDtThreads) dt_fit_kernel(DetrendParams p)
                 for (int i = tid; i < ns; i += kDtThreads) cu += used[i];
                 cu = __reduce_add_sync(0xffffffffu, cu);
                 if (lane == 0) s_cnt[warp] = cu;
-                // an interval's sums over its used points: N_x N_y (x <= y) and N_x f
-                for (int e = tid; e < 14 * (m + 1); e += kDtThreads) {
-                    const int j = e / 14, k = e - 14 * j;
-                    const int i0 = first[j], i1 = first[j + 1];
-                    const int x = k < 4 ? 0 : (k < 7 ? 1 : (k < 9 ? 2 : (k < 10 ? 3 : k - 10)));
-                    const int y = k < 4 ? k : (k < 7 ? k - 3 : (k < 9 ? k - 5 : 3));
-                    const double *Nd = reinterpret_cast<const double *>(N);
-                    double acc = 0.0;
-                    if (k < 10) {
-                        for (int i = i0; i < i1; ++i)
-                            if (used[i]) acc = fma(Nd[4 * (size_t)i + x], Nd[4 * (size_t)i + y], acc);
-                    } else {
-                        for (int i = i0; i < i1; ++i)
-                            if (used[i]) acc = fma(Nd[4 * (size_t)i + x], (double)f[i], acc);
-                    }
-                    P14[e] = acc;
-                }
                 __syncthreads();
                 int nused = 0;
                 for (int w = 0; w < kDtThreads / 32; ++w) nused += s_cnt[w];
@@ -449,22 +448,45 @@ __global__ void __launch_bounds__(kDtThreads) dt_fit_kernel(DetrendParams p)
                     valid = false;
                     break;
                 }
-                // rows of the normal equations from the intervals they reach over (B_r is the q-th
-                // spline of interval r - q), and the trace
                 double tr = 0.0;
-                for (int r = tid; r < np_; r += kDtThreads) {
-                    double g[4] = {0.0, 0.0, 0.0, 0.0}, v = 0.0;
-                    for (int q = 3; q >= 0; --q) {
-                        const int j = r - q;
-                        if (j < 0 || j > m) continue;
-                        const double *w = P14 + 14 * (size_t)j;
-                        const int at = q == 0 ? 0 : (q == 1 ? 4 : (q == 2 ? 7 : 9));
-                        for (int d = 0; q + d <= 3; ++d) g[d] += w[at + d];
-                        v += w[10 + q];
+                for (int r0 = 0; r0 < np_; r0 += kDtRows) {
+                    // an interval's sums over its used points: N_x N_y (x <= y) and N_x f
+                    const int j0 = max(0, r0 - 3), j1 = min(m + 1, r0 + kDtRows);
+                    for (int e = tid; e < 14 * (j1 - j0); e += kDtThreads) {
+                        const int j = j0 + e / 14, k = e % 14;
+                        const int i0 = first[j], i1 = first[j + 1];
+                        const int x = k < 4 ? 0 : (k < 7 ? 1 : (k < 9 ? 2 : (k < 10 ? 3 : k - 10)));
+                        const int y = k < 4 ? k : (k < 7 ? k - 3 : (k < 9 ? k - 5 : 3));
+                        const double *Nd = reinterpret_cast<const double *>(N);
+                        double acc = 0.0;
+                        if (k < 10) {
+                            for (int i = i0; i < i1; ++i)
+                                if (used[i]) acc = fma(Nd[4 * (size_t)i + x], Nd[4 * (size_t)i + y], acc);
+                        } else {
+                            for (int i = i0; i < i1; ++i)
+                                if (used[i]) acc = fma(Nd[4 * (size_t)i + x], (double)f[i], acc);
+                        }
+                        s_part[e] = acc;
                     }
-                    for (int d = 0; d < 4; ++d) G[4 * (size_t)r + d] = g[d];
-                    rhs[r] = v;
-                    tr += g[0];
+                    __syncthreads();
+                    // rows of the normal equations from the intervals they reach over (B_r is the q-th
+                    // spline of interval r - q), and the trace
+                    const int r = r0 + tid;
+                    if (r < np_) {
+                        double g[4] = {0.0, 0.0, 0.0, 0.0}, v = 0.0;
+                        for (int q = 3; q >= 0; --q) {
+                            const int j = r - q;
+                            if (j < 0 || j > m) continue;
+                            const double *w = s_part + 14 * (j - j0);
+                            const int at = q == 0 ? 0 : (q == 1 ? 4 : (q == 2 ? 7 : 9));
+                            for (int d = 0; q + d <= 3; ++d) g[d] += w[at + d];
+                            v += w[10 + q];
+                        }
+                        for (int d = 0; d < 4; ++d) G[4 * (size_t)r + d] = g[d];
+                        rhs[r] = v;
+                        tr += g[0];
+                    }
+                    __syncthreads();  // the sums are read before the next rows' replace them
                 }
                 const double trace = dt_block_sum(tr, red);
                 if (tid == 0) s_lambda = p.ridge * trace / (double)np_;
@@ -530,13 +552,14 @@ __global__ void __launch_bounds__(kDtThreads) dt_fit_kernel(DetrendParams p)
                 __syncthreads();
             }
         }
-        if (tid == 0) p.bic[(size_t)c * p.n + s] = valid ? bic : INFINITY;
+        if (tid == 0) dt_bic(p, c, a) = valid ? bic : INFINITY;
     }
 }
 
-// The spacing of each segment, and the light curve over its fit: kDtParts blocks a segment.
+// The spacing of each segment (of this group's and the best of the groups before, bic_in, or NULL)
+// and the light curve over its fit: kDtParts blocks a segment.
 constexpr int kDtParts = 8;
-__global__ void __launch_bounds__(kDtThreads) dt_choose_kernel(DetrendParams p)
+__global__ void __launch_bounds__(kDtThreads) dt_choose_kernel(DetrendParams p, const double *bic_in, double *bic_out)
 {
     const int64_t nseg = *p.n_seg;
     for (int64_t item = blockIdx.x; item < nseg * kDtParts; item += gridDim.x) {
@@ -544,19 +567,23 @@ __global__ void __launch_bounds__(kDtThreads) dt_choose_kernel(DetrendParams p)
         const int part = (int)(item - s * kDtParts);
         const int64_t a = p.seg_start[s], b = p.seg_start[s + 1], ns = b - a;
         int best = -1;
-        double bic = INFINITY;
-        for (int c = 0; c < p.n_sp; ++c) {
-            const double v = p.bic[(size_t)c * p.n + s];
+        double bic = bic_in ? bic_in[s] : INFINITY;
+        for (int c = 0; c < p.group; ++c) {
+            const double v = dt_bic(p, c, a);
             if (v < bic) {
                 bic = v;
                 best = c;
             }
         }
-        const double *trend = p.trend + (size_t)max(best, 0) * p.n;
-        const int64_t i1 = a + ns * (part + 1) / kDtParts;
-        for (int64_t i = a + ns * part / kDtParts + threadIdx.x; i < i1; i += kDtThreads)
-            p.det[i] = best >= 0 ? (float)((double)p.f[i] / trend[i]) : 0.f;
-        if (part == 0 && threadIdx.x == 0) p.seg_keep[s] = best >= 0 ? ns - 2 * (int64_t)p.edge : 0;
+        const double *trend = p.band + 8 * ((size_t)max(best, 0) * p.n + a) + 4 * (size_t)ns;
+        const int64_t i1 = ns * (part + 1) / kDtParts;
+        if (best >= 0 || !bic_in)
+            for (int64_t i = ns * part / kDtParts + threadIdx.x; i < i1; i += kDtThreads)
+                p.det[a + i] = best >= 0 ? (float)((double)p.f[a + i] / trend[i]) : 0.f;
+        if (part == 0 && threadIdx.x == 0) {
+            if (bic_out) bic_out[s] = bic;
+            p.seg_keep[s] = bic < INFINITY ? ns - 2 * (int64_t)p.edge : 0;
+        }
     }
 }
 
@@ -597,8 +624,14 @@ cudaError_t launch_detrend(const DetrendParams &p, int num_sms, cudaStream_t st)
     dt_scan_kernel<<<1, 32, 0, st>>>(p.blk_count, G, p.blk_off, p.n_seg);
     dt_starts_kernel<<<G, kDtThreads, 0, st>>>(p, 2);
     dt_close_starts_kernel<<<1, 32, 0, st>>>(p);
-    dt_fit_kernel<<<num_sms * 4, kDtThreads, 0, st>>>(p);
-    dt_choose_kernel<<<num_sms * 4, kDtThreads, 0, st>>>(p);
+    for (int c = 0, turn = 0; c < p.n_sp; c += p.group, ++turn) {
+        DetrendParams q = p;
+        q.sp0 = c;
+        q.group = p.n_sp - c < p.group ? p.n_sp - c : p.group;
+        dt_fit_kernel<<<num_sms * 4, kDtThreads, 0, st>>>(q);
+        dt_choose_kernel<<<num_sms * 4, kDtThreads, 0, st>>>(q, c > 0 ? p.best[turn & 1] : nullptr,
+                                                             p.best[(turn + 1) & 1]);
+    }
     dt_offsets_kernel<<<1, 32, 0, st>>>(p);
     dt_write_kernel<<<num_sms * 2, kDtThreads, 0, st>>>(p);
     return cudaGetLastError();

@@ -26,15 +26,16 @@ struct DetrendParams {
     int64_t *seg_start;     // [n + 1]
     int64_t *seg_keep;      // [n]
     int64_t *seg_off;       // [n]
-    // one copy per candidate spacing, [n_sp][n]: a point's four B-splines and its knot interval,
-    // the first point of each interval [n + 1], and per interval or coefficient (at its segment's
-    // points) the reciprocal knot differences [6], the 14 sums of the normal equations, the banded
-    // matrix [4], its factor [4], right side and solution
+    // one copy per candidate spacing of a group, [group][n]: a point's four B-splines and its knot
+    // interval, the first point of each interval [n + 1], and per interval or coefficient (at its
+    // segment's points) the reciprocal knot differences [6], in whose place come the banded matrix
+    // [4] and its factor [4], then the segment's BIC and the fit; right side and solution
+    int sp0, group;
     double4 *basis;
     int32_t *interval, *first;
-    double *inv6, *part14, *G4, *LB, *rhs, *coef, *trend;
+    double *band, *rhs, *coef;
     uint8_t *used, *used2;
-    double *bic;            // [n_sp][n]: by segment (infinite: the candidate was skipped)
+    double *best[2];        // [n]: smallest BIC of the segments so far, in turn (one group: NULL)
     float *det;             // [n]
     // outputs (caller-owned, device)
     double *t_out;
@@ -42,6 +43,10 @@ struct DetrendParams {
     int32_t *seg_out;       // or NULL
     int64_t *n_out;         // [1]
 };
+
+// Scratch of the spacings fitted at the same time: bytes per point of each, and their sum where more
+// than one is.
+constexpr size_t kDtPointBytes = 122, kDtScratch = (size_t)1 << 30;
 
 cudaError_t launch_detrend(const DetrendParams &p, int num_sms, cudaStream_t st);
 

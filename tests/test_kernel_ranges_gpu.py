@@ -105,3 +105,47 @@ def test_decision_of_several_stars_takes_no_longer_than_of_many(ctx):
         off = _dev(ctx, (np.arange(stars + 1) * n).astype(np.int64))
         return _ms(ctx, lambda: g.gpfc_peaks(ctx, s, p, off, max_peaks=4), reps=20)
     assert of(19) <= 1.25 * of(60)
+
+
+# ---------------------------------------------------------------- detrending
+
+def test_detrending_workspace_and_spacings_in_groups(ctx):
+    """1.2 million samples with eight spacings: the spacings go through in groups. The halves, each in one
+    group, give the same bits (no flux gap; the cut lies at a time gap), and the workspace stays near 1 GiB."""
+    import paper_2312_02063_gb300 as g
+    rng = np.random.default_rng(8)
+    n = 1200000
+    t = np.arange(n) * CADENCE + 4.0 * (np.arange(n) // 1500)
+    f = _dev(ctx, (1.0 + 1e-3 * np.sin(t / 2.0) + rng.normal(0, 2e-4, n)).astype(np.float32))
+    t = _dev(ctx, t)
+    kw = dict(edge=5, flux_gap_sigma=1e9, spacings=[0.4, 0.5, 0.7, 1.0, 1.5, 2.0, 3.0, 5.0], max_iter=3)
+    fresh = g.Context(0)
+    try:
+        torch.cuda.synchronize()
+        before = torch.cuda.mem_get_info()[0]
+        whole = g.gpfc_detrend(fresh, t, f, None, **kw)
+        fresh.sync()
+        held = before - torch.cuda.mem_get_info()[0]
+        whole = [x.clone() for x in whole]
+        assert held <= 1.5 * 2 ** 30  # (1 GiB, an eighth more, 44 bytes a sample and the outputs)
+        h = n // 2
+        parts = [g.gpfc_detrend(fresh, t[a:a + h].contiguous(), f[a:a + h].contiguous(), None, **kw) for a in (0, h)]
+        fresh.sync()
+        for i in range(2):
+            assert torch.equal(whole[i], torch.cat([p[i] for p in parts]))
+    finally:
+        fresh.close()
+
+
+def test_detrending_of_a_segment_longer_than_a_tile_of_intervals(ctx):
+    """One segment with 571 and 142 knot intervals (a block sums 256 at a time) against the oracle."""
+    import paper_2312_02063_gb300 as g
+    rng = np.random.default_rng(9)
+    n = 7000
+    t = np.arange(n) * CADENCE
+    f = (1.0 + 1e-3 * np.sin(t / 3.0) + 3e-4 * np.sin(t * 4.0) + rng.normal(0, 1e-4, n)).astype(np.float32)
+    to, fo, _ = g.gpfc_detrend(ctx, _dev(ctx, t), _dev(ctx, f), None, spacings=[0.25, 1.0])
+    ctx.sync()
+    r = oracle.detrend(t, f, None, spacings=(0.25, 1.0))
+    np.testing.assert_array_equal(to.cpu().numpy(), r["times"])
+    assert (np.abs(fo.cpu().numpy().astype(np.float64) / r["flux"] - 1.0)).max() <= 2e-7
