@@ -39,6 +39,7 @@ struct gpfc_ctx {
     };
     std::vector<Tuned> tuned;
     bool autotune = true;
+    uint32_t window = 0;    // shared address at which a block's dynamic memory starts
     int peak_clusters = 0;  // clusters of the decision's blocks that the device holds at a time
     // CUDA graph of the last batched search, replayed when the same call comes again
     bool use_graph = true;
@@ -160,9 +161,10 @@ struct FoldPlan {
 // a sample at one warp instruction per 64 cycles, takes 40 us a block at 8,192).
 int prep_groups(int64_t n) { return (int)std::min<int64_t>(256, std::max<int64_t>(1, (n + 1023) / 1024)); }
 
-cudaError_t launch_plan(const FoldPlan &pl, const FoldParams &p, int grid, cudaStream_t st)
+cudaError_t launch_plan(const gpfc_ctx *ctx, const FoldPlan &pl, const FoldParams &p, int grid, cudaStream_t st,
+                        int mode = kModeFold)
 {
-    return pl.packed ? launch_fold_pack(p, grid, st) : launch_fold(p, kModeFold, grid, st);
+    return pl.packed ? launch_fold_pack(p, ctx->window, grid, st) : launch_fold(p, mode, grid, st);
 }
 
 // At 256 bins and more the reduction layout: its updates need no load, so three period
@@ -203,7 +205,7 @@ bool pack_ok(const gpfc_ctx *ctx, int nbins)
     const gpfc_fold_config &c = ctx->fold_cfg;
     return default_layout(nbins) == kLayoutRed32 && (c.layout == 0 || c.layout == kLayoutRed32) && c.warps == 0 &&
            c.chunk == 0 && c.tile == 0 && c.blocks_per_sm == 0 && c.streams == 0 &&
-           fold_max_warps(nbins, kLayoutRed32, kTile) >= 1 && fold_pack_groups(nbins) >= 1;
+           fold_max_warps(nbins, kLayoutRed32, kTile) >= 1 && fold_pack_groups(nbins, ctx->window) >= 1;
 }
 
 // Below 256 bins the one-word fold takes the place of the FP32 layouts, with flux in 31 bits, where
@@ -232,7 +234,7 @@ FoldPlan plan_packed(const gpfc_ctx *ctx, int64_t n, int64_t np, int nbins, int6
     pl.bps = 1;
     const int64_t per_sm = (np + (int64_t)32 * ctx->num_sms - 1) / ((int64_t)32 * ctx->num_sms);
     const int maxg =
-        fold_pack_allowed(nbins, (int)std::max<int64_t>(1, std::min<int64_t>(fold_pack_groups(nbins), per_sm)));
+        fold_pack_allowed(nbins, (int)std::max<int64_t>(1, std::min<int64_t>(fold_pack_groups(nbins, ctx->window), per_sm)));
     pl.warps = maxg;
     if (nstars > 1) {
         const int64_t avg = std::max<int64_t>(1, np / nstars);
@@ -570,7 +572,7 @@ int run_fold(gpfc_ctx *ctx, const double *times, const float *flux, int64_t n, c
         if (e != cudaSuccess) return cuda_err(ctx, e, "cudaMemsetAsync");
     }
     KernelTimer timer(ctx);
-    e = pl.packed ? launch_fold_pack(p, pl.grid, ctx->stream) : launch_fold(p, mode, pl.grid, ctx->stream);
+    e = launch_plan(ctx, pl, p, pl.grid, ctx->stream, mode);
     if (e != cudaSuccess) return cuda_err(ctx, e, "fold kernel");
     timer.stop();
     if (out_fb) *out_fb = fb;
@@ -812,7 +814,7 @@ int run_search_box_warp(gpfc_ctx *ctx, const double *times, const float *flux, i
         p.counts = cc[b];
         p.status = ctx->status_dev;
         const int grid = chunk_shape(ctx, pl, nk, p);
-        return timed_fold(ctx, sf, [&] { return launch_plan(pl, p, grid, sf); });
+        return timed_fold(ctx, sf, [&] { return launch_plan(ctx, pl, p, grid, sf); });
     };
     auto box = [&](int64_t i, int b, cudaStream_t sb) {
         const int64_t k0 = i * chunk, nk = std::min<int64_t>(chunk, np - k0);
@@ -921,7 +923,7 @@ int run_search_cnn(gpfc_ctx *ctx, const double *times, const float *flux, int64_
         p.counts = cc[b];
         p.status = ctx->status_dev;
         const int grid = chunk_shape(ctx, pl, nk, p);
-        return launch_plan(pl, p, grid, sf);
+        return launch_plan(ctx, pl, p, grid, sf);
     };
     auto cnn = [&](int64_t i, int b, cudaStream_t sb) {
         const int64_t k0 = i * chunk, nk = std::min<int64_t>(chunk, np - k0);
@@ -1051,7 +1053,7 @@ int tune_fold(gpfc_ctx *ctx, const double *times, const float *flux, int64_t n, 
             p.w_max = bp->w_max;
             p.sigma_user = bp->sigma > 0.0 ? (float)bp->sigma : 0.f;
         }
-        auto fold = [&] { return pl.packed ? launch_fold_pack(p, pl.grid, ctx->stream) : launch_fold(p, mode, pl.grid, ctx->stream); };
+        auto fold = [&] { return launch_plan(ctx, pl, p, pl.grid, ctx->stream, mode); };
         e = fold();  // warm-up
         if (e == cudaSuccess) e = cudaEventRecord(ctx->ev_start, ctx->stream);
         for (int r = 0; r < 2 && e == cudaSuccess; ++r) e = fold();
@@ -1221,7 +1223,7 @@ cudaError_t enqueue_batched(gpfc_ctx *ctx, const BatchArgs &A, const FoldPlan &p
             q.slot_k = B.chunk_k[b];
             q.task_begin = i * wave;
             q.ntasks = std::min<int64_t>(T, q.task_begin + wave);
-            return launch_plan(pl, q, (int)(q.ntasks - q.task_begin), sf);
+            return launch_plan(ctx, pl, q, (int)(q.ntasks - q.task_begin), sf);
         };
         auto box = [&](int64_t i, int b, cudaStream_t sb) {
             const int64_t tb = i * wave, te = std::min<int64_t>(T, tb + wave);
@@ -1271,7 +1273,7 @@ cudaError_t enqueue_batched(gpfc_ctx *ctx, const BatchArgs &A, const FoldPlan &p
         q.slot_k = B.chunk_k[b];
         q.task_begin = i * wave;
         q.ntasks = std::min<int64_t>(T, q.task_begin + wave);
-        return launch_plan(pl, q, (int)(q.ntasks - q.task_begin), sf);
+        return launch_plan(ctx, pl, q, (int)(q.ntasks - q.task_begin), sf);
     };
     auto cnn = [&](int64_t i, int b, cudaStream_t sb) {
         const int64_t tb = i * wave, te = std::min<int64_t>(T, tb + wave);
@@ -1394,6 +1396,9 @@ int gpfc_create(gpfc_ctx **out, int device, void *stream)
     }
     if (e == cudaSuccess) e = static_cast<cudaError_t>(fold_register_kernels());
     if (e == cudaSuccess) e = static_cast<cudaError_t>(fold_pack_register());
+    int reserved = 0;  // (the driver's own shared memory comes first in a block's)
+    if (e == cudaSuccess) e = cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, device);
+    ctx->window = (uint32_t)reserved;
     if (e == cudaSuccess) ctx->peak_clusters = peaks_register();
     int prio_least = 0, prio_greatest = 0;
     if (e == cudaSuccess) e = cudaDeviceGetStreamPriorityRange(&prio_least, &prio_greatest);

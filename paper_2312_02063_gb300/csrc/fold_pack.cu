@@ -55,7 +55,6 @@ constexpr int kPackTile = kMaxTile;        // 2048 samples
 constexpr uint32_t kSlab = 65536;          // 256 bins: two period groups, 256-byte rows
 constexpr uint32_t kSlabPhase = 0x9000;    // slabs start at this offset from a multiple of 64 KB
 constexpr uint32_t kHdrBytes = 128 + 4 * kPackTile * 4 + 2 * (kPackTile / 16) * 4 + kPackMaxGroups * 32 * 4;
-constexpr uint32_t kWindow = 1024;         // shared addresses of a block's dynamic memory start here
 
 struct PackShared {
     uint64_t bars[2];
@@ -180,7 +179,7 @@ __global__ void __launch_bounds__(kPackThreads, 1) fold_pack_kernel(const FoldPa
     const uint32_t rec_bytes = pack_records_bytes(nbins, G);
     uint32_t dyn;
     asm("mov.u32 %0, %%dynamic_smem_size;" : "=r"(dyn));
-    if (rec + rec_bytes > base + dyn) {  // (the launch sized the block for a window at kWindow)
+    if (rec + rec_bytes > base + dyn) {  // (the launch sized the block for the device's window)
         report_error(p.status, kErrTimeout);
         return;
     }
@@ -736,15 +735,15 @@ __global__ void __launch_bounds__(kPackThreads, 1) fold_pack_kernel(const FoldPa
     }
 }
 
-size_t fold_pack_smem(int nbins, int groups)
+static size_t fold_pack_smem(int nbins, int groups, uint32_t window)
 {
-    return pack_records_addr(kWindow, nbins) - kWindow + pack_records_bytes(nbins, groups);
+    return pack_records_addr(window, nbins) - window + pack_records_bytes(nbins, groups);
 }
 
-int fold_pack_groups(int nbins)
+int fold_pack_groups(int nbins, uint32_t window)
 {
     int g = kPackMaxGroups;
-    while (g > 0 && fold_pack_smem(nbins, g) > kSmemLimit) --g;
+    while (g > 0 && fold_pack_smem(nbins, g, window) > kSmemLimit) --g;
     return fold_pack_allowed(nbins, g);
 }
 
@@ -786,9 +785,9 @@ int fold_pack_register()
     return (int)e;
 }
 
-cudaError_t launch_fold_pack(const FoldParams &p, int grid, cudaStream_t st)
+cudaError_t launch_fold_pack(const FoldParams &p, uint32_t window, int grid, cudaStream_t st)
 {
-    const size_t smem = fold_pack_smem(p.nbins, p.warps);
+    const size_t smem = fold_pack_smem(p.nbins, p.warps, window);
     if (p.warps < 1 || p.warps > kPackMaxGroups || smem > kSmemLimit || p.chunk != kPackChunk) return cudaErrorInvalidValue;
     return with_kernel(p.nbins, p.shift, p.warps, [&](auto kernel) {
         kernel<<<grid, kPackThreads, smem, st>>>(p);

@@ -152,11 +152,11 @@ constexpr int kPackPlanesHilo = 3 + 2 * (kPackSegs - 1);
 constexpr int kPackMinBins = 32;
 // prep's chunk below 256 bins: flux in 31 bits (the bound of two samples' sum)
 constexpr int kPackHiloChunk = 2;
-size_t fold_pack_smem(int nbins, int groups);
-int fold_pack_groups(int nbins);
+// `window`: the shared address at which a block's dynamic memory starts.
+int fold_pack_groups(int nbins, uint32_t window);
 int fold_pack_allowed(int nbins, int groups);  // the largest instance of at most that many groups
 int fold_pack_register();
-cudaError_t launch_fold_pack(const FoldParams &p, int grid, cudaStream_t st);
+cudaError_t launch_fold_pack(const FoldParams &p, uint32_t window, int grid, cudaStream_t st);
 // Shared memory of a kModeSearch block (0 if it does not fit or warps + 1 > 4).
 size_t search_smem_bytes(int nbins, int warps, int layout, int tile, int streams = 1);
 int search_blocks_per_sm(int nbins, int warps, int layout, int tile, int streams = 1);
