@@ -304,8 +304,10 @@ FoldPlan plan_with(const gpfc_ctx *ctx, int64_t n, int64_t np, int nbins, const 
 // What the fold gives: scores, profiles for a scorer (the plan may be the one-word fold's) or
 // profiles for the caller (so too below 256 bins).
 enum FoldOut { kScores, kForScorer, kForCaller };
+// The plan, and (below 256 bins, beside the one-word fold's) the FP32 plan of the same fold, else
+// the same plan again.
 FoldPlan plan_fold(gpfc_ctx *ctx, int64_t n, int64_t np, int nbins, const gpfc_ctx::Tuned *tuned, FoldOut out,
-                   int64_t nstars = 1)
+                   int64_t nstars = 1, FoldPlan *general = nullptr)
 {
     gpfc_fold_config cfg = ctx->fold_cfg;
     if (tuned && !tuned->packed) {
@@ -317,9 +319,10 @@ FoldPlan plan_fold(gpfc_ctx *ctx, int64_t n, int64_t np, int nbins, const gpfc_c
     const bool packed = (out != kScores && pack_ok(ctx, nbins) && (!tuned || tuned->packed)) ||
                         (out == kForCaller && hilo_ok(ctx, nbins));
     const FoldPlan pl = packed ? plan_packed(ctx, n, np, nbins, nstars) : plan_with(ctx, n, np, nbins, cfg);
-    // (below 256 bins the FP32 plan that it stands in for: layout 3 set by hand there would cut
-    // the flux to its chunk's fixed point)
+    // (below 256 bins the FP32 plan, which is launched behind the one-word fold: layout 3 set by hand
+    // there would cut the flux to its chunk's fixed point)
     const FoldPlan r = packed && nbins < 256 ? plan_with(ctx, n, np, nbins, cfg) : pl;
+    if (general) *general = r;
     ctx->last_plan = gpfc_fold_config{r.warps, r.layout, r.chunk, r.tile, r.bps, r.streams};
     return pl;
 }
@@ -533,10 +536,11 @@ int run_fold(gpfc_ctx *ctx, const double *times, const float *flux, int64_t n, c
              int64_t np, int32_t nbins, double t0, int mode, FoldParams p, bool want_key,
              FoldBuffers *out_fb)
 {
-    const FoldPlan pl =
-        plan_fold(ctx, n, np, nbins, find_tuned(ctx, nbins, mode, n), mode == kModeFold ? kForCaller : kScores);
+    FoldPlan general{};
+    const FoldPlan pl = plan_fold(ctx, n, np, nbins, find_tuned(ctx, nbins, mode, n),
+                                  mode == kModeFold ? kForCaller : kScores, 1, &general);
     FoldBuffers fb{};
-    const size_t need = carve_fold(nullptr, pl, n, 1, nbins, fb);
+    const size_t need = std::max(carve_fold(nullptr, pl, n, 1, nbins, fb), carve_fold(nullptr, general, n, 1, nbins, fb));
     int rc = ensure_ws(ctx, need);
     if (rc) return rc;
     carve_fold(ctx->ws, pl, n, 1, nbins, fb);
@@ -572,7 +576,23 @@ int run_fold(gpfc_ctx *ctx, const double *times, const float *flux, int64_t n, c
         if (e != cudaSuccess) return cuda_err(ctx, e, "cudaMemsetAsync");
     }
     KernelTimer timer(ctx);
+    p.when = hilo ? 1 : 0;
     e = launch_plan(ctx, pl, p, pl.grid, ctx->stream, mode);
+    if (hilo && e == cudaSuccess) {
+        // a star whose flux spreads too widely is left to the FP32 fold (else this launch is over in a
+        // few microseconds); its workspace lies in the same place
+        carve_fold(ctx->ws, general, n, 1, nbins, fb);
+        p.when = 2;
+        p.ntasks = general.ntasks;
+        p.warps = general.warps;
+        p.chunk = general.chunk;
+        p.layout = general.layout;
+        p.streams = general.streams;
+        p.tile = general.tile;
+        p.ws_sc = fb.ws_sc;
+        p.ws_cnt = fb.ws_cnt;
+        e = launch_plan(ctx, general, p, general.grid, ctx->stream);
+    }
     if (e != cudaSuccess) return cuda_err(ctx, e, "fold kernel");
     timer.stop();
     if (out_fb) *out_fb = fb;
@@ -1552,9 +1572,11 @@ int gpfc_workspace_size(gpfc_ctx *ctx, int64_t n, int64_t n_periods, int32_t nbi
     const gpfc_fold_config last = ctx->last_plan;
     const FoldPlan pb = plan_fold(ctx, n, n_periods, nbins, find_tuned(ctx, nbins, kModeBox, n), kScores);
     const FoldPlan pf = plan_fold(ctx, n, n_periods, nbins, find_tuned(ctx, nbins, kModeFold, n), kForScorer);
-    const FoldPlan pc = plan_fold(ctx, n, n_periods, nbins, find_tuned(ctx, nbins, kModeFold, n), kForCaller);
+    FoldPlan pg{};
+    const FoldPlan pc = plan_fold(ctx, n, n_periods, nbins, find_tuned(ctx, nbins, kModeFold, n), kForCaller, 1, &pg);
     FoldBuffers fb{};
     *bytes = std::max(carve_fold(nullptr, pb, n, 1, nbins, fb), carve_fold(nullptr, pc, n, 1, nbins, fb));
+    *bytes = std::max(*bytes, carve_fold(nullptr, pg, n, 1, nbins, fb));
     *bytes = std::max(*bytes, box_warp_bytes(pf, n, n_periods, nbins));
     FoldPlan ps{};
     if (fused_plan(ctx, n, n_periods, nbins, ps)) {

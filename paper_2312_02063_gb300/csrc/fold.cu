@@ -237,7 +237,12 @@ __global__ void prep_sigma_kernel(const double *partial, const long long *pmin, 
     // a chunk holds at most min(chunk, n) samples of the star
     const int lmax = min(chunk, max(1, stats[s].n));
     stats[s].qexp = fixed_point_exp(xm, floor(2147483647.0 / (double)lmax));
-    stats[s].pad = 0;
+    // 31 bits of the largest |x|, off by up to 2^-30 of it, are as good as each x's own 24 where that is
+    // below 2^-28 of the level (an eighth of the rounding of a mean at least), or where the mean |x|,
+    // at least sigma^2 / max|x|, is a 32nd of the largest. Else (an outlier on a level of zero, or far
+    // above it; a flux that is no number) the fold keeps FP32 sums.
+    const double var = t / (double)stats[s].n;
+    stats[s].wide = !(isfinite(t) && (xm <= 4.0 * fabs(stats[s].f_ref) || xm * xm <= 32.0 * var));
 }
 
 constexpr int32_t kThMixed = INT32_MIN;  // per-group high word marker: the samples differ
@@ -2007,6 +2012,7 @@ __global__ void __launch_bounds__(MAXW * 32, 1) fold_kernel(const FoldParams p)
     __shared__ int s_abort;
     __shared__ SearchShared sh;
     constexpr bool kRed = LAYOUT == kLayoutRed32;
+    if (MODE == kModeFold && !kRed && p.when == 2 && !p.stats[0].wide) return;  // (the one-word fold's)
     const int lane = threadIdx.x & 31;
     const int warp = threadIdx.x >> 5;
     const int nbins = p.nbins;

@@ -174,6 +174,7 @@ __global__ void __launch_bounds__(kPackThreads, 1) fold_pack_kernel(const FoldPa
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nbins = p.nbins;
     constexpr int ppc = 32 * G;  // G = p.warps period groups
+    if (KIND >= 3 && p.when == 1 && p.stats[0].wide) return;  // (the FP32 fold's)
     const uint32_t base = smem_u32(smem);
     const uint32_t rec = pack_records_addr(base, nbins);
     const uint32_t rec_bytes = pack_records_bytes(nbins, G);

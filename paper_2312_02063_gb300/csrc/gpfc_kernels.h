@@ -32,6 +32,7 @@ struct StarStats {
     int32_t n;      // samples of the star
     long long dtau0;  // smallest positive step between consecutive quantised times (0: none)
     int32_t qexp;     // fixed-point flux: xq = rint(x 2^qexp), |xq| <= (2^31 - 1) / chunk
+    int32_t wide;     // the flux spreads too widely for 31 bits of its largest value (prep)
     int32_t pad;
 };
 
@@ -97,6 +98,9 @@ struct FoldParams {
     float sigma_user;          // > 0: use it; else the star's flux std (1 if that is 0)
     size_t stage_off;          // kModeSearch: byte offset of the scorer staging in shared memory
     uint32_t *status;
+    // gpfc_fold below 256 bins launches the one-word fold and the FP32 fold: of one star, a fold
+    // with `when` 1 leaves a star marked wide alone, one with 2 every other (0: folds all)
+    int when;
 };
 
 // Box-SNR over profiles the fold wrote as centred sums and counts ([row][nbins]), one warp

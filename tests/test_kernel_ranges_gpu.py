@@ -93,6 +93,37 @@ def test_generated_profiles_of_wide_ranges(ctx, sigma, depth, n_cad):
     assert np.sqrt((np.concatenate(err) ** 2).mean()) <= 2.0 ** -23 / 12 ** 0.5
 
 
+# an outlier far above a flux about zero, or above its level: the FP32 sums; none, one within the level or a
+# normal spread about zero: 31 bits of the largest value, which are the more exact there
+@pytest.mark.parametrize("level,outlier,fp32", [(0.0, 1e6, True), (1.0, 1e6, True), (0.0, 1.0, True), (0.0, 0.0, False),
+                                                (1.0, 0.0, False), (1.0, 1.0, False), (1e5, 1e4, False)])
+@pytest.mark.parametrize("nbins", [64, 200])
+def test_fold_below_256_bins_with_an_outlier(ctx, level, outlier, fp32, nbins):
+    import paper_2312_02063_gb300 as g
+    rng = np.random.default_rng(2)
+    n = 20000
+    t = np.arange(n) * CADENCE
+    f = (level + rng.normal(0.0, 3e-4 * max(level, 1.0), n)).astype(np.float32)
+    f[5] += np.float32(outlier)
+    p = rng.uniform(0.2, 1.0, 50)
+    args = [_dev(ctx, x) for x in (t, f, p)]
+    a, ca = g.gpfc_fold(ctx, *args, nbins, 0.0)
+    ctx.set_fold_config(layout=1)
+    try:
+        b, cb = g.gpfc_fold(ctx, *args, nbins, 0.0)
+    finally:
+        ctx.reset_fold_config()
+    ctx.sync()
+    assert torch.equal(ca, cb)
+    if fp32:
+        assert torch.equal(torch.nan_to_num(a, 7.0), torch.nan_to_num(b, 7.0))
+        return
+    mean_o, cnt_o, _ = oracle.fold(t, f, p, nbins, 0.0)
+    nz = cnt_o > 0
+    rms = [np.sqrt(((x.cpu().numpy().astype(np.float64)[nz] - mean_o[nz]) ** 2).mean()) for x in (a, b)]
+    assert rms[0] <= rms[1] * (1.0 + 1e-3)
+
+
 def test_decision_of_several_stars_takes_no_longer_than_of_many(ctx):
     """19 stars of 16,384 periods: a block each, not clusters that take turns."""
     import paper_2312_02063_gb300 as g
