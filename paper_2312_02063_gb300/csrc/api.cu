@@ -35,7 +35,7 @@ struct gpfc_ctx {
         int nbins, mode, lg;
         gpfc_fold_config cfg;
         float ms;
-        bool packed;  // the one-word fold (fold_pack.cu) was the fastest
+        bool packed;  // the one-word fold (fold_pack.cu) was faster than cfg
     };
     std::vector<Tuned> tuned;
     bool autotune = true;
@@ -194,17 +194,27 @@ const gpfc_ctx::Tuned *find_tuned(const gpfc_ctx *ctx, int nbins, int mode, int6
     return nullptr;
 }
 
+// The one-word fold named by its own shape, as gpfc_last_fold_plan and the autotuner give it out: its
+// sixteen warps are streams of no period group of their own, so one stream a group, which the
+// two-word fold's plans never have.
+bool pack_named(const gpfc_fold_config &c)
+{
+    return c.layout == kLayoutRed32 && c.tile == kMaxTile && c.blocks_per_sm == 1 && c.streams == 1 &&
+           (c.chunk == 0 || c.chunk == kPackChunk);
+}
+
 // Whether a fold that writes profiles may take the one-word form of layout 3: wherever that
 // layout is the default (or set), fits (else the FP32 layout runs) and nothing else about the
-// launch is set. Its results are the layout's own, and it was the faster one at every size
+// launch is set, or its own shape. Its results are the layout's own, and it was the faster one at every size
 // measured: 192 periods of 62,835 samples and 256 bins in 1.04 M cycles of a multiprocessor,
 // against 2 x 0.755 M (fold_pack.cu); searches by CNN, two words -> one: 250,000 periods
 // 9.6 -> 8.4 ms, 100,000 periods 4.1 -> 3.8 ms.
 bool pack_ok(const gpfc_ctx *ctx, int nbins)
 {
     const gpfc_fold_config &c = ctx->fold_cfg;
-    return default_layout(nbins) == kLayoutRed32 && (c.layout == 0 || c.layout == kLayoutRed32) && c.warps == 0 &&
-           c.chunk == 0 && c.tile == 0 && c.blocks_per_sm == 0 && c.streams == 0 &&
+    const bool automatic = (c.layout == 0 || c.layout == kLayoutRed32) && c.warps == 0 && c.chunk == 0 && c.tile == 0 &&
+                           c.blocks_per_sm == 0 && c.streams == 0;
+    return default_layout(nbins) == kLayoutRed32 && (automatic || pack_named(c)) &&
            fold_max_warps(nbins, kLayoutRed32, kTile) >= 1 && fold_pack_groups(nbins, ctx->window) >= 1;
 }
 
@@ -236,7 +246,9 @@ FoldPlan plan_packed(const gpfc_ctx *ctx, int64_t n, int64_t np, int nbins, int6
     const int maxg =
         fold_pack_allowed(nbins, (int)std::max<int64_t>(1, std::min<int64_t>(fold_pack_groups(nbins, ctx->window), per_sm)));
     pl.warps = maxg;
-    if (nstars > 1) {
+    if (ctx->fold_cfg.warps > 0) {
+        pl.warps = std::min(ctx->fold_cfg.warps, fold_pack_groups(nbins, ctx->window));
+    } else if (nstars > 1) {
         const int64_t avg = std::max<int64_t>(1, np / nstars);
         int64_t best = INT64_MAX;
         for (int g = maxg; g >= 1; --g) {
@@ -249,7 +261,7 @@ FoldPlan plan_packed(const gpfc_ctx *ctx, int64_t n, int64_t np, int nbins, int6
         }
     }
     pl.ppc = 32 * pl.warps;
-    pl.streams = std::max(1, kMaxRedWarps / pl.warps);
+    pl.streams = 1;
     pl.ntasks = (np + pl.ppc - 1) / pl.ppc;
     pl.grid = (int)std::min<int64_t>(pl.ntasks, ctx->num_sms);
     pl.G = prep_groups(n);
@@ -316,7 +328,8 @@ FoldPlan plan_fold(gpfc_ctx *ctx, int64_t n, int64_t np, int nbins, const gpfc_c
         if (!cfg.tile) cfg.tile = tuned->cfg.tile;
         if (!cfg.blocks_per_sm) cfg.blocks_per_sm = tuned->cfg.blocks_per_sm;
     }
-    const bool packed = (out != kScores && pack_ok(ctx, nbins) && (!tuned || tuned->packed)) ||
+    const bool packed = (out != kScores && pack_ok(ctx, nbins) &&
+                         (pack_named(ctx->fold_cfg) || !tuned || tuned->packed)) ||
                         (out == kForCaller && hilo_ok(ctx, nbins));
     const FoldPlan pl = packed ? plan_packed(ctx, n, np, nbins, nstars) : plan_with(ctx, n, np, nbins, cfg);
     // (below 256 bins the FP32 plan, which is launched behind the one-word fold: layout 3 set by hand
@@ -1034,8 +1047,8 @@ int tune_fold(gpfc_ctx *ctx, const double *times, const float *flux, int64_t n, 
     float *score = reinterpret_cast<float *>(static_cast<char *>(ctx->ws) + ((need + 255) & ~(size_t)255));
     bool prepped = false;
     float best_ms = 0.f;
-    gpfc_fold_config best{};
-    bool best_packed = false;
+    gpfc_fold_config best{}, packed_shape{};
+    bool best_packed = false;  // (its candidate is the last: faster than every other)
     for (const Cand &c : cands) {
         if (2 * c.resident < best_res) continue;
         const FoldPlan pl = plan_of(c);
@@ -1086,8 +1099,9 @@ int tune_fold(gpfc_ctx *ctx, const double *times, const float *flux, int64_t n, 
         ms *= 0.5f;
         if (best_ms == 0.f || ms < best_ms) {
             best_ms = ms;
-            best = gpfc_fold_config{pl.warps, pl.layout, 0, pl.tile, pl.bps};
             best_packed = pl.packed != 0;
+            if (best_packed) packed_shape = gpfc_fold_config{pl.warps, pl.layout, 0, pl.tile, pl.bps, pl.streams};
+            else best = gpfc_fold_config{pl.warps, pl.layout, 0, pl.tile, pl.bps};
         }
     }
     ctx->timed = false;
@@ -1101,7 +1115,7 @@ int tune_fold(gpfc_ctx *ctx, const double *times, const float *flux, int64_t n, 
             found = true;
         }
     if (!found) ctx->tuned.push_back(gpfc_ctx::Tuned{nbins, mode, lg, best, best_ms, best_packed});
-    if (out) *out = best;
+    if (out) *out = best_packed ? packed_shape : best;
     return GPFC_OK;
 }
 

@@ -124,6 +124,58 @@ def test_fold_below_256_bins_with_an_outlier(ctx, level, outlier, fp32, nbins):
     assert rms[0] <= rms[1] * (1.0 + 1e-3)
 
 
+# ---------------------------------------------------------------- the one-word fold's range
+
+def _times(kind, n, rng):
+    t = np.arange(n) * CADENCE
+    if kind == "gaps":
+        t = t + 3.3 * (np.arange(n) // 911)
+    elif kind == "nights":
+        t = np.arange(n) // 1200 + (np.arange(n) % 1200) / 3600.0
+    elif kind == "unsorted":
+        t = rng.uniform(0.0, 900.0, n)
+    elif kind == "random":  # no cadence: the smallest step says nothing about the others
+        t = np.sort(rng.uniform(0.0, n * CADENCE, n))
+    elif kind == "equal":  # every sample in one bin of every period
+        t = np.full(n, 7.25)
+    elif kind == "barycentric":
+        t = t + 200.0 / 86400.0 * np.sin(2 * np.pi * t / 372.5)
+    return t
+
+
+def _one_word(g, groups):
+    """The one-word fold by its own shape, with that many groups of 32 periods a block."""
+    return dict(warps=groups, layout=g.LAYOUT_RED32, tile=2048, blocks_per_sm=1, streams=1)
+
+
+# lengths about the tile (256 to 2,048), the segments (1 to 8 tiles), the chunk (65,520) and the groups of 16;
+# periods about the group (32) and the block; a fine grid about twelve and a half cadences, whose groups
+# fail their checks and go on with shorter segments
+@pytest.mark.parametrize("n,kind,n_periods,nbins,groups", [
+    (1, "regular", 1, 256, 1), (15, "regular", 33, 256, 2), (17, "unsorted", 31, 512, 1), (300, "gaps", 193, 256, 6),
+    (2047, "regular", 200, 256, 6), (2049, "gaps", 64, 256, 2), (4096, "equal", 40, 256, 3), (3000, "random", 700, 512, 3),
+    (20000, "barycentric", 500, 256, 4), (32769, "gaps", 193, 256, 5), (65519, "regular", 96, 256, 3),
+    (65521, "gaps", 192, 256, 6), (70001, "unsorted", 65, 512, 2), (140000, "nights", 200, 256, 6),
+    (40000, "equal", 33, 512, 3), (200000, "random", 64, 256, 2)])
+def test_one_word_fold_equals_two_words(ctx, n, kind, n_periods, nbins, groups):
+    import paper_2312_02063_gb300 as g
+    rng = np.random.default_rng(n + nbins)
+    f = (1.0 + rng.normal(0.0, 3e-4, n)).astype(np.float32)
+    p = np.r_[np.linspace(12.45, 12.55, n_periods // 2) * CADENCE, rng.uniform(0.05, 1.0, n_periods - n_periods // 2)]
+    args = [_dev(ctx, x) for x in (_times(kind, n, rng), f, p)]
+    try:
+        ctx.set_fold_config(**_one_word(g, groups))
+        one = g.gpfc_fold(ctx, *args, nbins, 0.0)
+        assert ctx.last_fold_plan()["warps"] == groups and ctx.last_fold_plan()["streams"] == 1
+        ctx.set_fold_config(warps=1, layout=g.LAYOUT_RED32)
+        two = g.gpfc_fold(ctx, *args, nbins, 0.0)
+    finally:
+        ctx.reset_fold_config()
+    ctx.sync()
+    assert torch.equal(one[1], two[1])
+    assert torch.equal(torch.nan_to_num(one[0], 7.0), torch.nan_to_num(two[0], 7.0))
+
+
 def test_decision_of_several_stars_takes_no_longer_than_of_many(ctx):
     """19 stars of 16,384 periods: a block each, not clusters that take turns."""
     import paper_2312_02063_gb300 as g
