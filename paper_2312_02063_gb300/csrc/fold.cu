@@ -237,6 +237,7 @@ __global__ void prep_sigma_kernel(const double *partial, const long long *pmin, 
     // a chunk holds at most min(chunk, n) samples of the star
     const int lmax = min(chunk, max(1, stats[s].n));
     stats[s].qexp = fixed_point_exp(xm, floor(2147483647.0 / (double)lmax));
+    stats[s].nreg = 0;  // counted by the next pass
     // 31 bits of the largest |x|, off by up to 2^-30 of it, are as good as each x's own 24 where that is
     // below 2^-28 of the level (an eighth of the rounding of a mean at least), or where the mean |x|,
     // at least sigma^2 / max|x|, is a 32nd of the largest. Else (an outlier on a level of zero, or far
@@ -253,10 +254,10 @@ constexpr int32_t kThMixed = INT32_MIN;  // per-group high word marker: the samp
 // skips its per-group bin-collision check on flagged groups when the period allows it,
 // and forms their phases with one th * F_lo product per group. The same pass writes the
 // fixed-point flux xq = rint(x 2^qexp) when the scratch has room for it, with pack_chunk > 0 as
-// the one-word fold's increment xq + 2^S + L.
+// the one-word fold's increment xq + 2^S + L, and counts the star's regular steps.
 // grid = (G, stars).
 __global__ void prep_flags_kernel(const int64_t *lc_off, int64_t n, SampleScratch smp,
-                                  const StarStats *stats, int pack_chunk)
+                                  StarStats *stats, int pack_chunk)
 {
     const int s = blockIdx.y;
     int64_t b, e;
@@ -266,6 +267,7 @@ __global__ void prep_flags_kernel(const int64_t *lc_off, int64_t n, SampleScratc
     const long long d0 = stats[s].dtau0;
     const int64_t ngroups = (len + 255) / 256 * 16;  // every flag byte of the star's region
     const uint32_t add = pack_chunk > 0 ? pack_word(len, pack_chunk).add() : 0u;
+    int steps = 0;  // of about dtau0 (the barycentric correction makes a cadence vary by 10^-4)
     for (int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; q < ngroups;
          q += (int64_t)gridDim.x * blockDim.x) {
         const int64_t j0 = q * 16;
@@ -278,6 +280,7 @@ __global__ void prep_flags_kernel(const int64_t *lc_off, int64_t n, SampleScratc
                 const long long cur = ((long long)th << 32) | smp.tau_lo[base + j0 + k];
                 const long long d = cur - prev;
                 reg &= (d >= d0) & (d <= d0 + 2) & (th == th0);
+                steps += (d >= d0) & (d <= d0 + 2 + (d0 >> 8));
                 prev = cur;
             }
         }
@@ -303,6 +306,8 @@ __global__ void prep_flags_kernel(const int64_t *lc_off, int64_t n, SampleScratc
                     j0 + k < len ? (int32_t)((uint32_t)__double2int_rn((double)smp.x[base + j0 + k] * sc) + add) : 0;
         }
     }
+    steps = __reduce_add_sync(0xffffffffu, steps);
+    if ((threadIdx.x & 31) == 0 && steps) atomicAdd(&stats[s].nreg, steps);
 }
 
 cudaError_t launch_prep(const double *times, const float *flux, const int64_t *lc_off, int64_t n,

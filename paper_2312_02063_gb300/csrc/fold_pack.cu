@@ -14,11 +14,14 @@
 // Then nothing wrapped (the sums of the true and the stored words differ by a multiple of 2^32
 // and by less than 2^32, as 2 L n < 2^32 for a segment of n <= chunk samples), y <= 2 L c <=
 // 2 L c' < 2^S, and so c' and y' are the true count and sum. A group that fails (a period so
-// close to a multiple of the cadence that its samples pile up in a few bins) folds its segment
-// again in two passes of plain 32-bit words, counts and then sums, which cannot overflow; a
-// group predicted to fail takes shorter segments (down to a tile) of its own, so that a block
-// with such a period costs little more than the others (a launch lasts as long as its slowest
-// block).
+// close to a multiple of the cadence that its samples pile up in a few bins) needs only its counts
+// again: its words hold the sum of xq + c (2^S + L) mod 2^32, and |sum of xq| < 2^31 up to a chunk of
+// samples. So its words are put aside, the segment's samples counted plainly, and both give the
+// sum; from there on the group takes shorter segments, and in the end none: a blind group's words are
+// put aside at the end of the star (or chunk) and its samples counted in a second turn of the tiles, all
+// blind groups at once. A group predicted to fail starts with shorter segments, or blind. So a block
+// folds no sample more than twice (plus one failed segment a group), and the groups that pass do so as
+// ever.
 //
 // Below 256 bins, where the flux is not cut to the chunk's fixed point (layouts 1 and 2 sum FP32),
 // the same scheme takes 31-bit flux (HILO): xq = hi 2^15 + lo, the word holds the count and the
@@ -31,12 +34,11 @@
 // each), as in fold.cu.
 //
 // What bounds it: the integer multiplies of the phase (mad.hi 4.3 and mad.lo 2.0 cycles per
-// warp instruction and scheduler, measured; a reduction 4.0) and the moves the compiler puts on
-// their pipe. Inner loop alone, 256 bins, six groups, 16 warps: 4.3e12 updates/s against 3.15e12
-// with two reductions (12 warps: 4.0e12). A block of 192 periods x 62,835 samples: 0.88 M cycles
-// of folding, 0.06 M of checks and slots, 0.08 M of epilogue (the output rows and the slots are
-// L2 traffic that all blocks make at once), 0.015 M of set-up; the two-word fold takes
-// 0.755 M for 96 periods.
+// warp instruction and scheduler; a reduction 4.0) and the moves the compiler puts on their
+// pipe. A launch lasts as long as its slowest block. 30,000 periods of 65,000 samples into 256 bins,
+// two words / one word, by where the periods lie: 0.5 to 100 days 1.14 / 0.75 ms, 0.2 to 1 day
+// (the usual multiples of the cadence) 1.14 / 0.87, all within 10^-4 of 3, 7, 10 or 12.5 cadences
+// 1.14 / 0.75..0.81 (2.4 where a failed tile was folded twice more).
 #include <algorithm>
 #include <cmath>
 #include <cstdint>
@@ -61,7 +63,8 @@ struct PackShared {
     int abort;
     uint32_t risk;    // predictor: OR over the block's periods, four bits a group
     uint32_t bad[2];  // groups that failed a check (of this and the next boundary, in turn)
-    int pad[24];
+    int blind_from[8];  // first tile that a blind group's words hold
+    int pad[16];
 };
 static_assert(sizeof(PackShared) == 128, "header layout");
 
@@ -156,10 +159,10 @@ __device__ __forceinline__ void load_pack_half(uint32_t stl, uint32_t sxq, int i
 // samples k apart differ by k r mod 1; let that be d bins. The samples of one residue mod k
 // then put min(seg / k, 1 / d) of a segment of seg samples into a bin they cross, and
 // floor((k + seg d) / nbins) + 1 residues cross one. A group's segment length is at risk when a k up to
-// seg's own reach passes 0.95 M that way. Against counts (four grids and lengths, 80 blocks of
-// 192 periods each): the length chosen held in all but 1% of the blocks. Only a guess (gaps,
-// other cadences); the check after the segment decides.
-constexpr int kPackLevels = 4;  // a group's segments: the block's (about 8 tiles), 4, 2 and 1 tiles
+// seg's own reach passes 0.95 M that way. Only a guess (gaps, other cadences), and made only where at
+// least half the steps are about the smallest one; the check after the segment decides.
+constexpr int kPackLevels = 4;  // a group's segments: the block's (about 8 tiles), 4, 2 and 1 tiles, or
+constexpr uint32_t kBlind = 31u;  // none: counted once more afterwards
 constexpr int kPackSegTiles = 8;
 
 template <int KIND, int G>
@@ -210,12 +213,13 @@ __global__ void __launch_bounds__(kPackThreads, 1) fold_pack_kernel(const FoldPa
                            reinterpret_cast<uintptr_t>(p.counts)) & 31) == 0;
     // this block's workspace in L2, planes of [bin][32 G] words: two of 64-bit totals (count 2^40 +
     // biased sum up to 2^23 samples, else an int64 sum and, in the third plane, 32-bit counts),
-    // then the slots
+    // then the slots, then one for words put aside
     const size_t plane = (size_t)nbins * ppc;
     constexpr int kPlanes = HILO ? kPackPlanesHilo : kPackPlanes;
     uint32_t *ws = reinterpret_cast<uint32_t *>(p.ws_sc) + (size_t)blockIdx.x * kPlanes * plane + lane;
     unsigned long long *ws_tot = reinterpret_cast<unsigned long long *>(ws - lane) + lane;
     uint32_t *ws_cnt = ws + 2 * plane, *ws_slot = ws + 3 * plane;
+    uint32_t *ws_raw = ws + (size_t)(kPlanes - 1) * plane;  // words put aside
 
     int64_t task_end = p.ntasks;
     if (p.ntasks_dev) {
@@ -278,11 +282,10 @@ __global__ void __launch_bounds__(kPackThreads, 1) fold_pack_kernel(const FoldPa
         const PackWord pw = HILO ? PackWord{0u, 256u, 23} : pack_word(nsamp, p.chunk);
         const bool wide = HILO || nsamp > ((int64_t)1 << 23);
         const unsigned long long bias = (1ull << 40) + pw.L;  // per count in a 64-bit total
-        // Tiles of the star: no longer than a tenth of the samples over 0.86 M, so that one tile
-        // holds even for a period ten cadences long.
-        int tile = kPackTile;
-        while (tile > 256 && (float)tile > 8.6f * (float)pw.M) tile >>= 1;
+        constexpr int tile = kPackTile;
         const int ntiles = (int)((nsamp + tile - 1) / tile);
+        // (the plain sum of a blind group's samples fits 32 bits up to a chunk)
+        const int span_tiles = nsamp <= (int64_t)p.chunk ? ntiles : p.chunk / tile;
         // The block's segments: of seg_tiles tiles, about kPackSegTiles but no more than a mean load of
         // about half M allows; into slots where a star of one chunk has at most kPackSegs of them.
         const int most = max(1, (int)fminf(0.55f * (float)pw.M * (float)nbins / (float)tile, 1e6f));
@@ -312,7 +315,8 @@ __global__ void __launch_bounds__(kPackThreads, 1) fold_pack_kernel(const FoldPa
                 kall = max(kall, kmax[v]);
                 if (kmax[v] > 0) top = fmaxf(top, seg[v]);
             }
-            const long long d0 = p.stats[s].dtau0;
+            // (of times without a regular cadence it would say nothing)
+            const long long d0 = 2 * (int64_t)p.stats[s].nreg >= nsamp ? p.stats[s].dtau0 : 0;
 #pragma unroll
             for (int j = 0; j < G; ++j) {
                 if (((live >> j) & 1u) && d0 > 0) {
@@ -338,13 +342,15 @@ __global__ void __launch_bounds__(kPackThreads, 1) fold_pack_kernel(const FoldPa
             if (lane == 0 && risk) atomicOr(&sh.risk, risk);
         }
         __syncthreads();
-        // five bits a group: 0 (the block's segments) or 4, 2 or 1 tiles (1 also if all are at risk)
+        // five bits a group: 0 (the block's segments), 4, 2 or 1 tiles, or blind
         uint32_t own = 0u;
 #pragma unroll
         for (int j = 0; j < G; ++j) {
             const uint32_t risk = (sh.risk >> (5 * j)) & 15u;
-            own |= (!(risk & 1u) ? 0u : (!(risk & 2u) ? 4u : (!(risk & 4u) ? 2u : 1u))) << (5 * j);
+            own |= (!(risk & 1u) ? 0u : (!(risk & 2u) ? 4u : (!(risk & 4u) ? 2u : (!(risk & 8u) ? 1u : kBlind)))) << (5 * j);
         }
+        if (threadIdx.x < 8) sh.blind_from[threadIdx.x] = 0;
+        auto len_of = [&](int j) { return (own >> (5 * j)) & 31u; };
 
         // each group's part of the address, kept in a register (formed again for every group of
         // samples it costs moves on the multiplies' pipe: 0.578 -> 0.555 ms for 152 blocks)
@@ -370,8 +376,10 @@ __global__ void __launch_bounds__(kPackThreads, 1) fold_pack_kernel(const FoldPa
             ++issued;
         };
 
-        // Every sample of tile t into the bins of all groups. False (all threads) when a wait gave up.
-        auto fold_tile = [&](int t) -> bool {
+        // Every sample of tile t into the bins of all groups; or (count) a plain 1 into those of the
+        // groups in mask. False (all threads) when a wait gave up.
+        auto fold_tile = [&](int t, auto count, uint32_t mask) -> bool {
+            constexpr bool COUNT = decltype(count)::value;
             const uint32_t b = consumed & 1u;
             const bool ok = mbar_wait_bounded(&sh.bars[b], (consumed >> 1) & 1u);
             ++consumed;
@@ -390,8 +398,11 @@ __global__ void __launch_bounds__(kPackThreads, 1) fold_pack_kernel(const FoldPa
                     const uint32_t x = lds_u32(sxq + 4u * i);
 #pragma unroll
                     for (int j = 0; j < G; ++j) {
-                        sample_add<KIND>(word_addr<KIND>(phase_hi(tl, th * Fl[j], Fl[j], Fh[j]), tl, Fl[j], gaddr[j],
-                                                         (uint32_t)nbins, p.shift), x, 1u << pw.S);
+                        if (COUNT && !((mask >> j) & 1u)) continue;
+                        const uint32_t w = word_addr<KIND>(phase_hi(tl, th * Fl[j], Fl[j], Fh[j]), tl, Fl[j], gaddr[j],
+                                                           (uint32_t)nbins, p.shift);
+                        if (COUNT) word_add<KIND>(w, 1u);
+                        else sample_add<KIND>(w, x, 1u << pw.S);
                     }
                 };
                 // a group whose samples differ in their high word (every ~256 days, or
@@ -407,6 +418,7 @@ __global__ void __launch_bounds__(kPackThreads, 1) fold_pack_kernel(const FoldPa
                     auto half = [&](const PackHalf &H, uint32_t th) {
 #pragma unroll
                         for (int j = 0; j < G; ++j) {
+                            if (COUNT && !((mask >> j) & 1u)) continue;
                             const uint32_t thF = th * Fl[j];
                             uint32_t ad[8];
 #pragma unroll
@@ -421,7 +433,10 @@ __global__ void __launch_bounds__(kPackThreads, 1) fold_pack_kernel(const FoldPa
                             for (int q = 0; q < 2; ++q) {
                                 const uint32_t xx[4] = {H.x[q].x, H.x[q].y, H.x[q].z, H.x[q].w};
 #pragma unroll
-                                for (int u = 0; u < 4; ++u) sample_add<KIND>(ad[4 * q + u], xx[u], 1u << pw.S);
+                                for (int u = 0; u < 4; ++u) {
+                                    if (COUNT) word_add<KIND>(ad[4 * q + u], 1u);
+                                    else sample_add<KIND>(ad[4 * q + u], xx[u], 1u << pw.S);
+                                }
                             }
                         }
                     };
@@ -461,33 +476,35 @@ __global__ void __launch_bounds__(kPackThreads, 1) fold_pack_kernel(const FoldPa
             return true;
         };
 
-        // The word (and HILO's second) of a segment: sum of xq and count, by what they hold: 0 both;
-        // after a redone segment's passes 1 counts (and hi), 2 the rest of the sums.
+        // The word (and HILO's second) of a segment that passed its check: sum of xq and count.
         using Sum = typename std::conditional<HILO, long long, int32_t>::type;
         const uint32_t ymask = (1u << pw.S) - 1u;
-        auto decode = [&](int what, uint32_t w, uint32_t w2, Sum &ds, uint32_t &dc) {
-            dc = what == 0 ? w >> pw.S : (what == 1 ? w : 0u);
-            if constexpr (HILO) {
-                ds = (long long)(int32_t)w2 * (1 << kLoBits) + (long long)(what == 0 ? w & ymask : (what == 1 ? 0u : w));
-            } else {
-                ds = what == 0 ? (int32_t)((w & ymask) - pw.L * dc) : (what == 2 ? (int32_t)w : 0);
-            }
+        auto decode = [&](uint32_t w, uint32_t w2, Sum &ds, uint32_t &dc) {
+            dc = w >> pw.S;
+            if constexpr (HILO) ds = (long long)(int32_t)w2 * (1 << kLoBits) + (long long)(w & ymask);
+            else ds = (int32_t)((w & ymask) - pw.L * dc);
         };
-        // Empty this warp's bins of group j into its totals (written, not added to, the first time).
-        auto flush = [&](int j, int what, bool first) {
+        // Empty this warp's bins of group j into its totals (written, not added to, the first time):
+        // words that passed; or, `raw` given, words that hold the counts beside the words before (mod
+        // 2^32, w - count x increment is the sum: it fits 32 bits; HILO's sum of lo is below 2^32 and
+        // its second word, from raw2 or as it is in shared memory, needs no count).
+        auto flush = [&](int j, bool first, const uint32_t *raw, const uint32_t *raw2) {
             const uint32_t a = group_rec(j);
             for (int b0 = blo; b0 < bhi; b0 += 8) {
                 const int nb = min(8, bhi - b0);
                 unsigned long long tot[8];
-                uint32_t cn[8];
+                uint32_t cn[8], rw[8], rw2[8];
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
+                    const size_t i = (size_t)(b0 + u) * ppc + 32 * j;
                     tot[u] = 0ull;
-                    cn[u] = 0u;
+                    cn[u] = rw[u] = rw2[u] = 0u;
                     if (u < nb && !first) {
-                        tot[u] = ws_tot[(size_t)(b0 + u) * ppc + 32 * j];
-                        if (wide) cn[u] = ws_cnt[(size_t)(b0 + u) * ppc + 32 * j];
+                        tot[u] = ws_tot[i];
+                        if (wide) cn[u] = ws_cnt[i];
                     }
+                    if (u < nb && raw) rw[u] = raw[i];
+                    if (HILO && u < nb && raw2) rw2[u] = raw2[i];
                 }
 #pragma unroll
                 for (int u = 0; u < 8; ++u) {
@@ -495,7 +512,15 @@ __global__ void __launch_bounds__(kPackThreads, 1) fold_pack_kernel(const FoldPa
                         Sum ds;
                         uint32_t dc;
                         const uint32_t w = a + (uint32_t)(b0 + u) * row;
-                        decode(what, lds_u32(w), HILO ? lds_u32(w + 128u) : 0u, ds, dc);
+                        const uint32_t v = lds_u32(w), v2 = HILO ? (raw2 ? rw2[u] : lds_u32(w + 128u)) : 0u;
+                        if (!raw) {
+                            decode(v, v2, ds, dc);
+                        } else {
+                            dc = v;
+                            if constexpr (HILO)
+                                ds = (long long)(int32_t)v2 * (1 << kLoBits) + (long long)(rw[u] - (v << pw.S));
+                            else ds = (int32_t)(rw[u] - v * pw.add());
+                        }
                         sts_u32(w, 0u);
                         if (HILO) sts_u32(w + 128u, 0u);
                         tot[u] += (unsigned long long)(long long)ds + (wide ? 0ull : (unsigned long long)dc * bias);
@@ -505,130 +530,208 @@ __global__ void __launch_bounds__(kPackThreads, 1) fold_pack_kernel(const FoldPa
                 }
             }
         };
-        // Group j's samples [i0, i1) (a failed segment) into its totals by two passes of plain words:
-        // counts, then sums. All threads together.
-        auto redo = [&](int j, int64_t i0, int64_t i1, bool first) {
-            const uint32_t a = group_rec(j), ab = a - (KIND == 0 ? kSlabPhase : 0u);
-            uint32_t fl = 0u, fh = 0u;
-            const int64_t k = k0 + 32 * j;
-            if (k < ge) {
-                const double q = 1099511627776.0 / p.periods[k];
-                if (q > 0.0 && q < 9223372036854775808.0) {  // (else reported above)
-                    const unsigned long long F = (unsigned long long)__double2ll_rn(q);
-                    fl = (uint32_t)F;
-                    fh = (uint32_t)(F >> 32);
-                }
-            }
+        // The words of group j (this warp's bins) put aside and cleared for the counts.
+        auto put_aside = [&](int j) {
+            const uint32_t a = group_rec(j);
             for (int b = blo; b < bhi; ++b) {
+                ws_raw[(size_t)b * ppc + 32 * j] = lds_u32(a + (uint32_t)b * row);
                 sts_u32(a + (uint32_t)b * row, 0u);
-                if (HILO) sts_u32(a + (uint32_t)b * row + 128u, 0u);
+            }
+        };
+        // Group j's samples [i0, i1) of a failed segment (i0 is a multiple of 256) counted plainly, its words
+        // being at raw (raw2), or put aside now; then into its totals. All threads together, a warp
+        // sixteen samples at a time, half of them loaded while the other half is folded.
+        auto redo = [&](int j, int64_t i0, int64_t i1, bool first, const uint32_t *raw, const uint32_t *raw2) {
+            const uint32_t ab = group_rec(j) - (KIND == 0 ? kSlabPhase : 0u);
+            uint32_t fl = 0u, fh = 0u;
+#pragma unroll
+            for (int q = 0; q < G; ++q)
+                if (q == j) {
+                    fl = Fl[q];
+                    fh = Fh[q];
+                }
+            if (!raw) {
+                put_aside(j);
+                raw = ws_raw;
             }
             __syncthreads();
-            const uint32_t unbias = HILO ? 0u : 0u - pw.add();
-#pragma unroll 1
-            for (int pass = 1; pass <= 2; ++pass) {
-#pragma unroll 4
-                for (int64_t i = i0 + warp; i < i1; i += kPackWarps) {
-                    const uint32_t tl = __ldg(p.smp.tau_lo + sbase + i), th = (uint32_t)__ldg(p.smp.tau_hi + sbase + i);
-                    const uint32_t x = (uint32_t)__ldg(p.smp.xq + sbase + i) + unbias;
-                    const uint32_t w =
-                        word_addr<KIND>(phase_hi(tl, th * fl, fl, fh), tl, fl, ab, (uint32_t)nbins, p.shift);
-                    if (!HILO) {
-                        word_add<KIND>(w, pass == 1 ? 1u : x);
-                    } else if (pass == 1) {  // counts and hi, then lo
-                        word_add<KIND>(w, 1u);
-                        word_add<KIND>(w + 128u, (uint32_t)((int32_t)x >> kLoBits));
-                    } else {
-                        word_add<KIND>(w, x & ((1u << kLoBits) - 1u));
-                    }
+            const uint32_t *gtl = p.smp.tau_lo + sbase;
+            const int32_t *gth = p.smp.tau_hi + sbase, *gtg = p.smp.thg + sbase / 16;
+            auto one = [&](uint32_t tl, uint32_t thF) {
+                word_add<KIND>(word_addr<KIND>(phase_hi(tl, thF, fl, fh), tl, fl, ab, (uint32_t)nbins, p.shift), 1u);
+            };
+            auto load = [&](int64_t h, uint4 (&A)[2]) {  // samples 8 h .. 8 h + 7 of the star
+#pragma unroll
+                for (int u = 0; u < 2; ++u) A[u] = __ldg(reinterpret_cast<const uint4 *>(gtl + 8 * h) + u);
+            };
+            auto half = [&](const uint4 (&A)[2], uint32_t thF) {
+#pragma unroll
+                for (int u = 0; u < 2; ++u) {
+                    one(A[u].x, thF);
+                    one(A[u].y, thF);
+                    one(A[u].z, thF);
+                    one(A[u].w, thF);
                 }
-                __syncthreads();
-                flush(j, pass, first && pass == 1);
-                __syncthreads();
+            };
+            const int64_t g1 = i1 >> 4;  // whole groups of sixteen
+            int64_t g = (i0 >> 4) + warp;
+            if (g < g1) {
+                uint4 A[2], B[2];
+                load(2 * g, A);
+                uint32_t th = (uint32_t)__ldg(gtg + g);
+#pragma unroll 1
+                for (; g < g1; g += kPackWarps) {
+                    const int64_t gn = min(g + kPackWarps, g1 - 1);  // (past the end: loaded, not used)
+                    load(2 * g + 1, B);
+                    const uint32_t thn = (uint32_t)__ldg(gtg + gn);
+                    if (th == 0x80000000u) {  // (the group's samples differ in their high word)
+#pragma unroll 1
+                        for (int u = 0; u < 16; ++u) one(__ldg(gtl + 16 * g + u), (uint32_t)__ldg(gth + 16 * g + u) * fl);
+                        load(2 * gn, A);
+                    } else {
+                        half(A, th * fl);
+                        load(2 * gn, A);
+                        half(B, th * fl);
+                    }
+                    th = thn;
+                }
             }
+            const int64_t i = 16 * g1 + warp;  // the star's last few
+            if (i < i1) one(__ldg(gtl + i), (uint32_t)__ldg(gth + i) * fl);
+            __syncthreads();
+            flush(j, first, raw, raw2);
         };
 
         uint32_t have = 0u;   // groups whose totals hold something
         uint32_t turn = 0u;   // checks made
         uint32_t stored = 0u;  // kPackSegs - 1 bits a group: its slots that count
-        if (ntiles > 0) push(0);
-        if (ntiles > 1) push(1);
-        for (int t = 0, rt = 1, seg = 0; t < ntiles; ++t) {
-            if (!fold_tile(t)) return;
-            if (t + 2 < ntiles) push(t + 2);
-            const bool last = t + 1 == ntiles, seg_end = last || rt == seg_tiles;
-            uint32_t due = 0u;  // groups whose segment ends here
+        int seg = 0;
+        for (int t0 = 0; t0 < ntiles; t0 += span_tiles) {
+            const int t1 = min(ntiles, t0 + span_tiles);
+            push(t0);
+            if (t0 + 1 < t1) push(t0 + 1);
+            for (int t = t0, rt = 1; t < t1; ++t) {
+                if (!fold_tile(t, std::false_type{}, 0u)) return;
+                if (t + 2 < t1) push(t + 2);
+                const bool last = t + 1 == ntiles, seg_end = t + 1 == t1 || rt == seg_tiles;
+                uint32_t due = 0u;  // groups whose segment ends here
+#pragma unroll
+                for (int j = 0; j < G; ++j) {
+                    const int len = (int)len_of(j);
+                    if (len != (int)kBlind && (seg_end || (len && rt % len == 0))) due |= 1u << j;
+                }
+                if (due) {
+                    const bool to_slot = slots && seg_end && !last;
+                    uint32_t *slot = ws_slot + (size_t)(HILO ? 2 * seg : seg) * plane;
+                    auto first_tile = [&](int j) {  // of group j's segment
+                        const int len = (int)len_of(j);
+                        return t + 1 - rt + (len ? (rt - 1) / len * len : 0);
+                    };
+                    // the check: every count at most M, and all samples counted; on the way the words
+                    // of a group that keeps to the block's segments go to their slot
+                    uint32_t bad = 0u;
+#pragma unroll 1
+                    for (int j = 0; j < G; ++j) {
+                        if (!((due >> j) & 1u)) continue;
+                        const uint32_t a = group_rec(j);
+                        uint32_t sum = 0u, big = 0u;
+                        const bool store = to_slot && !len_of(j);
+                        uint32_t *w = slot + 32 * j;
+#pragma unroll 4
+                        for (int b = blo; b < bhi; ++b) {
+                            const uint32_t v = lds_u32(a + (uint32_t)b * row), c = v >> pw.S;
+                            if (store) {
+                                w[(size_t)b * ppc] = v;
+                                sts_u32(a + (uint32_t)b * row, 0u);
+                                if (HILO) {
+                                    w[plane + (size_t)b * ppc] = lds_u32(a + (uint32_t)b * row + 128u);
+                                    sts_u32(a + (uint32_t)b * row + 128u, 0u);
+                                }
+                            }
+                            sum += c;
+                            big = max(big, c);
+                        }
+                        atomicAdd(&cnt_sum[32 * j + lane], sum);
+                        if (big > pw.M && ((live >> j) & 1u)) bad |= 1u << j;
+                    }
+                    __syncthreads();
+                    if (warp < G && ((due >> warp) & 1u)) {
+                        const int64_t n = min(nsamp, (int64_t)(t + 1) * tile) - (int64_t)first_tile(warp) * tile;
+                        if (cnt_sum[threadIdx.x] != (uint32_t)n && ((live >> warp) & 1u)) bad |= 1u << warp;
+                        cnt_sum[threadIdx.x] = 0u;
+                    }
+                    bad = __reduce_or_sync(0xffffffffu, bad);
+                    if (lane == 0 && bad) atomicOr(&sh.bad[turn & 1u], bad);
+                    if (threadIdx.x == 0) sh.bad[(turn + 1u) & 1u] = 0u;
+                    __syncthreads();
+                    bad = sh.bad[turn & 1u];
+                    ++turn;
+#pragma unroll 1
+                    for (int j = 0; j < G; ++j) {
+                        if (!((due >> j) & 1u)) continue;
+                        const bool first = !((have >> j) & 1u);
+                        const uint32_t len = len_of(j);
+                        if ((bad >> j) & 1u) {
+                            const bool stored_now = to_slot && !len;
+                            redo(j, (int64_t)first_tile(j) * tile, min(nsamp, (int64_t)(t + 1) * tile), first,
+                                 stored_now ? slot : nullptr, stored_now ? slot + plane : nullptr);
+                            have |= 1u << j;
+                            // what piled its samples up does so again: shorter segments from here on (a
+                            // boundary of the present length is one of the new length too), then none
+                            const uint32_t now =
+                                len ? len : (seg_tiles > 4 ? 8u : (seg_tiles > 2 ? 4u : (uint32_t)seg_tiles));
+                            const uint32_t cut = now > 1u ? now >> 1 : kBlind;
+                            own = (own & ~(31u << (5 * j))) | (cut << (5 * j));
+                            if (threadIdx.x == 0) sh.blind_from[j] = t + 1;
+                        } else if (to_slot && !len) {
+                            stored |= 1u << (seg + (kPackSegs - 1) * j);
+                        } else if (!last) {
+                            flush(j, first, nullptr, nullptr);
+                            have |= 1u << j;
+                        }
+                    }
+                    __syncthreads();  // emptied before the next tile's reductions, or the epilogue
+                }
+                if (seg_end) {
+                    rt = 1;
+                    ++seg;
+                } else {
+                    ++rt;
+                }
+            }
+            // blind groups: their words put aside, and their samples since then counted, all at once
+            uint32_t blind = 0u;
+            int from = t1;
 #pragma unroll
             for (int j = 0; j < G; ++j) {
-                const int len = (int)((own >> (5 * j)) & 31u);
-                if (seg_end || (len && rt % len == 0)) due |= 1u << j;
+                if (len_of(j) == kBlind && sh.blind_from[j] < t1) {
+                    blind |= 1u << j;
+                    from = min(from, sh.blind_from[j]);
+                }
             }
-            if (due) {
-                const bool to_slot = slots && seg_end && !last;
-                auto first_tile = [&](int j) {  // of group j's segment
-                    const int len = (int)((own >> (5 * j)) & 31u);
-                    return t + 1 - rt + (len ? (rt - 1) / len * len : 0);
-                };
-                // the check: every count at most M, and all samples counted; on the way the words
-                // of a group that keeps to the block's segments go to their slot
-                uint32_t bad = 0u;
+            if (blind) {
 #pragma unroll 1
-                for (int j = 0; j < G; ++j) {
-                    if (!((due >> j) & 1u)) continue;
-                    const uint32_t a = group_rec(j);
-                    uint32_t sum = 0u, big = 0u;
-                    const bool store = to_slot && !((own >> (5 * j)) & 31u);
-                    uint32_t *w = ws_slot + (size_t)(HILO ? 2 * seg : seg) * plane + 32 * j;
-#pragma unroll 4
-                    for (int b = blo; b < bhi; ++b) {
-                        const uint32_t v = lds_u32(a + (uint32_t)b * row), c = v >> pw.S;
-                        if (store) {
-                            w[(size_t)b * ppc] = v;
-                            sts_u32(a + (uint32_t)b * row, 0u);
-                            if (HILO) {
-                                w[plane + (size_t)b * ppc] = lds_u32(a + (uint32_t)b * row + 128u);
-                                sts_u32(a + (uint32_t)b * row + 128u, 0u);
-                            }
-                        }
-                        sum += c;
-                        big = max(big, c);
-                    }
-                    atomicAdd(&cnt_sum[32 * j + lane], sum);
-                    if (big > pw.M && ((live >> j) & 1u)) bad |= 1u << j;
-                }
+                for (int j = 0; j < G; ++j)
+                    if ((blind >> j) & 1u) put_aside(j);
                 __syncthreads();
-                if (warp < G && ((due >> warp) & 1u)) {
-                    const int64_t n = min(nsamp, (int64_t)(t + 1) * tile) - (int64_t)first_tile(warp) * tile;
-                    if (cnt_sum[threadIdx.x] != (uint32_t)n && ((live >> warp) & 1u)) bad |= 1u << warp;
-                    cnt_sum[threadIdx.x] = 0u;
+                push(from);
+                if (from + 1 < t1) push(from + 1);
+                for (int t = from; t < t1; ++t) {
+                    uint32_t mask = 0u;
+#pragma unroll
+                    for (int j = 0; j < G; ++j)
+                        if (((blind >> j) & 1u) && sh.blind_from[j] <= t) mask |= 1u << j;
+                    if (!fold_tile(t, std::true_type{}, mask)) return;
+                    if (t + 2 < t1) push(t + 2);
                 }
-                bad = __reduce_or_sync(0xffffffffu, bad);
-                if (lane == 0 && bad) atomicOr(&sh.bad[turn & 1u], bad);
-                if (threadIdx.x == 0) sh.bad[(turn + 1u) & 1u] = 0u;
-                __syncthreads();
-                bad = sh.bad[turn & 1u];
-                ++turn;
 #pragma unroll 1
-                for (int j = 0; j < G; ++j) {
-                    if (!((due >> j) & 1u)) continue;
-                    const bool first = !((have >> j) & 1u);
-                    if ((bad >> j) & 1u) {
-                        redo(j, (int64_t)first_tile(j) * tile, min(nsamp, (int64_t)(t + 1) * tile), first);
+                for (int j = 0; j < G; ++j)
+                    if ((blind >> j) & 1u) {
+                        flush(j, !((have >> j) & 1u), ws_raw, nullptr);
                         have |= 1u << j;
-                    } else if (to_slot && !((own >> (5 * j)) & 31u)) {
-                        stored |= 1u << (seg + (kPackSegs - 1) * j);
-                    } else if (!last) {
-                        flush(j, 0, first);
-                        have |= 1u << j;
+                        if (threadIdx.x == 0) sh.blind_from[j] = t1;
                     }
-                }
-                __syncthreads();  // emptied before the next tile's reductions, or the epilogue
-            }
-            if (seg_end) {
-                rt = 1;
-                ++seg;
-            } else {
-                ++rt;
+                __syncthreads();
             }
         }
 
@@ -658,7 +761,7 @@ __global__ void __launch_bounds__(kPackThreads, 1) fold_pack_kernel(const FoldPa
                     c[u] = 0u;
                     ds[u] = 0;
                     const uint32_t w = a + (uint32_t)(b0 + u) * row;
-                    if (b0 + u < bhi) decode(0, lds_u32(w), HILO ? lds_u32(w + 128u) : 0u, ds[u], c[u]);
+                    if (b0 + u < bhi) decode(lds_u32(w), HILO ? lds_u32(w + 128u) : 0u, ds[u], c[u]);
                 }
                 if (slots) {
                     // (a star of at most one chunk: without HILO its bin sums are 32-bit integers)
@@ -679,7 +782,7 @@ __global__ void __launch_bounds__(kPackThreads, 1) fold_pack_kernel(const FoldPa
                         for (int u = 0; u < kEpi; ++u) {
                             Sum es;
                             uint32_t ec;
-                            decode(0, w[q][0][u], w[q][W - 1][u], es, ec);
+                            decode(w[q][0][u], w[q][W - 1][u], es, ec);
                             ds[u] += es;
                             c[u] += ec;
                         }

@@ -32,6 +32,7 @@ struct StarStats {
     int32_t n;      // samples of the star
     long long dtau0;  // smallest positive step between consecutive quantised times (0: none)
     int32_t qexp;     // fixed-point flux: xq = rint(x 2^qexp), |xq| <= (2^31 - 1) / chunk
+    int32_t nreg;     // steps of about dtau0 inside the 16-sample groups
     int32_t wide;     // the flux spreads too widely for 31 bits of its largest value (prep)
     int32_t pad;
 };
@@ -149,10 +150,10 @@ cudaError_t launch_fold(const FoldParams &p, int mode, int grid, cudaStream_t st
 constexpr int kPackMaxGroups = 6;
 constexpr int kPackChunk = 65520;
 constexpr int kPackSegs = 4;                  // segments of a star whose words go to slots
-// 32-bit words of workspace (ws_sc) per bin and period of a resident block: totals (3) and slots
-// (below 256 bins two words each)
-constexpr int kPackPlanes = 3 + kPackSegs - 1;
-constexpr int kPackPlanesHilo = 3 + 2 * (kPackSegs - 1);
+// 32-bit words of workspace (ws_sc) per bin and period of a resident block: totals (3), slots
+// (below 256 bins two words each) and words put aside
+constexpr int kPackPlanes = 3 + kPackSegs;
+constexpr int kPackPlanesHilo = 4 + 2 * (kPackSegs - 1);
 constexpr int kPackMinBins = 32;
 // prep's chunk below 256 bins: flux in 31 bits (the bound of two samples' sum)
 constexpr int kPackHiloChunk = 2;

@@ -176,6 +176,24 @@ def test_one_word_fold_equals_two_words(ctx, n, kind, n_periods, nbins, groups):
     assert torch.equal(torch.nan_to_num(one[0], 7.0), torch.nan_to_num(two[0], 7.0))
 
 
+def test_one_word_fold_of_hard_periods_takes_at_most_a_second_turn(ctx):
+    """Periods all within 10^-4 of seven cadences (every sample in seven bins), and times without a cadence,
+    against periods that spread the samples: no sample is folded more than twice, but for a failed segment."""
+    import paper_2312_02063_gb300 as g
+    rng = np.random.default_rng(5)
+    f = (1.0 + rng.normal(0.0, 3e-4, 65000)).astype(np.float32)
+    easy, narrow = np.linspace(24.5, 4900.0, 29184) * CADENCE, np.linspace(6.999, 7.001, 29184) * CADENCE
+    t = []
+    ctx.set_fold_config(**_one_word(g, 6))
+    try:
+        for kind, p in (("regular", easy), ("regular", narrow), ("random", easy)):
+            args = [_dev(ctx, x) for x in (_times(kind, 65000, rng), f, p)]
+            t.append(_ms(ctx, lambda: g.gpfc_fold(ctx, *args, 256, 0.0)))  # noqa: B023
+    finally:
+        ctx.reset_fold_config()
+    assert t[1] <= 2.2 * t[0] and t[2] <= 1.2 * t[0]
+
+
 def test_decision_of_several_stars_takes_no_longer_than_of_many(ctx):
     """19 stars of 16,384 periods: a block each, not clusters that take turns."""
     import paper_2312_02063_gb300 as g
