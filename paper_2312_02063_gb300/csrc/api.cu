@@ -194,6 +194,10 @@ const gpfc_ctx::Tuned *find_tuned(const gpfc_ctx *ctx, int nbins, int mode, int6
     return nullptr;
 }
 
+// What the fold gives: scores, profiles for a scorer (the plan may be the one-word fold's) or
+// profiles for the caller (so too below 256 bins).
+enum FoldOut { kScores, kForBox, kForCnn, kForCaller };
+
 // The one-word fold named by its own shape, as gpfc_last_fold_plan and the autotuner give it out: its
 // sixteen warps are streams of no period group of their own, so one stream a group, which the
 // two-word fold's plans never have.
@@ -203,38 +207,56 @@ bool pack_named(const gpfc_fold_config &c)
            (c.chunk == 0 || c.chunk == kPackChunk);
 }
 
-// Whether a fold that writes profiles may take the one-word form of layout 3: wherever that
-// layout is the default (or set), fits (else the FP32 layout runs) and nothing else about the
-// launch is set, or its own shape. Its results are the layout's own, and it was the faster one at every size
-// measured: 192 periods of 62,835 samples and 256 bins in 1.04 M cycles of a multiprocessor,
-// against 2 x 0.755 M (fold_pack.cu); searches by CNN, two words -> one: 250,000 periods
-// 9.6 -> 8.4 ms, 100,000 periods 4.1 -> 3.8 ms.
-bool pack_ok(const gpfc_ctx *ctx, int nbins)
+// Whether a fold that writes profiles can take the one-word form of layout 3 (the same results): 256 or
+// 512 bins, where its own shape or nothing but the layout is set.
+bool pack_fits(const gpfc_ctx *ctx, int nbins)
 {
     const gpfc_fold_config &c = ctx->fold_cfg;
     const bool automatic = (c.layout == 0 || c.layout == kLayoutRed32) && c.warps == 0 && c.chunk == 0 && c.tile == 0 &&
                            c.blocks_per_sm == 0 && c.streams == 0;
-    return default_layout(nbins) == kLayoutRed32 && (automatic || pack_named(c)) &&
-           fold_max_warps(nbins, kLayoutRed32, kTile) >= 1 && fold_pack_groups(nbins, ctx->window) >= 1;
+    return nbins >= 256 && (automatic || pack_named(c)) && fold_pack_groups(nbins, ctx->window) >= 1;
+}
+
+// Whether it is the faster form for np periods of nstars stars of about n samples. A block takes 192
+// periods at a time where the two-word fold's takes 96, and has more to set up and to finish: it pays
+// where there are samples enough, and periods for several launches (or, with 512 bins, of which the
+// two-word fold's blocks hold one group, soon). Times of the two folds in the same call, one word / two,
+// regular cadence with gaps, grids through its multiples:
+//   256 bins, one star, 16,000 to 65,000 samples: box search, widths to 108, 0.84..0.98 from 45,000
+//     periods (to 32 0.80..1.03) and 0.95..1.15 from 2,000 to 30,000; CNN 0.79..0.97 and 0.92..1.1.
+//     2,000 to 8,000 samples: 0.91..1.1 at any grid.
+//   256 bins, batches: 0.75..0.98 from 14,000 samples a star and 44,000 periods in all; 0.81..1.18 below.
+//   256 bins, profiles to the caller: 0.66..1.0 from 24,000 samples and 15,000 periods, 1.05..1.4 below.
+//   512 bins: searches 0.61..0.93 from 10,000 periods in all at any length, 0.8..1.16 below; profiles to
+//     the caller 0.78..0.97 from 24,000 samples and 10,000 periods, 0.75..1.2 below.
+constexpr int64_t kPackScored = 14000, kPackCaller = 24000;
+bool pack_pays(const gpfc_ctx *ctx, int64_t n, int64_t np, int nbins, FoldOut out)
+{
+    const int64_t group = (int64_t)32 * ctx->num_sms;  // a group of 32 periods for every multiprocessor
+    if (out == kForCaller) return n >= kPackCaller && np >= (nbins == 512 ? 2 : 3) * group;
+    return nbins == 512 ? np >= 2 * group : n >= kPackScored && np >= 9 * group;
 }
 
 // Below 256 bins the one-word fold takes the place of the FP32 layouts, with flux in 31 bits, where
-// the caller gets the profiles and set nothing: measured, 12,345 periods of 28,800 samples and 200
-// bins, 747 -> 416 us (one warp a group of 32 periods waits out a read-modify-write per sample; here
-// sixteen share it). Below kPackMinBins a segment holds too few samples for its check to pay. A
-// search keeps the FP32 sums: its scores would change in their last bits.
-bool hilo_ok(const gpfc_ctx *ctx, int nbins)
+// the caller gets the profiles and set nothing. One word / FP32, 32 to 255 bins, by the groups of 32
+// periods a multiprocessor has: one 0.09..1.0 from 100 samples (there one warp a group waits out a
+// read-modify-write per sample; here sixteen share it), two and three 0.13..0.95 from 2,000 samples
+// (0.8..1.45 at 100 and 500), more, where the FP32 fold has many groups in flight, 0.24..0.89 from 16,000
+// samples (up to 1.6 at 2,000). Below kPackMinBins a segment holds too few samples for its check
+// to pay. A search keeps the FP32 sums: its scores would change in their last bits.
+bool hilo_ok(const gpfc_ctx *ctx, int64_t n, int64_t np, int nbins)
 {
     const gpfc_fold_config &c = ctx->fold_cfg;
+    const int64_t per_sm = (np + (int64_t)32 * ctx->num_sms - 1) / ((int64_t)32 * ctx->num_sms);
     return nbins >= kPackMinBins && nbins < 256 && c.layout == 0 && c.warps == 0 && c.chunk == 0 && c.tile == 0 &&
-           c.blocks_per_sm == 0 && c.streams == 0;
+           c.blocks_per_sm == 0 && c.streams == 0 && (per_sm <= 1 || n >= (per_sm <= 3 ? 2000 : 16000));
 }
 
 // Its plan over np periods in nstars grids of about equal length. A block takes as many
 // period groups as fit (each sample is read once for all), fewer where the grid would leave
 // multiprocessors idle, or where a star's last block would be mostly empty: the cost of a
 // star's blocks is taken as their period groups plus one each for the reading.
-FoldPlan plan_packed(const gpfc_ctx *ctx, int64_t n, int64_t np, int nbins, int64_t nstars)
+FoldPlan plan_packed(const gpfc_ctx *ctx, int64_t n, int64_t np, int nbins, int64_t nstars, FoldOut out)
 {
     FoldPlan pl{};
     pl.packed = 1;
@@ -248,12 +270,14 @@ FoldPlan plan_packed(const gpfc_ctx *ctx, int64_t n, int64_t np, int nbins, int6
     pl.warps = maxg;
     if (ctx->fold_cfg.warps > 0) {
         pl.warps = std::min(ctx->fold_cfg.warps, fold_pack_groups(nbins, ctx->window));
-    } else if (nstars > 1) {
+    } else if (nstars > 1 || out == kForCaller) {
+        // (of a single star all blocks go in one launch, in whole waves of the multiprocessors)
         const int64_t avg = std::max<int64_t>(1, np / nstars);
         int64_t best = INT64_MAX;
         for (int g = maxg; g >= 1; --g) {
             if (fold_pack_allowed(nbins, g) != g) continue;
-            const int64_t cost = (avg + 32 * g - 1) / (32 * g) * (g + 1);
+            const int64_t blocks = (avg + 32 * g - 1) / (32 * g);
+            const int64_t cost = (nstars > 1 ? blocks : (blocks + ctx->num_sms - 1) / ctx->num_sms) * (g + 1);
             if (cost < best) {
                 best = cost;
                 pl.warps = g;
@@ -313,25 +337,23 @@ FoldPlan plan_with(const gpfc_ctx *ctx, int64_t n, int64_t np, int nbins, const 
     return pl;
 }
 
-// What the fold gives: scores, profiles for a scorer (the plan may be the one-word fold's) or
-// profiles for the caller (so too below 256 bins).
-enum FoldOut { kScores, kForScorer, kForCaller };
 // The plan, and (below 256 bins, beside the one-word fold's) the FP32 plan of the same fold, else
 // the same plan again.
 FoldPlan plan_fold(gpfc_ctx *ctx, int64_t n, int64_t np, int nbins, const gpfc_ctx::Tuned *tuned, FoldOut out,
                    int64_t nstars = 1, FoldPlan *general = nullptr)
 {
     gpfc_fold_config cfg = ctx->fold_cfg;
-    if (tuned && !tuned->packed) {
+    if (tuned) {
         if (!cfg.warps) cfg.warps = tuned->cfg.warps;
         if (!cfg.layout) cfg.layout = tuned->cfg.layout;
         if (!cfg.tile) cfg.tile = tuned->cfg.tile;
         if (!cfg.blocks_per_sm) cfg.blocks_per_sm = tuned->cfg.blocks_per_sm;
     }
-    const bool packed = (out != kScores && pack_ok(ctx, nbins) &&
-                         (pack_named(ctx->fold_cfg) || !tuned || tuned->packed)) ||
-                        (out == kForCaller && hilo_ok(ctx, nbins));
-    const FoldPlan pl = packed ? plan_packed(ctx, n, np, nbins, nstars) : plan_with(ctx, n, np, nbins, cfg);
+    const bool packed = (out != kScores && pack_fits(ctx, nbins) &&
+                         (pack_named(ctx->fold_cfg) ||
+                          (pack_pays(ctx, n, np, nbins, out) && (!tuned || tuned->packed)))) ||
+                        (out == kForCaller && hilo_ok(ctx, n, np, nbins));
+    const FoldPlan pl = packed ? plan_packed(ctx, n, np, nbins, nstars, out) : plan_with(ctx, n, np, nbins, cfg);
     // (below 256 bins the FP32 plan, which is launched behind the one-word fold: layout 3 set by hand
     // there would cut the flux to its chunk's fixed point)
     const FoldPlan r = packed && nbins < 256 ? plan_with(ctx, n, np, nbins, cfg) : pl;
@@ -807,7 +829,7 @@ int run_search_box_warp(gpfc_ctx *ctx, const double *times, const float *flux, i
                         int64_t np, int32_t nbins, double t0, const gpfc_box_params *bp, float *score,
                         int64_t *best_index, float *best_score)
 {
-    const FoldPlan pl = plan_fold(ctx, n, np, nbins, find_tuned(ctx, nbins, kModeFold, n), kForScorer);
+    const FoldPlan pl = plan_fold(ctx, n, np, nbins, find_tuned(ctx, nbins, kModeFold, n), kForBox);
     const int64_t chunk = std::min<int64_t>(np, (int64_t)pl.grid * pl.ppc);
     FoldBuffers fb{};
     int rc = ensure_ws(ctx, box_warp_bytes(pl, n, np, nbins));
@@ -899,7 +921,7 @@ int run_search_cnn(gpfc_ctx *ctx, const double *times, const float *flux, int64_
                    int64_t np, int32_t nbins, double t0, const gpfc_cnn_weights *wt, float *score,
                    int64_t *best_index, float *best_score)
 {
-    const FoldPlan pl = plan_fold(ctx, n, np, nbins, find_tuned(ctx, nbins, kModeFold, n), kForScorer);
+    const FoldPlan pl = plan_fold(ctx, n, np, nbins, find_tuned(ctx, nbins, kModeFold, n), kForCnn);
     const int64_t wave = (int64_t)pl.grid * pl.ppc;
     const int64_t chunk = std::min<int64_t>(np, wave);
     const int64_t half = (chunk + 1) / 2;
@@ -1030,9 +1052,9 @@ int tune_fold(gpfc_ctx *ctx, const double *times, const float *flux, int64_t n, 
             }
         }
     }
-    if (mode == kModeFold && pack_ok(ctx, nbins)) cands.push_back(Cand{gpfc_fold_config{}, best_res, true});
+    if (mode == kModeFold && pack_fits(ctx, nbins)) cands.push_back(Cand{gpfc_fold_config{}, best_res, true});
     auto plan_of = [&](const Cand &c) {
-        return c.packed ? plan_packed(ctx, n, P, nbins, 1) : plan_with(ctx, n, P, nbins, c.cfg);
+        return c.packed ? plan_packed(ctx, n, P, nbins, 1, kForBox) : plan_with(ctx, n, P, nbins, c.cfg);
     };
     if (cands.empty()) return set_err(ctx, GPFC_ENOTSUP, "no fold launch config fits nbins = %d", nbins);
     // workspace: the largest carve of any candidate plus the sample score buffer
@@ -1585,7 +1607,7 @@ int gpfc_workspace_size(gpfc_ctx *ctx, int64_t n, int64_t n_periods, int32_t nbi
     // and the one-kernel search; planning them leaves the context's last plan as it was
     const gpfc_fold_config last = ctx->last_plan;
     const FoldPlan pb = plan_fold(ctx, n, n_periods, nbins, find_tuned(ctx, nbins, kModeBox, n), kScores);
-    const FoldPlan pf = plan_fold(ctx, n, n_periods, nbins, find_tuned(ctx, nbins, kModeFold, n), kForScorer);
+    const FoldPlan pf = plan_fold(ctx, n, n_periods, nbins, find_tuned(ctx, nbins, kModeFold, n), kForBox);
     FoldPlan pg{};
     const FoldPlan pc = plan_fold(ctx, n, n_periods, nbins, find_tuned(ctx, nbins, kModeFold, n), kForCaller, 1, &pg);
     FoldBuffers fb{};
@@ -2219,7 +2241,9 @@ int gpfc_search_batched(gpfc_ctx *ctx, int32_t n_stars, const int64_t *lc_offset
     const bool capturing = cs != cudaStreamCaptureStatusNone;
     const int64_t n_avg = n_total / n_stars;
     const gpfc_ctx::Tuned *tuned = find_tuned(ctx, nbins, mode, n_avg);
-    const bool pack = mode == kModeFold && pack_ok(ctx, nbins);
+    const FoldOut fold_out = mode != kModeFold ? kScores : (scorer == GPFC_SCORER_CNN ? kForCnn : kForBox);
+    const bool pack = mode == kModeFold && pack_fits(ctx, nbins) &&
+                      (pack_named(ctx->fold_cfg) || pack_pays(ctx, n_avg, n_periods_total, nbins, fold_out));
     if (!tuned && ctx->autotune && !capturing && !pack) {
         // tune on the first star (its offsets are read back once)
         int64_t off[2] = {0, 0};
@@ -2235,7 +2259,7 @@ int gpfc_search_batched(gpfc_ctx *ctx, int32_t n_stars, const int64_t *lc_offset
         }
     }
     FoldPlan pl = plan_fold(ctx, n_avg, n_periods_total, nbins, tuned,
-                            mode == kModeFold ? kForScorer : kScores, n_stars);
+                            fold_out, n_stars);
     if (A.box_warp && ctx->box_path != GPFC_BOX_WARP && !(pl.packed && ctx->box_path == GPFC_BOX_AUTO)) {
         // the one-kernel search, with the tuned fold config if its block fits, else the
         // default one

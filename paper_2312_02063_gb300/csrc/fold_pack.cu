@@ -91,8 +91,8 @@ __device__ __forceinline__ uint32_t phase_hi(uint32_t tl, uint32_t thF, uint32_t
     return h;
 }
 
-// Shared address of a sample's bin word for one period (KIND 0: 256 bins, 1: a power of two,
-// 2: any; 3 and 4: below 256 bins, HILO, a power of two or any). With 256 bins the bin is the top
+// Shared address of a sample's bin word for one period (KIND 0: 256 bins, 1: a larger power of two;
+// 2 and 3: below 256 bins, HILO, a power of two or any). With 256 bins the bin is the top
 // byte of the phase and rows are 256 bytes, so one byte permutation builds the address: byte 0 =
 // lane and group parity, byte 1 = bin, the rest the slab; the slab's distance from a multiple of
 // 64 KB is the reduction's immediate offset.
@@ -102,10 +102,10 @@ __device__ __forceinline__ uint32_t word_addr(uint32_t hi, uint32_t tl, uint32_t
 {
     if (KIND == 0) return __byte_perm(hi, base, 0x7634);
     if (KIND == 1) return base + ((hi >> shift) << 7);
-    if (KIND == 3) return base + ((hi >> shift) << 8);
+    if (KIND == 2) return base + ((hi >> shift) << 8);
     const uint32_t lo = tl * Fl;
     const unsigned long long t = (unsigned long long)hi * nbins + (unsigned long long)__umulhi(lo, nbins);
-    return base + ((uint32_t)(t >> 32) << (KIND == 4 ? 8 : 7));
+    return base + ((uint32_t)(t >> 32) << 8);
 }
 
 template <int KIND>
@@ -129,7 +129,7 @@ constexpr int kLoBits = 15;
 template <int KIND>
 __device__ __forceinline__ void sample_add(uint32_t a, uint32_t x, uint32_t one)
 {
-    if (KIND >= 3) {
+    if (KIND >= 2) {
         asm volatile("red.shared.add.u32 [%0], %1;" ::"r"(a), "r"((x & ((1u << kLoBits) - 1u)) + one) : "memory");
         asm volatile("red.shared.add.u32 [%0+128], %1;" ::"r"(a), "r"((uint32_t)((int32_t)x >> kLoBits)) : "memory");
     } else {
@@ -177,7 +177,7 @@ __global__ void __launch_bounds__(kPackThreads, 1) fold_pack_kernel(const FoldPa
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int nbins = p.nbins;
     constexpr int ppc = 32 * G;  // G = p.warps period groups
-    if (KIND >= 3 && p.when == 1 && p.stats[0].wide) return;  // (the FP32 fold's)
+    if (KIND >= 2 && p.when == 1 && p.stats[0].wide) return;  // (the FP32 fold's)
     const uint32_t base = smem_u32(smem);
     const uint32_t rec = pack_records_addr(base, nbins);
     const uint32_t rec_bytes = pack_records_bytes(nbins, G);
@@ -188,7 +188,7 @@ __global__ void __launch_bounds__(kPackThreads, 1) fold_pack_kernel(const FoldPa
         return;
     }
     // row stride of a bin and start of period group j's words (lane's own)
-    constexpr bool HILO = KIND >= 3;
+    constexpr bool HILO = KIND >= 2;
     constexpr uint32_t row = KIND == 0 || HILO ? 256u : 128u;
     auto group_rec = [&](int j) {
         return (KIND == 0 ? rec + (uint32_t)(j >> 1) * kSlab + (uint32_t)(j & 1) * 128u
@@ -846,32 +846,33 @@ static size_t fold_pack_smem(int nbins, int groups, uint32_t window)
 
 int fold_pack_groups(int nbins, uint32_t window)
 {
+    if (nbins > 256 && nbins != 512) return 0;
     int g = kPackMaxGroups;
     while (g > 0 && fold_pack_smem(nbins, g, window) > kSmemLimit) --g;
     return fold_pack_allowed(nbins, g);
 }
 
 // f(kernel) for the instance of these bins and groups (each kind with the groups it can hold;
-// HILO with 1, 2, 3 or 6)
+// HILO with all but 5)
 template <int KIND, int G, class F>
 static cudaError_t with_groups(int groups, F f)
 {
     if constexpr (G < 1) return cudaErrorInvalidValue;
     else if (groups == G) return f(fold_pack_kernel<KIND, G>);
-    else return with_groups<KIND, (KIND >= 3 && G == 6 ? 3 : G - 1)>(groups, f);
+    else return with_groups<KIND, (KIND >= 2 && G == 6 ? 4 : G - 1)>(groups, f);
 }
 template <class F>
 static cudaError_t with_kernel(int nbins, int shift, int groups, F f)
 {
     if (nbins < 256)
-        return shift >= 0 ? with_groups<3, kPackMaxGroups>(groups, f) : with_groups<4, kPackMaxGroups>(groups, f);
+        return shift >= 0 ? with_groups<2, kPackMaxGroups>(groups, f) : with_groups<3, kPackMaxGroups>(groups, f);
     if (nbins == 256) return with_groups<0, kPackMaxGroups>(groups, f);
-    if (shift >= 0) return with_groups<1, 3>(groups, f);  // 512 bins: 64 KB a group
-    return with_groups<2, 5>(groups, f);                  // 257 bins and more
+    if (nbins == 512) return with_groups<1, 3>(groups, f);  // 64 KB a group
+    return cudaErrorInvalidValue;
 }
 
-// (4 and 5 have no HILO instance: a grid of that few periods a multiprocessor takes 3)
-int fold_pack_allowed(int nbins, int groups) { return nbins < 256 && (groups == 4 || groups == 5) ? 3 : groups; }
+// (5 has no HILO instance: a grid of that few periods a multiprocessor takes 4)
+int fold_pack_allowed(int nbins, int groups) { return nbins < 256 && groups == 5 ? 4 : groups; }
 
 int fold_pack_register()
 {
@@ -882,7 +883,6 @@ int fold_pack_register()
     for (int g = 1; g <= kPackMaxGroups && e == cudaSuccess; ++g) {
         e = with_kernel(256, 24, g, attr);
         if (e == cudaSuccess && g <= 3) e = with_kernel(512, 23, g, attr);
-        if (e == cudaSuccess && g <= 5) e = with_kernel(300, -1, g, attr);
         if (e == cudaSuccess && fold_pack_allowed(64, g) == g) e = with_kernel(64, 26, g, attr);
         if (e == cudaSuccess && fold_pack_allowed(64, g) == g) e = with_kernel(100, -1, g, attr);
     }

@@ -194,6 +194,101 @@ def test_one_word_fold_of_hard_periods_takes_at_most_a_second_turn(ctx):
     assert t[1] <= 2.2 * t[0] and t[2] <= 1.2 * t[0]
 
 
+# below 256 bins with many groups a multiprocessor (5 groups have no instance of their own)
+@pytest.mark.parametrize("n_periods,nbins", [(24000, 64), (24000, 100), (60011, 32)])
+def test_fold_below_256_bins_of_long_grids(ctx, n_periods, nbins):
+    import paper_2312_02063_gb300 as g
+    rng = np.random.default_rng(nbins)
+    n = 24001
+    f = (1.0 + rng.normal(0.0, 3e-4, n)).astype(np.float32)
+    args = [_dev(ctx, x) for x in (_times("gaps", n, rng), f, rng.uniform(0.05, 1.0, n_periods))]
+    a, ca = g.gpfc_fold(ctx, *args, nbins, 0.0)
+    ctx.set_fold_config(layout=1)
+    try:
+        b, cb = g.gpfc_fold(ctx, *args, nbins, 0.0)
+    finally:
+        ctx.reset_fold_config()
+    ctx.sync()
+    assert torch.equal(ca, cb) and torch.equal(torch.isfinite(a), torch.isfinite(b))
+    assert not torch.equal(torch.nan_to_num(a, 7.0), torch.nan_to_num(b, 7.0))  # (another sum: the one-word fold ran)
+    assert float((torch.nan_to_num(a, 1.0) - torch.nan_to_num(b, 1.0)).abs().max()) <= 2.0 ** -22
+
+
+def test_plans_of_the_one_word_fold_name_it(ctx):
+    """The plan given out, set by hand, is the same fold of the same shape; so is the autotuner's."""
+    import paper_2312_02063_gb300 as g
+    rng = np.random.default_rng(3)
+    n = 62000
+    f = (1.0 + rng.normal(0.0, 3e-4, n)).astype(np.float32)
+    args = [_dev(ctx, x) for x in (_times("gaps", n, rng), f, np.linspace(0.2, 1.0, 30000))]
+    for two_words in (False, True):
+        p = args[2][:2000] if two_words else args[2]
+        try:
+            a = g.gpfc_fold(ctx, args[0], args[1], p, 256, 0.0)
+            plan = ctx.last_fold_plan()
+            assert (plan["streams"] == 1) != two_words
+            ctx.set_fold_config(**plan)
+            b = g.gpfc_fold(ctx, args[0], args[1], p, 256, 0.0)
+            assert ctx.last_fold_plan() == plan
+        finally:
+            ctx.reset_fold_config()
+        ctx.sync()
+        assert torch.equal(a[1], b[1]) and torch.equal(torch.nan_to_num(a[0], 7.0), torch.nan_to_num(b[0], 7.0))
+    try:
+        cfg = g.gpfc_autotune(ctx, *args, 256, g.SCORER_BOX, 1, 40, 0.0)
+        ref, _, _ = g.gpfc_search(ctx, *args, 256, 0.0, g.SCORER_BOX, 1, 40, 0.0)
+        plan = ctx.last_fold_plan()
+        ctx.set_autotune(-1)
+        ctx.set_fold_config(**cfg)
+        sc, _, _ = g.gpfc_search(ctx, *args, 256, 0.0, g.SCORER_BOX, 1, 40, 0.0)
+        assert ctx.last_fold_plan() == plan
+    finally:
+        ctx.reset_fold_config()
+        ctx.set_autotune(-1)
+        ctx.set_autotune(1)
+    ctx.sync()
+    assert torch.equal(ref, sc)
+
+
+# the automatic fold against the two-word fold's automatic shape: no slower, wherever the periods lie
+# about the cadence, whatever the times, short and long (a fifth for noise)
+@pytest.mark.parametrize("n,kind,n_periods,nbins", [
+    (100, "regular", 40, 256), (1000, "regular", 60000, 256), (3000, "random", 20000, 256), (3000, "random", 20000, 512),
+    (20000, "gaps", 10000, 256), (20000, "gaps", 10000, 300), (65000, "gaps", 1000, 256), (65000, "gaps", 10000, 512),
+    (65000, "gaps", 30000, 256), (65000, "random", 30000, 256), (65000, "barycentric", 30000, 512), (5000, "gaps", 20000, 700)])
+def test_automatic_fold_is_no_slower_than_two_words(ctx, n, kind, n_periods, nbins):
+    import paper_2312_02063_gb300 as g
+    rng = np.random.default_rng(n)
+    f = (1.0 + rng.normal(0.0, 3e-4, n)).astype(np.float32)
+    args = [_dev(ctx, x) for x in (_times(kind, n, rng), f, 1.0 / np.linspace(1.0, 5.0, n_periods))]
+    call = lambda: g.gpfc_fold(ctx, *args, nbins, 0.0)  # noqa: E731
+    auto = _ms(ctx, call)
+    per_sm = -(-n_periods // (32 * ctx.num_sms))
+    ctx.set_fold_config(warps=max(1, min(per_sm, ctx.fold_max_warps(nbins, 3))), layout=g.LAYOUT_RED32)
+    try:
+        two = _ms(ctx, call)
+    finally:
+        ctx.reset_fold_config()
+    assert auto <= 1.2 * two
+
+
+@pytest.mark.parametrize("n,n_periods,nbins", [(100, 60000, 64), (1000, 60000, 32), (2000, 20000, 200), (24000, 60000, 100),
+                                               (65000, 10000, 64), (300, 3000, 128)])
+def test_automatic_fold_below_256_bins_is_no_slower_than_fp32(ctx, n, n_periods, nbins):
+    import paper_2312_02063_gb300 as g
+    rng = np.random.default_rng(n)
+    f = (1.0 + rng.normal(0.0, 3e-4, n)).astype(np.float32)
+    args = [_dev(ctx, x) for x in (_times("gaps", n, rng), f, 1.0 / np.linspace(1.0, 5.0, n_periods))]
+    call = lambda: g.gpfc_fold(ctx, *args, nbins, 0.0)  # noqa: E731
+    auto = _ms(ctx, call)
+    ctx.set_fold_config(layout=1)
+    try:
+        fp32 = _ms(ctx, call)
+    finally:
+        ctx.reset_fold_config()
+    assert auto <= 1.2 * fp32
+
+
 def test_decision_of_several_stars_takes_no_longer_than_of_many(ctx):
     """19 stars of 16,384 periods: a block each, not clusters that take turns."""
     import paper_2312_02063_gb300 as g
