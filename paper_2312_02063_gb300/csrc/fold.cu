@@ -145,7 +145,7 @@ __global__ void prep_quant_kernel(const double *times, const float *flux, const 
     const int64_t j0 = (int64_t)blockIdx.x * per;
     const int64_t j1 = min(len, j0 + per);
     double acc = 0.0;
-    float amax = 0.f;  // largest |x| of this block's samples
+    float amax = 0.f;  // largest finite |x| of this block's samples
     bool bad = false;
     long long dmin = LLONG_MAX;  // smallest positive step tau_j - tau_{j-1}
     for (int64_t j = j0 + threadIdx.x; j < j1; j += blockDim.x) {
@@ -158,7 +158,7 @@ __global__ void prep_quant_kernel(const double *times, const float *flux, const 
         smp.tau_hi[base + j] = (int32_t)(tau >> 32);
         const double d = (double)flux[b + j] - f_ref;
         smp.x[base + j] = (float)d;
-        amax = fmaxf(amax, fabsf((float)d));
+        if (isfinite((float)d)) amax = fmaxf(amax, fabsf((float)d));
         acc += d * d;
     }
     if (bad) report_error(status, kErrRange);
@@ -299,11 +299,15 @@ __global__ void prep_flags_kernel(const int64_t *lc_off, int64_t n, SampleScratc
         }
         if (smp.xq) {
             // fixed-point flux (exact: scaling by a power of two, then rounding to nearest
-            // even); zero past the star's end
+            // even); zero past the star's end, and for an x that is no number or infinite (a mean flux
+            // that is neither makes every x so), which no fixed point holds: the one-word fold needs
+            // every |xq| within the star's bound to count right
             const double sc = ldexp(1.0, stats[s].qexp);
-            for (int k = 0; k < 16; ++k)
-                smp.xq[base + j0 + k] =
-                    j0 + k < len ? (int32_t)((uint32_t)__double2int_rn((double)smp.x[base + j0 + k] * sc) + add) : 0;
+            for (int k = 0; k < 16; ++k) {
+                const float x = j0 + k < len ? smp.x[base + j0 + k] : 0.f;
+                const int32_t q = isfinite(x) ? __double2int_rn((double)x * sc) : 0;
+                smp.xq[base + j0 + k] = j0 + k < len ? (int32_t)((uint32_t)q + add) : 0;
+            }
         }
     }
     steps = __reduce_add_sync(0xffffffffu, steps);

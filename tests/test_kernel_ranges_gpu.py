@@ -93,6 +93,40 @@ def test_generated_profiles_of_wide_ranges(ctx, sigma, depth, n_cad):
     assert np.sqrt((np.concatenate(err) ** 2).mean()) <= 2.0 ** -23 / 12 ** 0.5
 
 
+# ---------------------------------------------------------------- flux
+
+@pytest.mark.parametrize("nbins", [256, 300, 512])
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+@pytest.mark.parametrize("width", [1.0, 0.5, 0.125])
+def test_counts_with_a_flux_that_is_no_number(ctx, nbins, bad, width):
+    """The counts stay exact (phases in all of a period and in parts of it, some 128 samples a bin and
+    segment), the means are no numbers, and the scores are those of the two-word fold."""
+    import paper_2312_02063_gb300 as g
+    rng = np.random.default_rng(1)
+    n = 65000
+    t = np.arange(n) // 128 + (np.arange(n) % 128) / 128.0 * width + 1e-4
+    f = (1.0 + rng.normal(0.0, 3e-4, n)).astype(np.float32)
+    f[77] = bad
+    p = np.r_[1.0, 0.5, rng.uniform(0.3, 1.0, 300)]
+    args = [_dev(ctx, x) for x in (t, f, p)]
+    try:
+        if nbins in (256, 512):
+            ctx.set_fold_config(**_one_word(g, 3))
+        folded, counts = g.gpfc_fold(ctx, *args, nbins, 0.0)
+        score, _, _ = g.gpfc_search(ctx, *args, nbins, 0.0, g.SCORER_BOX, 1, 20, 0.0)
+        ctx.set_fold_config(warps=1, layout=g.LAYOUT_RED32)
+        folded2, counts2 = g.gpfc_fold(ctx, *args, nbins, 0.0)
+        score2, _, _ = g.gpfc_search(ctx, *args, nbins, 0.0, g.SCORER_BOX, 1, 20, 0.0)
+    finally:
+        ctx.reset_fold_config()
+    ctx.sync()
+    assert torch.equal(counts, counts2)
+    assert torch.equal(torch.isfinite(folded), torch.isfinite(folded2)) and not torch.isfinite(folded).any()
+    assert torch.equal(torch.nan_to_num(score, 7.0), torch.nan_to_num(score2, 7.0))
+    _, cnt_o, _ = oracle.fold(t, np.ones(n, np.float32), p[:6], nbins, 0.0)
+    np.testing.assert_array_equal(counts[:6].cpu().numpy(), cnt_o)
+
+
 # an outlier far above a flux about zero, or above its level: the FP32 sums; none, one within the level or a
 # normal spread about zero: 31 bits of the largest value, which are the more exact there
 @pytest.mark.parametrize("level,outlier,fp32", [(0.0, 1e6, True), (1.0, 1e6, True), (0.0, 1.0, True), (0.0, 0.0, False),
