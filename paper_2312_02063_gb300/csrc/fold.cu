@@ -1525,11 +1525,18 @@ __device__ __forceinline__ void score_row(const BoxCoopParams &p, int64_t r, int
 // the few starts and boxes whose v lies within kNear of the profile's largest. v is off by a few
 // 2^-23, the walk's products by 2^-23: a box further below the largest can neither win the walk
 // nor decide which of the near ones does, so the box, and every output, is the walk's. Profiles
-// with more than kMaxNearStarts near starts (a flat one: every box 0) go through the walk itself.
+// with more than kMaxNearStarts near starts (a flat one: every box 0) go through the walk itself,
+// and so do those of so large or small a scale that the walk's products leave the FP32 range.
 // What bounds it now: instruction issue. 262,144 profiles of 256 bins (before -> now): widths
 // 1..32 2.15 -> 1.05 ms, 1..108 3.96 -> 2.34 ms, 1..160 5.33 -> 3.20 ms.
+//
+// Up to kScanMaxBins bins. On a smooth profile of more, neighbouring starts differ by less than
+// kNear and both passes run, and the bins continued past the end leave fewer warps a block: the
+// walk / the scan on sinusoids, widths up to 0.42 of the bins, 10,000 profiles of 1,024 bins
+// 1.98 / 1.84 ms, 5,000 of 2,048 4.41 / 5.72 ms, 3,000 of 4,096 13.7 / 43.2 ms.
 constexpr float kNear = 1e-5f;
 constexpr int kMaxNearStarts = 8;
+constexpr int kScanMaxBins = 1024;
 
 // (sum, count) pairs of one profile staged by a warp, circularly continued past its end, at
 // index b + b / 8 (so b's that differ by 8 lie in different banks): a walk of w_max bins from
@@ -1803,7 +1810,9 @@ __device__ __forceinline__ BoxWinner scan_row(const BoxCoopParams &p, int64_t r,
     float top = -INFINITY, bv = -INFINITY;
     int bkey = 0x7fffffff;
     int nnear = 0;
-    for (int pass0 = 0; pass0 < nbins; pass0 += 32 * kCoopR) {
+    // (three quarters of the bins empty: still too many starts, at the blocks' ends)
+    const bool sparse = 4 * nnz < nbins;
+    for (int pass0 = 0; pass0 < nbins && !sparse; pass0 += 32 * kCoopR) {
         const int s0 = pass0 + lane * kCoopR;
         float mx[kCoopR];
 #pragma unroll
@@ -1824,9 +1833,14 @@ __device__ __forceinline__ BoxWinner scan_row(const BoxCoopParams &p, int64_t r,
         // correct candidates: the merge keeps the larger)
         top = fmaxf(top, big);
         const float near = fabsf(top) < INFINITY ? top - kNear * fabsf(top) : top;
+        // (a box that starts with an empty bin is the next start's box of one bin less, bit for bit in
+        // the same block of eight, and loses to it: of sparse profiles that leaves the few starts)
         uint32_t mine = 0u;
 #pragma unroll
-        for (int i = 0; i < kCoopR; ++i) mine |= (mx[i] >= near ? 1u : 0u) << i;
+        for (int i = 0; i < kCoopR; ++i)
+            if (mx[i] >= near &&
+                (i == kCoopR - 1 || s0 + i == nbins - 1 || p.w_min > 1 || Bw[s0 + (s0 >> 3) + i].y > 0.f))
+                mine |= 1u << i;
         int n = __popc(mine);
         for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
         nnear += n;
@@ -1844,6 +1858,8 @@ __device__ __forceinline__ BoxWinner scan_row(const BoxCoopParams &p, int64_t r,
         }
     }
     const PairBins B{Bw};
+    // (the walk compares products of up to top^2 Ntot^4 / 16 and of top^2 at least)
+    if (sparse || !(top * Ntot * Ntot < 1e19f && fabsf(top) > 1e-15f)) nnear = nbins;
     if (nnear > kMaxNearStarts) {
         bv = -INFINITY;
         bkey = 0x7fffffff;
@@ -2604,6 +2620,22 @@ cudaError_t launch_fold(const FoldParams &p_in, int mode, int grid, cudaStream_t
     return cudaGetLastError();
 }
 
+// One profile per warp at a time, by the walk: bin counts above kScanMaxBins.
+__global__ void __launch_bounds__(kCoopWarps * 32, 2) box_walk_kernel(const BoxCoopParams p)
+{
+    extern __shared__ __align__(128) uint8_t smem[];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int nw = blockDim.x >> 5;
+    float2 *Bw = reinterpret_cast<float2 *>(smem) + (size_t)warp * coop_pairs(p.nbins);
+    int cur_s = -1;
+    unsigned long long cur_key = 0ull;
+    for (int64_t r = (int64_t)blockIdx.x * nw + warp; r < p.rows; r += (int64_t)gridDim.x * nw) {
+        const int64_t k = p.slot_k ? p.slot_k[r] : p.k_begin + r;
+        if (k >= 0) score_row(p, r, k, Bw, lane, cur_s, cur_key);
+    }
+    if (lane == 0 && p.best_key && cur_key) atomicMax(&p.best_key[cur_s], cur_key);
+}
+
 // One profile per warp at a time. The FP64 tail of the score runs once per 32 profiles, one
 // profile a lane (a division, a square root and a dozen FP64 operations: a tail per profile
 // costs as much as a third of its search).
@@ -2665,7 +2697,7 @@ __global__ void __launch_bounds__(kCoopWarps * 32, kCoopBlocks) box_coop_kernel(
 
 static size_t box_coop_bytes(int nbins, int w_max, int warps)
 {
-    return (size_t)warps * scan_pairs(nbins, w_max) * sizeof(float2);
+    return (size_t)warps * (nbins > kScanMaxBins ? coop_pairs(nbins) : scan_pairs(nbins, w_max)) * sizeof(float2);
 }
 
 // Warps per block of the scorer: kCoopWarps, fewer when their profiles do not fit shared memory.
@@ -2678,7 +2710,11 @@ static int box_coop_warps(int nbins, int w_max)
 
 cudaError_t box_coop_register()
 {
-    return cudaFuncSetAttribute(box_coop_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSmemLimit - 1024));
+    cudaError_t e = cudaSuccess;
+    for (auto kernel : {box_coop_kernel, box_walk_kernel})
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kSmemLimit - 1024));
+    return e;
 }
 
 cudaError_t launch_box_coop(const BoxCoopParams &p, int num_sms, cudaStream_t st)
@@ -2687,12 +2723,13 @@ cudaError_t launch_box_coop(const BoxCoopParams &p, int num_sms, cudaStream_t st
     const int warps = box_coop_warps(p.nbins, p.w_max);
     const size_t smem = box_coop_bytes(p.nbins, p.w_max, warps);
     if (smem > kSmemLimit - 1024) return cudaErrorInvalidValue;
+    const auto kernel = p.nbins > kScanMaxBins ? box_walk_kernel : box_coop_kernel;
     int occ = 0;
-    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, box_coop_kernel, warps * 32, smem);
+    cudaError_t e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, kernel, warps * 32, smem);
     if (e != cudaSuccess) return e;
     const int64_t want = (p.rows + warps - 1) / warps;
     const int grid = (int)std::min<int64_t>(want, (int64_t)num_sms * std::max(1, occ));
-    box_coop_kernel<<<grid, warps * 32, smem, st>>>(p);
+    kernel<<<grid, warps * 32, smem, st>>>(p);
     return cudaGetLastError();
 }
 

@@ -323,6 +323,76 @@ def test_automatic_fold_below_256_bins_is_no_slower_than_fp32(ctx, n, n_periods,
     assert auto <= 1.2 * fp32
 
 
+# ---------------------------------------------------------------- box scorer, decision
+
+def test_box_scorer_of_wide_smooth_profiles(ctx):
+    """A smooth profile of thousands of bins costs what noise does."""
+    import paper_2312_02063_gb300 as g
+    rng = np.random.default_rng(1)
+    x = np.arange(4096) / 4096
+    smooth = 1.0 + 1e-3 * np.sin(2 * np.pi * (x[None] + rng.uniform(0, 1, (600, 1))))
+    noise = 1.0 + rng.normal(0, 1e-4, (600, 4096))
+    counts = _dev(ctx, np.full((600, 4096), 40, np.int32))
+    t = [_ms(ctx, lambda p=_dev(ctx, p.astype(np.float32)): g.gpfc_score_box(ctx, p, counts, 1, 1720, 1e-4))
+         for p in (smooth, noise)]
+    assert t[0] <= 1.25 * t[1]
+
+
+@pytest.mark.parametrize("scale", [1e-25, 1.0, 1e12])
+def test_box_scores_of_any_scale_are_the_same_on_every_path(ctx, scale):
+    """The separate scorer against the one-kernel search, whose comparisons it promises, also where their
+    products leave the FP32 range."""
+    import paper_2312_02063_gb300 as g
+    rng = np.random.default_rng(4)
+    n = 3000
+    f = (scale * (1.0 + rng.normal(0.0, 0.3, n))).astype(np.float32)
+    args = [_dev(ctx, x) for x in (_times("gaps", n, rng), f, rng.uniform(0.2, 1.0, 300))]
+    out = []
+    try:
+        ctx.set_fold_config(warps=2, layout=1)
+        for path in (g.BOX_WARP, g.BOX_FUSED):
+            ctx.set_box_path(path)
+            out.append(g.gpfc_search(ctx, *args, 256, 0.0, g.SCORER_BOX, 1, 60, scale * 0.3)[0])
+    finally:
+        ctx.set_box_path(g.BOX_AUTO)
+        ctx.reset_fold_config()
+    ctx.sync()
+    assert torch.equal(torch.nan_to_num(out[0], 7.0), torch.nan_to_num(out[1], 7.0))
+
+
+# boxes that start with empty bins tie with the next start's, but not across a block of eight starts or the end
+@pytest.mark.parametrize("n,nbins", [(20, 100), (60, 256), (150, 256), (150, 300), (400, 301), (90, 64)])
+def test_box_scores_of_sparse_profiles_are_the_same_on_every_path(ctx, n, nbins):
+    import paper_2312_02063_gb300 as g
+    rng = np.random.default_rng(n)
+    f = (1.0 + rng.normal(0.0, 1e-3, n)).astype(np.float32)
+    args = [_dev(ctx, x) for x in (_times("random", n, rng), f, rng.uniform(0.2, 1.0, 2000))]
+    out = []
+    try:
+        ctx.set_fold_config(warps=2, layout=1)
+        for path in (g.BOX_WARP, g.BOX_EPILOGUE):
+            ctx.set_box_path(path)
+            out.append(g.gpfc_search(ctx, *args, nbins, 0.0, g.SCORER_BOX, 1, nbins // 2, 1e-3)[0])
+    finally:
+        ctx.set_box_path(g.BOX_AUTO)
+        ctx.reset_fold_config()
+    ctx.sync()
+    assert torch.equal(torch.nan_to_num(out[0], 7.0), torch.nan_to_num(out[1], 7.0))
+
+
+def test_box_scorer_of_sparse_profiles(ctx):
+    """A profile with every second bin empty costs no more than a full one."""
+    import paper_2312_02063_gb300 as g
+    rng = np.random.default_rng(2)
+    t = []
+    for density in (0.6, 40.0):
+        c = rng.poisson(density, (1000, 512)).astype(np.int32)
+        p = np.where(c > 0, 1.0 + rng.normal(0, 1e-4, c.shape), np.nan).astype(np.float32)
+        args = [_dev(ctx, p), _dev(ctx, c)]
+        t.append(_ms(ctx, lambda: g.gpfc_score_box(ctx, *args, 1, 128, 1e-4), reps=20))  # noqa: B023
+    assert t[0] <= 1.4 * t[1]
+
+
 def test_decision_of_several_stars_takes_no_longer_than_of_many(ctx):
     """19 stars of 16,384 periods: a block each, not clusters that take turns."""
     import paper_2312_02063_gb300 as g
