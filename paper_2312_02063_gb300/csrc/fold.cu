@@ -1812,7 +1812,7 @@ __device__ __forceinline__ BoxWinner scan_row(const BoxCoopParams &p, int64_t r,
     int nnear = 0;
     // (three quarters of the bins empty: still too many starts, at the blocks' ends)
     const bool sparse = 4 * nnz < nbins;
-    for (int pass0 = 0; pass0 < nbins && !sparse; pass0 += 32 * kCoopR) {
+    for (int pass0 = sparse ? nbins : 0; pass0 < nbins; pass0 += 32 * kCoopR) {
         const int s0 = pass0 + lane * kCoopR;
         float mx[kCoopR];
 #pragma unroll
@@ -1833,14 +1833,16 @@ __device__ __forceinline__ BoxWinner scan_row(const BoxCoopParams &p, int64_t r,
         // correct candidates: the merge keeps the larger)
         top = fmaxf(top, big);
         const float near = fabsf(top) < INFINITY ? top - kNear * fabsf(top) : top;
-        // (a box that starts with an empty bin is the next start's box of one bin less, bit for bit in
-        // the same block of eight, and loses to it: of sparse profiles that leaves the few starts)
         uint32_t mine = 0u;
 #pragma unroll
-        for (int i = 0; i < kCoopR; ++i)
-            if (mx[i] >= near &&
-                (i == kCoopR - 1 || s0 + i == nbins - 1 || p.w_min > 1 || Bw[s0 + (s0 >> 3) + i].y > 0.f))
-                mine |= 1u << i;
+        for (int i = 0; i < kCoopR; ++i) mine |= (mx[i] >= near ? 1u : 0u) << i;
+        // (a box that starts with an empty bin is the next start's box of one bin less, bit for bit in
+        // the same block of eight, and loses to it: of sparse profiles that leaves the few starts)
+        if (mine && p.w_min == 1)
+            for (uint32_t m = mine & ((1u << (kCoopR - 1)) - 1u); m; m &= m - 1) {
+                const int i = __ffs((int)m) - 1;
+                if (s0 + i != nbins - 1 && Bw[s0 + (s0 >> 3) + i].y == 0.f) mine &= ~(1u << i);
+            }
         int n = __popc(mine);
         for (int o = 16; o > 0; o >>= 1) n += __shfl_xor_sync(0xffffffffu, n, o);
         nnear += n;
