@@ -204,15 +204,17 @@ __device__ __forceinline__ float two_sum(float a, float b, float &e)
 }
 
 // Threads per light curve: 256, so that several blocks share an SM and one's set-up overlaps
-// the others' samples; 1,024 where there are too few light curves to fill the SMs that way.
-constexpr int kSynthThreads = 256, kSynthWide = 1024;
+// the others' samples; 1,024 where there are too few light curves to fill the SMs that way. Curves
+// of few samples are set-up above all and take four blocks an SM, with 64 registers a thread: 4,096 of
+// 1,000 samples 168 -> 143 us, of 65,536 1.32 -> 1.44 ms.
+constexpr int kSynthThreads = 256, kSynthWide = 1024, kSynthShort = 4096;
 
 // Samples between emptyings of the 32-bit bin words (|hi| <= 2^14 and lo < 2^15 a sample: sums up to
 // 2^31 and below 2^32) and of a lane's squares (512 of 2^52 at most).
 constexpr int kSynthSpan = 1 << 17;
 
-template <bool POW2, int THREADS>
-__global__ void __launch_bounds__(THREADS) synth_fold_kernel(SynthParams P, int shift)
+template <bool POW2, int THREADS, int BLOCKS>
+__global__ void __launch_bounds__(THREADS, BLOCKS) synth_fold_kernel(SynthParams P, int shift)
 {
     __shared__ uint32_t s_lo[256], s_hi[256], s_cnt[256];  // sum = hi 2^15 + lo, hi signed
     __shared__ LcParams s_lp;
@@ -428,13 +430,15 @@ cudaError_t launch_synth(const SynthParams &p, int num_sms, cudaStream_t st)
     int shift = 32;
     while (shift > 0 && (1 << (32 - shift)) < p.nbins) --shift;
     const bool pow2 = (p.nbins & (p.nbins - 1)) == 0;
-    if (threads == kSynthThreads) {
-        if (pow2) synth_fold_kernel<true, kSynthThreads><<<grid, threads, 0, st>>>(p, shift);
-        else synth_fold_kernel<false, kSynthThreads><<<grid, threads, 0, st>>>(p, 0);
-    } else {
-        if (pow2) synth_fold_kernel<true, kSynthWide><<<grid, threads, 0, st>>>(p, shift);
-        else synth_fold_kernel<false, kSynthWide><<<grid, threads, 0, st>>>(p, 0);
-    }
+    auto launch = [&](auto k_pow2, auto k_any) {
+        if (pow2) k_pow2<<<grid, threads, 0, st>>>(p, shift);
+        else k_any<<<grid, threads, 0, st>>>(p, 0);
+    };
+    if (threads == kSynthWide)
+        launch(synth_fold_kernel<true, kSynthWide, 0>, synth_fold_kernel<false, kSynthWide, 0>);
+    else if (p.sp.n_cadences < kSynthShort)
+        launch(synth_fold_kernel<true, kSynthThreads, 4>, synth_fold_kernel<false, kSynthThreads, 4>);
+    else launch(synth_fold_kernel<true, kSynthThreads, 0>, synth_fold_kernel<false, kSynthThreads, 0>);
     return cudaGetLastError();
 }
 
