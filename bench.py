@@ -39,7 +39,7 @@ SM_FOLD_UPDATES_PER_CLK = 32          # the pipe model: 128 B/clk / one 4-byte r
 # DRAM bytes (read + write) of the fold kernel's launches of one 250,000-period search of
 # the same light curve in steady state (no cache flush, one ncu pass), per period:
 # profiles/dram_traffic_steady_state_kepler62835.md
-SEARCH_DRAM_BYTES_PER_PERIOD = (433.066240e6 + 1206.379008e6) / 250000
+SEARCH_DRAM_BYTES_PER_PERIOD = (441.472768e6 + 1210.173184e6) / 250000
 L2_FLUSH_BYTES = 256 << 20
 
 

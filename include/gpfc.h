@@ -87,11 +87,14 @@ int gpfc_fold_launch_times(gpfc_ctx *ctx, float *total_ms, int32_t *launches);
  * multiples of 2^-e (e per star, the largest with chunk x max|x| 2^e < 2^31) exactly and
  * rounds each bin once to FP32: bit-identical for any warps, streams, tile and
  * blocks_per_sm; chunk sets e.
- * With every field 0 (layout 0 or 3), up to 800 bins or so, the fold keeps sum and count in one
- * shared-memory word: from 256 bins with layout 3's arithmetic and bit-identical outputs, from 32
- * to 255 bins in gpfc_fold only, as said there. gpfc_last_fold_plan then reports layout 3
- * with up to 6 warps (groups of 32 periods), below 256 bins the FP32 layout's plan that the
- * one-word fold stands in for.
+ * With every field 0 (layout 0 or 3) a fold that writes profiles may keep sum and count in one
+ * shared-memory word: at 256 and 512 bins, with layout 3's arithmetic and bit-identical outputs,
+ * where samples and periods are enough for it to pay; from 32 to 255 bins in gpfc_fold only, as
+ * said there. The one-word fold at 256 and 512 bins has a shape of its own: layout 3, tile 2048,
+ * blocks_per_sm 1, streams 1 (its sixteen warps fold all of a block's period groups, up to six of 32
+ * periods: `warps`). gpfc_last_fold_plan reports it, and set by hand (chunk 0 or 65520) it selects
+ * that fold whatever the sizes. Below 256 bins gpfc_last_fold_plan reports the FP32 layout's plan,
+ * which is launched behind the one-word fold.
  *   warps          warps per block, 32 trial periods per warp (1..16, capped by shared memory)
  *   layout         shared-memory bins: 1 = FP32 sum + 16-bit count (6 B per bin),
  *                  2 = FP32 sum + 32-bit count in one 64-bit word (8 B per bin),
@@ -134,14 +137,17 @@ int gpfc_last_fold_plan(const gpfc_ctx *ctx, gpfc_fold_config *out);
  * config gives the same results as the default one; it keeps the fastest in the context under
  * (nbins, scorer, floor(log2 n)). scorer GPFC_SCORER_BOX times the fold with its box-SNR
  * epilogue (scorer_params: gpfc_box_params*), GPFC_SCORER_CNN the fold that writes
- * profiles (scorer_params unused). The chosen config goes to *out (host, may be NULL).
+ * profiles (scorer_params unused), with the one-word fold among the candidates. The chosen config
+ * goes to *out (host, may be NULL); set by hand it selects the same fold.
  * It synchronises the context's stream (GPFC_EINVAL under stream capture) and writes
  * nothing the caller owns.
  * With autotuning enabled (the default), gpfc_fold, gpfc_search and gpfc_search_batched
- * use a tuned config with a matching key, and gpfc_search_batched tunes on its first
- * star when there is none (keyed by the average star length), unless its stream is
- * capturing or the automatic plan is the one-word fold (see gpfc_fold_config).
- * gpfc_set_autotune(ctx, 0) disables both; enable < 0 also forgets the tuned configs. Fields set by gpfc_set_fold_config take precedence. */
+ * use a tuned config with a matching key (the one-word fold only at sizes where it is chosen
+ * untuned; below 256 bins in gpfc_fold a tuned config shapes the FP32 fold alone, since the one-word
+ * fold there sums otherwise), and gpfc_search_batched tunes on its first star when there is none
+ * (keyed by the average star length), unless its stream is capturing or the automatic plan is the
+ * one-word fold (see gpfc_fold_config). gpfc_set_autotune(ctx, 0) disables both; enable < 0 also
+ * forgets the tuned configs. Fields set by gpfc_set_fold_config take precedence. */
 int gpfc_autotune(gpfc_ctx *ctx, const double *times, const float *flux, int64_t n,
                   const double *periods, int64_t n_periods, int32_t nbins, int scorer,
                   const void *scorer_params, gpfc_fold_config *out);
@@ -182,11 +188,14 @@ int gpfc_workspace_size(gpfc_ctx *ctx, int64_t n, int64_t n_periods, int32_t nbi
  * layout 3, the default) x is rounded to a multiple of 2^-e, e per star the largest with
  * max|x| 2^e <= floor((2^31 - 1) / min(chunk, n)), and the multiples are summed exactly
  * (shared-memory integer reductions, int64 across chunks), each bin rounded once to FP32:
- * a bin mean is within 2^-e / 2 of the exact mean of the x. From 32 to
- * 255 bins, with every field of the fold config 0, the same holds of gpfc_fold's profiles with
- * max|x| 2^e <= 2^30 whatever n: 2^-31 max|x|, the FP32 rounding of a value 128 times smaller.
- * Below 32 bins, in the searches, and with any field set, layouts 1 and 2 accumulate x in FP32 with Kahan compensation (chunk partials in shared memory,
- * compensated across chunks). Above 1024 bins (more than a lane's shared-memory share) the
+ * a bin mean is within 2^-e / 2 of the exact mean of the x. An x that is no number or infinite
+ * counts as 0 there (one such flux makes the mean flux, and so every returned mean, no number or
+ * infinite; the counts stay exact). From 32 to 255 bins, with every field of the fold config 0 and
+ * samples enough for the number of periods, the same holds of gpfc_fold's profiles with the largest
+ * e with max|x| 2^e <= 2^30 - 1 whatever n (within 2^-30 max|x|), unless max|x| is above both 4 times
+ * the mean flux and 5.6 times the flux's standard deviation (an outlier). Otherwise, below 32 bins, in
+ * the searches, and with any field set, layouts 1 and 2 accumulate x in FP32 with Kahan compensation
+ * (chunk partials in shared memory, compensated across chunks). Above 1024 bins (more than a lane's shared-memory share) the
  * fold adds each sample with shared-memory atomics per period into count << 40 plus the
  * flux sum in fixed point (quantum 2^-k with n max|x| 2^k < 2^38, or up to 65,536 samples
  * two 32-bit reductions with n max|x| 2^k < 2^31): exact sums, rounded once.
@@ -214,7 +223,8 @@ typedef struct {
  * counts [n_periods][nbins] int32 (required); score [n_periods] float32;
  * best_s / best_w [n_periods] int32, may be NULL. Limits: nbins 2..4096,
  * per-profile sample count N <= 2^24. Each profile is centred on its count-weighted
- * mean (FP64) and scored by one warp (the search kernel of gpfc_set_box_path). */
+ * mean (a double-float sum, FP64 above 1024 bins; rounded to FP32) and scored by one warp (the
+ * search kernel of gpfc_set_box_path). */
 int gpfc_score_box(gpfc_ctx *ctx, const float *folded, const int32_t *counts,
                    int64_t n_periods, int32_t nbins, const gpfc_box_params *params,
                    float *score, int32_t *best_s, int32_t *best_w);
@@ -298,8 +308,8 @@ int gpfc_adam(gpfc_ctx *ctx, float *param, const float *grad, float *m, float *v
  * (Salmon et al. 2011) keyed by `seed`; counter (j, 0, 0, 2^32-1) and (j, 1, 0, 2^32-1)
  * for the parameters, (j, i/4, 1, 0) for the normals of samples 4(i/4)..4(i/4)+3 via
  * Box-Muller on u = (x >> 8) 2^-24. The fold is the 64-bit fixed-point fold of
- * gpfc_fold (t0 = 0), one light curve per block, bins merged within a warp with
- * __match_any_sync; the means are 1 + (sum of (flux - 1)) / count. */
+ * gpfc_fold (t0 = 0), one light curve per block; flux - 1 is summed as multiples of 2^-e, e per light
+ * curve with 2^28 <= 2^e max|flux - 1| < 2^29, exactly; the means are 1 + (sum of (flux - 1)) / count. */
 typedef struct {
     int32_t n_cadences;
     double cadence;
@@ -500,6 +510,8 @@ typedef struct {
  *  - times_out [n] float64, flux_out [n] float32 (flux / fit), segment_out [n] int32 (the
  *    sample's segment index, or NULL): device, caller-owned; the first *n_out entries are
  *    written. n_out [1] int64: device.
+ * Workspace: 122 bytes a sample for each spacing fitted at the same time (as many as 1 GiB holds,
+ * one at least) and 28 (44 if the spacings take several turns) more: 2.8 GB at most.
  * Everything runs in FP64 on the device; reductions run in a fixed order, so the result
  * does not depend on scheduling. Returns GPFC_OK, GPFC_EINVAL, GPFC_ENOMEM or GPFC_ECUDA. */
 int gpfc_detrend(gpfc_ctx *ctx, const double *times, const float *flux, const uint8_t *mask, int64_t n,

@@ -823,8 +823,8 @@ size_t box_warp_bytes(const FoldPlan &pl, int64_t n, int64_t np, int nbins)
 }
 
 // Fold + box-SNR search of one star with the search in its own kernel. Periods go
-// through in chunks of one fold wave; a chunk's centred bin sums and counts stay resident
-// in L2 between the fold and the warp-per-profile scorer.
+// through in chunks of one fold wave; a chunk's centred bin sums and counts go from the fold
+// to the warp-per-profile scorer mostly through the L2.
 int run_search_box_warp(gpfc_ctx *ctx, const double *times, const float *flux, int64_t n, const double *periods,
                         int64_t np, int32_t nbins, double t0, const gpfc_box_params *bp, float *score,
                         int64_t *best_index, float *best_score)
@@ -914,9 +914,9 @@ CnnSrc cnn_src(const gpfc_cnn_weights *wt)
                   wt->conv3_b, wt->fc1_w,   wt->fc1_b,   wt->fc2_w,   wt->fc2_b};
 }
 
-// Fold + CNN search of one star. Periods go through in chunks of one fold wave (one
-// block of 4 x 32 periods per SM); each chunk's means and counts, and the CNN's fc1
-// operand tiles for half a chunk at a time, stay resident in L2 between the kernels.
+// Fold + CNN search of one star. Periods go through in chunks of one fold wave (a lane's
+// period for each lane of the plan's blocks); each chunk's means and counts, and the CNN's fc1
+// operand tiles for half a chunk at a time, go from kernel to kernel mostly through the L2.
 int run_search_cnn(gpfc_ctx *ctx, const double *times, const float *flux, int64_t n, const double *periods,
                    int64_t np, int32_t nbins, double t0, const gpfc_cnn_weights *wt, float *score,
                    int64_t *best_index, float *best_score)

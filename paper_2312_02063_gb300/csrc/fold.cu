@@ -11,7 +11,8 @@
 // are staged into shared memory by the bulk-copy (TMA) engine, double-buffered behind an
 // mbarrier, and every lane reads the same sample (a broadcast). Three bin layouts:
 //
-// * kLayoutRed32 (the default from 256 bins): per bin a row of the 32 lanes' 32-bit
+// * kLayoutRed32 (the default from 256 bins; long folds at 256 and 512 bins take its one-word form,
+//   fold_pack.cu): per bin a row of the 32 lanes' 32-bit
 //   fixed-point sums and a row of their 32-bit counts; an update is two no-return
 //   red.shared.add.u32. The flux is pre-quantised per star (x_q = rint(x 2^e), e from the
 //   largest |x| and the chunk length, so a chunk's bin sum fits in 32 bits), the sums are
